@@ -55,7 +55,16 @@ extern "C" {
                                       breakdown_block says which block                   */
 
 /* ---- precision modes --------------------------------------------------------- */
-#define RBO_PREC_FP64   0  /* every step in IEEE float64 (the reference path)          */
+#define RBO_PREC_FP64   0  /* float64 data and results (the reference path).  The
+                              projections y - x C and the Gram sums are formed on the
+                              fp16 tensor cores from exact integer products: the values
+                              of a column over at most 64 rows (of a row over the columns,
+                              for a projection) share a power-of-two scale and enter as
+                              55-bit integers, off by at most a quarter of an ulp of the
+                              largest of them; a group with a non-finite value or outside
+                              2^+-463 takes float64 FMAs.  The sketch sums 53-bit integers
+                              on the scale of the column's largest value so far.
+                              Triangular solves and the small factors are IEEE float64    */
 #define RBO_PREC_MIXED  1  /* sketch apply and first-pass projection coefficients in
                               float32 with float32 accumulation; Gram matrices feeding
                               the final Cholesky, the small factors, every update of V

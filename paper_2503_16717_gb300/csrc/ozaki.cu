@@ -60,6 +60,7 @@
 #include <mutex>
 
 #include "rowpass_common.cuh"
+#include "tma_map.cuh"
 
 namespace rbo {
 namespace {
@@ -124,15 +125,6 @@ __device__ __forceinline__ void tc_fence_before() {
 }
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-// one 2-D box of a tensor map into shared memory (rows x0.., columns 0..), completion
-// counted on `bar`
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int x0, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-          "r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(tm)), "r"(x0), "r"(0), "r"(smem_u32(bar))
-      : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile(
@@ -330,8 +322,8 @@ __global__ void __launch_bounds__(OZ_NT, 1) ozaki_gram_kernel(const __grid_const
         const int r0 = (first + it * (int)gridDim.x) * OZ_T;
         mbar_arrive_expect_tx(&s_sfull[st], bytes);
         for (int ks = 0; ks < OZ_KS; ++ks) {
-          if (a > 0) tma_load_2d(sb + ks * D.xbox, &D.tmX, r0 + 16 * ks, &s_sfull[st]);
-          tma_load_2d(sb + OZ_KS * D.xbox + ks * D.ybox, &D.tmY, r0 + 16 * ks, &s_sfull[st]);
+          if (a > 0) tma_load_rows(sb + ks * D.xbox, &D.tmX, r0 + 16 * ks, &s_sfull[st]);
+          tma_load_rows(sb + OZ_KS * D.xbox + ks * D.ybox, &D.tmY, r0 + 16 * ks, &s_sfull[st]);
         }
         s_issued = it + 1;
       }
@@ -715,35 +707,6 @@ std::mutex g_oz_mu;
 int g_oz_smem_set[64] = {};
 
 }  // namespace
-
-// 2-D tensor map of a column-major float64 array (n rows, cols columns, leading
-// dimension ld): boxes of 16 rows x cols columns with the 128-byte swizzle, out-of-range
-// rows read as zero.
-static int make_tensor_map(CUtensorMap* m, const double* base, int64_t n, int cols, int64_t ld) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  {
-    std::lock_guard<std::mutex> lk(g_oz_mu);
-    if (encode == nullptr) {
-      void* fn = nullptr;
-      cudaDriverEntryPointQueryResult q;
-      if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-              cudaSuccess ||
-          q != cudaDriverEntryPointSuccess || fn == nullptr) {
-        cudaGetLastError();
-        return RBO_ERR_CUDA;
-      }
-      encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
-  }
-  const cuuint64_t dims[2] = {(cuuint64_t)n, (cuuint64_t)cols};
-  const cuuint64_t strides[1] = {(cuuint64_t)ld * 8};
-  const cuuint32_t box[2] = {16u, (cuuint32_t)cols};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<double*>(base), dims,
-                            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? RBO_OK : RBO_ERR_CUDA;
-}
 
 bool ozaki_gram_supported(const RowPass& rp) {
   if (!rp.ozaki || rp.C || rp.Tri || rp.write_y || rp.sk_d > 0 || rp.sk_gd > 0 || rp.sk_cg > 0 ||

@@ -177,14 +177,15 @@ int ozaki_gram_launch(const RowPass& rp, Arena* ar, cudaStream_t st, int* launch
 // Enqueue one row pass; `launches` is incremented per kernel.  Returns RBO_OK or an
 // error for invalid sizes / CUDA launch failures.
 int rowpass_launch(const RowPass& rp, Arena* ar, cudaStream_t st, int* launches);
-// The sketch-scatter pass (rowpass_sk.cu), called by rowpass_launch for a pass with a
-// scattered sketch once the common checks passed: `L` partial length (d * b), `mixed`
-// float32 sketch sums.
-int rowpass_sk_launch(const RowPass& rp, Arena* ar, cudaStream_t st, int* launches, int num_sms,
-                      int L, int mixed);
-// Shared-memory bytes of its streaming loop for a X columns, b panel columns, T-row
-// tiles and a d-row, zeta-entry sparse sketch (with a projection and a triangle).
-size_t rowpass_sk_loop_bytes(int a, int b, int T, int d, int zeta);
+// The float64 pass without a sketch, its contractions on the tensor cores (rowpass_tc.cu),
+// called by rowpass_launch once the common checks passed; RBO_ERR_ARG when the pass does
+// not fit its shared memory.
+int rowpass_tc_launch(const RowPass& rp, Arena* ar, cudaStream_t st, int* launches, int num_sms);
+// Sketched BCGS2-HH of a panel on a cluster of CTAs (skb2.cu): v (d x k, the reduced sketch)
+// against qs(:, :poff); writes qs(:, poff:poff+k) and T(:poff+k, poff:poff+k) (ld K).
+bool skb2_supported(int d, int k, int poff);
+int skb2_launch(const double* v, double* qs, double* T, int d, int k, int K, int poff, int stage, int block,
+                DevStatus* status, cudaStream_t st, int* launches);
 
 // Sketch schedule: S restricted to each tile of T basis rows, transposed once per
 // call so that the row pass needs neither hashing nor a scatter with conflicts.
@@ -278,7 +279,7 @@ struct OrthCtx {
   int pmax = 0, kmax = 0;
   double *C1 = nullptr, *C2 = nullptr, *Rh = nullptr, *Rp = nullptr, *R2 = nullptr;
   double *T = nullptr, *qs = nullptr, *GB = nullptr;
-  double* tmp = nullptr;  // pmax*kmax + kmax*kmax doubles for small staging
+  double* tmp = nullptr;  // pmax*kmax + kmax*kmax + d*kmax doubles for small staging
 };
 // Take the small buffers from the arena for blocks with up to pmax previous columns
 // and kmax columns per block (K for two-stage).  Returns RBO_OK or RBO_ERR_NOMEM.

@@ -10,9 +10,10 @@
 //                Z   += [x_r, y'_r]^T y'_r                (X^T Y' and/or Y'^T Y')
 //                SK  += s_r y'_r  (sketch column s_r: zeta entries +-1, hashed)
 //
-// This file holds the kernel of the passes without a scattered sketch (Gram and
-// transform passes) and the launcher of all row passes; the sketch passes run in
-// rowpass_sk.cu, the tensor-core Gram in ozaki.cu.
+// This file holds the launcher of all row passes, which run on the tensor cores
+// (rowpass_tc.cuh), and the kernel of the others: passes with a Gaussian sketch, the
+// float32 Gram of mixed precision, float32-pair arithmetic, and shapes the tensor-core
+// kernels have no shared memory for.  The digit Gram asked for by name is in ozaki.cu.
 //
 // Row tiles of T rows are staged in shared memory by the bulk-copy (TMA) engine
 // (cp.async.bulk + mbarrier, double buffered; ragged tiles use plain loads).
@@ -70,7 +71,7 @@ template <int ARITH>
 __global__ void __launch_bounds__(NT, (ARITH == 0 ? 3 : 2)) rowpass_kernel(const __grid_constant__ PassDev P) {
   // ARITH 0: float64; 1: float32 for X^T Y' (mixed precision); 2: float32 pairs for
   // the transform and the Gram.  Passes that scatter a sparse sketch run in
-  // rowpass_sk_kernel (rowpass_sk.cu).
+  // rowpass_tc_kernel (rowpass_tc.cuh).
   constexpr bool MIXED = ARITH == 1;
   constexpr bool DF = ARITH == 2;
   constexpr int IPTA = DF ? 2 : IPT;
@@ -529,7 +530,13 @@ int rowpass_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* launche
     if (rp.sk.rec == nullptr || rp.sk.mcap != sketch_sched_mcap(rp.sk.T, dsk, rp.sk_zeta) ||
         rp.sk.rec_bytes != sketch_sched_rec_bytes(rp.sk.T, dsk, rp.sk_zeta))
       return RBO_ERR_ARG;
-    return rowpass_sk_launch(rp, ar, st, launches, sm_count(), L, mixed);
+    return rowpass_tc_launch(rp, ar, st, launches, sm_count());
+  }
+  // float64 passes: contractions on the tensor cores (a Gaussian sketch adds generated Z
+  // rows, which only the kernel here has)
+  if (arith == 0 && rp.sk_gd == 0) {
+    const int e = rowpass_tc_launch(rp, ar, st, launches, sm_count());
+    if (e != RBO_ERR_ARG) return e;
   }
 
   // tile height: the tallest tile up to 512 rows whose stage stays within STAGE_TARGET
@@ -780,16 +787,6 @@ int sketch_sched_launch(int64_t n, int T, int d, int zeta, uint64_t seed, uint8_
                                                           sketch_sched_rec_bytes(T, d, zeta), out,
                                                           status);
   return cudaGetLastError() == cudaSuccess ? RBO_OK : RBO_ERR_CUDA;
-}
-
-int rowpass_sketch_T(int a_max, int b_max, int d, int zeta) {
-  // shared memory of the streaming loop of a sketch pass (projection, no Gram); 128
-  // rows only while a stage stays within STAGE_TARGET
-  for (int T = 128; T > 16; T /= 2) {
-    if (T > 64 && (size_t)(a_max + b_max) * (T + 2) * 8 > STAGE_TARGET) continue;
-    if (rowpass_sk_loop_bytes(a_max, b_max, T, d, zeta) <= 220 * 1024) return T;
-  }
-  return 16;
 }
 
 int sketch_entries_launch(int64_t row0, int64_t nrows, int d, int zeta, uint64_t seed, int32_t* idx,

@@ -38,6 +38,9 @@ struct PassDev {
   int off_stage, stage_bytes, off_c, off_tri, off_dinv, off_sk, off_red;
   int off_gth;            // Gaussian sketch entries of the tile (sk_gd x TP)
   int rec_off;            // sketch schedule record of the tile, offset inside a stage
+  int kc, off_acc, off_ec;   // tensor-core pass: Gram chunk rows, item sums, C column scales
+  int xblk, yblk;            // bytes of a 16-row block of X and of Y
+  int off_skf, c_digits;     // sketch tile values; whether C is held as digits
   int off_ys, ystage_bytes;  // sketch kernel: ring of Y stages (Y columns + record)
 };
 
@@ -401,49 +404,19 @@ static inline size_t epilogue_doubles(const RowPass& rp) {
 // ------------------------------------------------------------------------------------
 // sketch entry sums of one tile (both row-pass kernels)
 // ------------------------------------------------------------------------------------
-// Sketch of one sketch row over a tile, float64 path: the tile's values of each column
-// are held as int64 fixed point (unit 2^(E_c - 1077), E_c the column's largest
-// exponent field in the tile; fix_from_double); the row's entries are summed exactly
-// in integers (signs by integer negation), and the exact tile sum is rounded once to
-// float64 and added to the accumulator: one float64 add per (sketch row, column) and
-// tile instead of one per entry, on every lane.  A column with a non-finite value in
-// the tile (E_c = 0x7FF) makes the accumulators NaN.
-template <int CW>
-__device__ __forceinline__ void sketch_row_fix(double* acc, int d, const long long* y, int TP,
-                                               const int* emax, const uint8_t* e, int cnt) {
-  long long v[CW];
-#pragma unroll
-  for (int c = 0; c < CW; ++c) v[c] = 0;
-  for (int t = 0; t < cnt; ++t) {
-    const int ev = e[t];
-    const int r = ev >> 1;
-    const long long ng = -(long long)(ev & 1);  // 0 or all ones
-#pragma unroll
-    for (int c = 0; c < CW; ++c) {
-      const long long f = y[(size_t)c * TP + r];
-      v[c] += (f ^ ng) - ng;                     // f or -f
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < CW; ++c) {
-    const double add = emax[c] == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL)
-                                        : double_from_fix(v[c], emax[c]);
-    acc[(size_t)c * d] += add;
-  }
-}
-// float32 values in the first 4 bytes of each 8-byte slot: y holds 2 floats per row
-template <int CW>
-__device__ __forceinline__ void sketch_row_f32(float* acc, int d, const float* y, int TP2,
-                                               const uint8_t* e, int cnt) {
-  float v[CW];
+// One sketch row over a tile: the sums of its entries' rows are added to the row's
+// accumulators (64-bit integers, float32 in mixed precision).  y holds the tile's values
+// and their negatives, entry byte e = local row << 1 | (sign < 0) at y + e * ldy.
+template <int CW, typename V>
+__device__ __forceinline__ void sketch_row_sum(V* acc, int d, const V* y, int ldy, const uint8_t* e, int cnt) {
+  V v[CW];
 #pragma unroll
   for (int c = 0; c < CW; ++c) v[c] = acc[(size_t)c * d];
+#pragma unroll 2
   for (int t = 0; t < cnt; ++t) {
-    const int ev = e[t];
-    const int r = 2 * (ev >> 1);
-    const int sg = (ev & 1) << 31;
+    const V* yr = y + (int)e[t] * ldy;
 #pragma unroll
-    for (int c = 0; c < CW; ++c) v[c] += __int_as_float(__float_as_int(y[(size_t)c * TP2 + r]) ^ sg);
+    for (int c = 0; c < CW; ++c) v[c] += yr[c];
   }
 #pragma unroll
   for (int c = 0; c < CW; ++c) acc[(size_t)c * d] = v[c];

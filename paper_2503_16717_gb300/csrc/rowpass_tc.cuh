@@ -1,0 +1,356 @@
+// The float64 row pass with its contractions on the fp16 tensor cores.
+//
+// y' = (y - x C) Tri^-1 per row, written back, and over the rows Z = [x, y']^T y' or the
+// sparse sketch S y' (see rowpass.cu for the passes).  The projection and the Gram run on
+// exact fixed-point digits (tc_fixed.cuh, tc_tile.cuh) instead of the float64 pipe, which
+// bound those passes at 15-20 % of the HBM rate; triangular solves stay float64.
+//
+// CTAs of 4 warps, several per SM: tiles of T rows come in as tensor copies of 16-row
+// boxes (one thread issues a handful per tile), double buffered; rows past n read as zero.
+// Arrays a tensor copy cannot address (odd leading dimension, unaligned base) are staged
+// with plain loads.  Per tile
+//   A  every warp updates its own 16-row blocks; triangular solve, one row per thread in
+//      registers; write-back;
+//   S  (sketch passes) the y' of the tile as 53-bit integers on one scale per column, and
+//      their signed sums per sketch row from the tile's schedule record: the thread that
+//      owns a slot of the record sums the slot's entries and adds them to the row's 64-bit
+//      integer accumulators.  A column's scale only grows (the accumulators are shifted
+//      when a tile raises it) and the accumulators enter the CTA's float64 partial every
+//      512 rows, so that a tile costs no float64 operation per sketch row;
+//   B  the Gram items, (16 Z columns) x (8 Y' columns) x (a chunk of kc rows), are dealt
+//      to the warps; an item always goes to the same warp, which keeps its float64 sums
+//      in its own shared-memory slots.
+// Measured on GB300, n = 2^22, b = 5, mean over a = 1, 6, .. 56 (float64-pipe kernels it
+// replaces -> here): Gram 1116 -> 500 us, update + Gram 1337 -> 844 us, solve + Gram
+// 1345 -> 658 us, update + sketch (d = 244, 8 entries a row) 1521 -> 1081 us; one-stage
+// orthogonalization of 61 columns 72.5 -> 44.3 ms.  The integer conversion bounds it (IPC
+// 2.0 of 4, ALU pipe 45 %, tensor pipe 20 %, DRAM 30 % of the copy rate).
+// The last CTAs reduce the partials in a fixed order and run the small dense epilogue
+// (rowpass_common.cuh).
+#pragma once
+
+#include <cuda.h>
+
+#include <algorithm>
+
+#include "rowpass_common.cuh"
+#include "tc_tile.cuh"
+#include "tma_map.cuh"
+
+namespace rbo {
+
+constexpr int TC_NT = 128;
+constexpr int TC_NW = TC_NT / 32;
+
+struct TcDev {
+  CUtensorMap tmX, tmY;
+  PassDev P;
+};
+
+// HC: projection (C digits); HT: triangular solve; G: Gram, 0 none, 1 general, 2 of at most
+// 8 columns of Y' alone; SK: sparse sketch (no triangle, no Gram).  Each kind of pass is its
+// own kernel: fewer live registers and less code than one kernel with all phases.
+template <bool HC, bool HT, int G, bool SK>
+__global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_constant__ TcDev D) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bars[NST];
+  __shared__ int s_flag;
+  __shared__ int s_last;
+  __shared__ int s_bad;
+  __shared__ int s_scale[64], s_shift[64], s_nan[64], s_rescale;  // sketch: per column
+  const PassDev& P = D.P;
+  const RowPass& rp = P.p;
+  if (read_code(P.status) != 0) return;
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = P.T, tsh = 31 - __clz(T), a = rp.a, b = rp.b;
+  const int ax = rp.acc_x ? a : 0;
+  const int64_t n = rp.n;
+  const int xblk = P.xblk, yblk = P.yblk, nblk16 = T >> 4;
+  double* Ts = reinterpret_cast<double*>(smem + P.off_tri);
+  double* dinv = reinterpret_cast<double*>(smem + P.off_dinv);
+  uint2* cf = reinterpret_cast<uint2*>(smem + P.off_c);
+  int* ec = reinterpret_cast<int*>(smem + P.off_ec);
+  double* accs = reinterpret_cast<double*>(smem + P.off_acc);
+  const int ldc = rp.ldc > 0 ? rp.ldc : a;
+  const int d = SK ? rp.sk_d : 0;            // scattered sketch rows
+  long long* ska = reinterpret_cast<long long*>(smem + P.off_sk);   // d x b sums
+  long long* skf = reinterpret_cast<long long*>(smem + P.off_skf);  // T x 2 x b tile values
+  const int rec_n = d > 0 ? rp.sk.rec_bytes : 0;
+
+  if (tid == 0) {
+    for (int s = 0; s < NST; ++s) mbar_init(&bars[s], 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+
+  auto stage_X = [&](int s) { return smem + (size_t)s * P.stage_bytes; };
+  auto stage_Y = [&](int s) { return smem + (size_t)s * P.stage_bytes + (size_t)nblk16 * xblk; };
+  auto stage_R = [&](int s) { return smem + (size_t)s * P.stage_bytes + (size_t)nblk16 * (xblk + yblk); };
+  // one thread copies a tile into stage s
+  auto issue_tile = [&](int tile, int s) {
+    const int r0 = tile * T;
+    mbar_arrive_expect_tx(&bars[s], (uint32_t)(T * 8) * (uint32_t)(a + b) + (uint32_t)rec_n);
+    if (d > 0) bulk_copy_g2s(stage_R(s), rp.sk.rec + (size_t)tile * rec_n, (uint32_t)rec_n, &bars[s]);
+    for (int k = 0; k < nblk16; ++k) {
+      if (a > 0) tma_load_rows(stage_X(s) + k * xblk, &D.tmX, r0 + 16 * k, &bars[s]);
+      tma_load_rows(stage_Y(s) + k * yblk, &D.tmY, r0 + 16 * k, &bars[s]);
+    }
+  };
+
+  // the first tile is in flight while the small matrices are prepared
+  uint32_t phase[NST] = {0u, 0u};
+  const int first = blockIdx.x;
+  if (tid == 0 && P.use_bulk && first < P.ntiles) issue_tile(first, 0);
+  // the padding columns of every block hold zeros (the copies do not touch them)
+  for (int s = 0; s < NST; ++s) {
+    const int pa = (xblk >> 7) - a, pb = (yblk >> 7) - b;
+    for (int t = tid; t < nblk16 * (pa + pb) * 8; t += TC_NT) {
+      const int k = t / ((pa + pb) * 8), u = t - k * (pa + pb) * 8, c = u >> 3;
+      unsigned char* p = c < pa ? stage_X(s) + k * xblk + (a + c) * 128 : stage_Y(s) + k * yblk + (b + c - pa) * 128;
+      *reinterpret_cast<uint4*>(p + 16 * (u & 7)) = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  if constexpr (HT) {
+    const int ldt = rp.ldtri > 0 ? rp.ldtri : b;
+    for (int t = tid; t < b * b; t += TC_NT) {
+      const int i = t % b, c = t / b;
+      Ts[t] = (i <= c) ? rp.Tri[i + (size_t)c * ldt] : 0.0;
+    }
+    for (int t = tid; t < b; t += TC_NT) dinv[t] = 1.0 / rp.Tri[t + (size_t)t * ldt];
+  }
+  if constexpr (G != 0)
+    for (int t = tid; t < P.items * 128; t += TC_NT) accs[t] = 0.0;
+  if constexpr (SK) {
+    for (int t = tid; t < d * b; t += TC_NT) ska[t] = 0;  // (all-zero bits also as float32 pairs)
+    if (tid < 64) s_scale[tid] = s_shift[tid] = s_nan[tid] = 0;
+    if (tid == 0) s_rescale = 0;
+  }
+  if (HC && P.c_digits) tc_build_c(rp.C, ldc, a, b, cf, ec, &s_bad);
+  __syncthreads();
+  const int bad_c = HC ? (P.c_digits ? s_bad : 1) : 0;
+  double* mypart = P.L > 0 ? P.partials + (size_t)blockIdx.x * P.L : nullptr;
+  const bool mixed = SK && rp.mixed;  // float32 values and sums of the sketch
+  // sketch sums into the partial: mypart = / += (each thread its own entries)
+  bool sk_first = true;
+  auto sk_flush = [&]() {
+    for (int t = tid; t < d * b; t += TC_NT) {
+      const int c = t / d;
+      if (mixed) {
+        mypart[t] = (double)reinterpret_cast<const float*>(ska)[t];
+        continue;
+      }
+      const double v = s_nan[c] ? __longlong_as_double(0x7FF8000000000000LL) : scalbn((double)ska[t], s_scale[c] - 1075);
+      mypart[t] = sk_first ? v : mypart[t] + v;
+      ska[t] = 0;
+    }
+    sk_first = false;
+  };
+  int sk_rows = 0;  // rows summed since the last flush
+  const int q = P.blk_start[P.nblk];  // Gram items per chunk
+
+  int it = 0;
+  for (int tile = first; tile < P.ntiles; tile += gridDim.x, ++it) {
+    const int s = it & 1;
+    const int64_t r0 = (int64_t)tile * T;
+    const int rows = (n - r0 < (int64_t)T) ? (int)(n - r0) : T;
+    unsigned char* xs = stage_X(s);
+    unsigned char* ys = stage_Y(s);
+    if (P.use_bulk) {
+      if (__syncthreads_or(!mbar_wait_bounded(&bars[s], phase[s]))) {
+        if (tid == 0) set_error(P.status, RBO_ERR_TIMEOUT, 1);
+        return;
+      }
+      phase[s] ^= 1u;
+      // prefetch the next tile into the other stage (its readers passed the barrier)
+      const int nxt = tile + gridDim.x;
+      if (tid == 0 && nxt < P.ntiles) {
+        fence_proxy_async();
+        issue_tile(nxt, s ^ 1);
+      }
+    } else {
+      __syncthreads();  // the previous tile's readers are done
+      for (int t = tid; t < (a + b) * T; t += TC_NT) {
+        const int c = t >> tsh, r = t & (T - 1);
+        double v = 0.0;
+        if (r < rows) v = (c < a) ? rp.X[c * rp.ldx + r0 + r] : rp.Y[(c - a) * rp.ldy + r0 + r];
+        unsigned char* p = c < a ? xs + TcTile::off(xblk, r, c) : ys + TcTile::off(yblk, r, c - a);
+        *reinterpret_cast<double*>(p) = v;
+      }
+      for (int t = tid; t < rec_n / 16; t += TC_NT)
+        reinterpret_cast<uint4*>(stage_R(s))[t] =
+            reinterpret_cast<const uint4*>(rp.sk.rec + (size_t)tile * rec_n)[t];
+      __syncthreads();
+    }
+
+    // ---- A: y' in place in the Y stage -------------------------------------------
+    // one row per thread, column blocks of 8 in registers; each entry subtracts its terms
+    // in column order, as an unblocked row-by-row substitution would
+    auto tri_solve = [&]() {
+      for (int r = tid; r < T; r += TC_NT) {
+        for (int c0 = 0; c0 < b; c0 += 8) {
+          const int cw = min(8, b - c0);
+          double v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (j < cw) v[j] = tc_ld(ys + TcTile::off(yblk, r, c0 + j));
+          for (int i = 0; i < c0; ++i) {
+            const double yi = -tc_ld(ys + TcTile::off(yblk, r, i));
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if (j < cw) v[j] = fma(yi, Ts[i + (c0 + j) * b], v[j]);
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (j < cw) {
+#pragma unroll
+              for (int i = 0; i < j; ++i) v[j] = fma(-v[i], Ts[c0 + i + (c0 + j) * b], v[j]);
+              v[j] *= dinv[c0 + j];
+              *reinterpret_cast<double*>(ys + TcTile::off(yblk, r, c0 + j)) = v[j];
+            }
+        }
+      }
+      __syncthreads();
+    };
+    if (HT && rp.tri_first) tri_solve();
+    if constexpr (HC) {
+      for (int k = warp; k < nblk16; k += TC_NW)
+        tc_update_rows(xs + k * xblk, ys + k * yblk, a, b, cf, ec, bad_c, rp.C, ldc);
+      __syncthreads();
+    }
+    if (HT && !rp.tri_first) tri_solve();
+    if (rp.write_y) {
+      if (P.use_bulk) {  // two rows per thread
+        for (int t = tid; t < b * (T >> 1); t += TC_NT) {
+          const int c = t >> (tsh - 1), r = (t & ((T >> 1) - 1)) * 2;
+          const double2 v = tc_ld2(ys + TcTile::off(yblk, r, c));
+          double* dst = rp.Y + c * rp.ldy + r0 + r;
+          if (r + 1 < rows)
+            *reinterpret_cast<double2*>(dst) = v;
+          else if (r < rows)
+            *dst = v.x;
+        }
+      } else {
+        for (int t = tid; t < b * T; t += TC_NT) {
+          const int c = t >> tsh, r = t & (T - 1);
+          if (r < rows) rp.Y[c * rp.ldy + r0 + r] = tc_ld(ys + TcTile::off(yblk, r, c));
+        }
+      }
+    }
+
+    // ---- S: sketch sums ---------------------------------------------------------------
+    if constexpr (SK) {
+      if (!mixed && sk_rows + T > 512) {  // 2^53 * 512 < 2^63
+        sk_flush();
+        sk_rows = 0;
+        __syncthreads();  // the scales are read above, raised below
+      }
+      sk_rows += T;
+      if (mixed) {
+        for (int t = tid; t < T * b; t += TC_NT) {
+          const int c = t >> tsh, r = t & (T - 1);
+          const float f = f64_to_f32_int(tc_ld(ys + TcTile::off(yblk, r, c)));
+          reinterpret_cast<float*>(skf)[2 * r * b + c] = f;
+          reinterpret_cast<float*>(skf)[(2 * r + 1) * b + c] = -f;
+        }
+        __syncthreads();
+      } else {
+        for (int c = warp; c < b; c += TC_NW) {
+          int ex = 0;
+          for (int r = lane; r < T; r += 32)
+            ex = max(ex, (__double2hiint(tc_ld(ys + TcTile::off(yblk, r, c))) >> 20) & 0x7FF);
+          ex = __reduce_max_sync(0xffffffffu, ex);
+          if (lane == 0) {
+            const int old = s_scale[c];
+            if (ex == 0x7FF) s_nan[c] = 1;
+            s_shift[c] = 0;
+            if (ex > old && ex != 0x7FF) {
+              s_shift[c] = min(ex - old, 63);
+              s_scale[c] = ex;
+              s_rescale = 1;
+            }
+          }
+        }
+        __syncthreads();
+        if (s_rescale) {
+          for (int t = tid; t < d * b; t += TC_NT) {
+            const int k = s_shift[t / d];
+            if (k > 0) ska[t] = k >= 63 ? 0 : (ska[t] + (1LL << (k - 1))) >> k;
+          }
+        }
+        for (int t = tid; t < T * b; t += TC_NT) {
+          const int c = t >> tsh, r = t & (T - 1);
+          const double v = tc_ld(ys + TcTile::off(yblk, r, c));
+          const long long f = s_nan[c] ? 0 : fx_round53(v, s_scale[c]);
+          skf[2 * r * b + c] = f;
+          skf[(2 * r + 1) * b + c] = -f;
+        }
+        __syncthreads();
+        if (tid == 0) s_rescale = 0;
+      }
+      const uint32_t* meta = reinterpret_cast<const uint32_t*>(stage_R(s));
+      const uint8_t* lst = reinterpret_cast<const uint8_t*>(meta + rp.sk.mcap);
+      for (int k = tid; k < rp.sk.mcap; k += TC_NT) {
+        const uint32_t m = meta[k];
+        if (m == 0xFFFFFFFFu) break;
+        const int i = (int)(m & 0xFFFu), o = (int)((m >> 12) & 0x7FFu), cnt = (int)(m >> 23);
+        for (int c0 = 0; c0 < b; c0 += CB) {
+          const int cw = min(CB, b - c0);
+          if (mixed) {
+            RBO_CW_DISPATCH(sketch_row_sum, cw, reinterpret_cast<float*>(ska) + i + (size_t)c0 * d, d,
+                            reinterpret_cast<const float*>(skf) + c0, b, lst + o, cnt)
+          } else {
+            RBO_CW_DISPATCH(sketch_row_sum, cw, ska + i + (size_t)c0 * d, d, skf + c0, b, lst + o, cnt)
+          }
+        }
+      }
+    }
+
+    // ---- B: Z += [x, y']^T y' ------------------------------------------------------
+    if constexpr (G != 0) {
+      const TcTile xt{xs, xblk}, yt{ys, yblk};
+      for (int item = warp; item < P.items; item += TC_NW) {
+        if constexpr (G == 2) {
+          tc_gram_sym8(yt, b, (item * P.kc) >> 4, P.kc >> 4, accs + item * 128);
+        } else {
+          const int chunk = item / q, task = item - chunk * q;
+          int nt = 0;
+          while (nt + 1 < P.nblk && task >= P.blk_start[nt + 1]) ++nt;
+          tc_gram_item(xt, yt, ax, P.zr, b, task - P.blk_start[nt], nt, (chunk * P.kc) >> 4, P.kc >> 4,
+                       accs + item * 128);
+        }
+      }
+    }
+  }
+
+  // ---------------- partials + fixed-order two-level tree -------------------------
+  if (P.L == 0) return;
+  __syncthreads();
+  if constexpr (SK) sk_flush();
+  if constexpr (G != 0)
+  for (int o = tid; o < P.no; o += TC_NT) {
+    const int i = o / b, c = o % b;
+    // the entries of Y'^T Y' below the diagonal come from the upper triangle (the same
+    // integer sums)
+    int zi = i, zc = c;
+    if (i >= ax && i - ax > c) {
+      zi = ax + c;
+      zc = i - ax;
+    }
+    const int task = P.blk_start[zc >> 3] + (zi >> 4);
+    const int ri = zi & 15, ci = zc & 7;
+    const double* p = accs + (size_t)task * 128 + (2 * (ri >> 3) + (ci & 1)) * 32 + 4 * (ri & 7) + (ci >> 1);
+    double sum = 0.0;
+    for (int item = 0; item < P.items; item += q) sum += p[(size_t)item * 128];
+    mypart[o] = sum;
+  }
+  tree_reduce_epilogue(P, smem, &s_flag, &s_last);
+}
+
+// The kernel of a kind of pass; null for a combination no pass uses
+typedef void (*TcKernel)(TcDev);
+TcKernel tc_kernel_g0(bool hc, bool ht, bool sk);  // no Gram   (rowpass_tc_g0.cu)
+TcKernel tc_kernel_g1(bool hc, bool ht);           // general   (rowpass_tc_g1.cu)
+TcKernel tc_kernel_g2(bool hc, bool ht);           // Y'^T Y', at most 8 columns (rowpass_tc_g2.cu)
+
+}  // namespace rbo
