@@ -33,7 +33,7 @@ size_t orth_ctx_bytes(int pmax, int kmax, int d, int64_t n, int zeta, int type, 
   sched_shape(type, d, d_inner, zeta, &ds, &zs);
   const size_t tab =
       (d > 0 && ds > 0) ? sketch_sched_bytes(n, rowpass_sketch_T(pmax, kmax, ds, zs), ds, zs) + 256 : 0;
-  return (2 * pk + 6 * kk + dd + pk + kk) * 8 + 16 * 256 + tab;
+  return (2 * pk + 6 * kk + 2 * dd + pk + kk) * 8 + 16 * 256 + tab;
 }
 
 void set_sketch(RowPass& r, const OrthCtx& c) {
@@ -66,7 +66,7 @@ int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int64_t n) {
   c.T = (double*)c.ar->take(kk * 8);
   c.GB = (double*)c.ar->take(kk * 8);
   c.qs = (double*)c.ar->take(dd * 8);
-  c.tmp = (double*)c.ar->take((pk + kk) * 8);
+  c.tmp = (double*)c.ar->take((pk + kk + dd) * 8);
   if (!c.C1 || !c.C2 || !c.Rh || !c.Rp || !c.R2 || !c.T || !c.GB || !c.qs || !c.tmp)
     return RBO_ERR_NOMEM;
   c.sk = SketchSched();
@@ -259,9 +259,17 @@ int bigpanel_add(OrthCtx& c, BigPanel& bp, int k) {
     if (P > 0) { r.C = c.C1 + (size_t)cols * P; r.ldc = P; r.write_y = 1; }
     set_sketch(r, c);
     r.mixed = c.mixed;
-    r.epi.op = EPI_SKB2; r.epi.qs = c.qs; r.epi.T = c.T; r.epi.K = K; r.epi.poff = cols;
+    const bool cluster = skb2_supported(c.d, k, cols);
+    if (cluster) {
+      r.epi.op = EPI_SKETCH_OUT; r.epi.out_sk = c.tmp;
+    } else {
+      r.epi.op = EPI_SKB2; r.epi.qs = c.qs; r.epi.T = c.T; r.epi.K = K; r.epi.poff = cols;
+    }
     r.epi.stage = RBO_STAGE_BIGPANEL; r.epi.block = bp.blk;
     RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
+    if (cluster)
+      RBO_TRY(skb2_launch(c.tmp, c.qs, c.T, c.d, k, K, cols, RBO_STAGE_BIGPANEL, bp.blk, c.ar->status, c.st,
+                          &c.launches));
   }
   {
     RowPass r;
