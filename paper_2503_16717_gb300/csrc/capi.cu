@@ -258,7 +258,7 @@ int rbo_sketch_apply(rbo_sketch sk, int64_t n, int32_t k, const double* W, int64
   const int dmax = std::max(sk->d, sk->d_inner);
   const int L = orth_max_L(0, k, dmax);
   const size_t bytes = reduction_bytes(L) + (size_t)sk->d * k * 8 +
-                       orth_ctx_bytes(0, k, sk->d, n, sk->zeta, sk->type, sk->d_inner) + 2048;
+                       orth_ctx_bytes(0, k, k, sk->d, n, sk->zeta, sk->type, sk->d_inner) + 2048;
   if ((e = arena_prepare(&ar, bytes))) return e;
   if ((e = arena_reserve_reduction(ar, L, st))) return e;
   double* dout = (double*)ar->take((size_t)sk->d * k * 8);
@@ -267,7 +267,7 @@ int rbo_sketch_apply(rbo_sketch sk, int64_t n, int32_t k, const double* W, int64
   c.ar = ar;
   c.st = st;
   c.d = sk->d; c.zeta = sk->zeta; c.seed = sk->seed; c.sk_type = sk->type; c.d_inner = sk->d_inner;
-  if ((e = orth_ctx_alloc(c, 0, k, n))) return e;
+  if ((e = orth_ctx_alloc(c, 0, k, k, n))) return e;
   RowPass r;
   r.n = n; r.Y = const_cast<double*>(W); r.ldy = ldw; r.b = k;
   set_sketch(r, c);
@@ -365,7 +365,7 @@ static int block_orth_impl(rbo_sketch sk, int64_t n, int32_t ncols, int32_t s, i
   Arena* ar = nullptr;
   const bool mixed = opts && opts->precision == RBO_PREC_MIXED;
   size_t bytes = reduction_bytes(maxL) +
-                 orth_ctx_bytes(pmax, kmax, d, n, rand ? sk->zeta : 0, rand ? sk->type : 0,
+                 orth_ctx_bytes(pmax, kmax, s, d, n, rand ? sk->zeta : 0, rand ? sk->type : 0,
                                 rand ? sk->d_inner : 0) +
                  (size_t)ncols * ncols * 8 + 4096;
   if (mixed) bytes += (size_t)n * kmax * 8 + 256;  // copy of the block in flight
@@ -389,7 +389,7 @@ static int block_orth_impl(rbo_sketch sk, int64_t n, int32_t ncols, int32_t s, i
     c.sk_type = sk->type;
     c.d_inner = sk->d_inner;
   }
-  if ((e = orth_ctx_alloc(c, pmax, kmax, n))) return info_done(info, e, 0, t0);
+  if ((e = orth_ctx_alloc(c, pmax, kmax, s, n))) return info_done(info, e, 0, t0);
   // Mixed precision: a block (two-stage: a big panel) that the float32 steps could not
   // precondition -- its final CholQR lost orthogonality or a Cholesky pivot broke down --
   // is redone in float64 from a copy of its columns taken before it started, and float64

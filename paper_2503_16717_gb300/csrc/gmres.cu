@@ -85,7 +85,7 @@ int sstep_gmres_impl(const rbo_csr* A, const double* Mval, const double* b, doub
 
   const int pmax = m + 1, kmax = K;
   const int maxL = std::max(orth_max_L(pmax, kmax, std::max(d, d_inner)), 1);
-  size_t bytes = reduction_bytes(maxL) + orth_ctx_bytes(pmax, kmax, d, n, zeta, sk_type, d_inner) +
+  size_t bytes = reduction_bytes(maxL) + orth_ctx_bytes(pmax, kmax, s, d, n, zeta, sk_type, d_inner) +
                  (size_t)ldq * (m + 1) * 8 + (size_t)A->nnz * 8 + 2 * (size_t)n * 8 +
                  (size_t)(m + 1) * (m + 1) * 8 + (size_t)(m + 1) * K * 8 + (size_t)m * 8 + 16 * 1024;
   // the MPK operator in SELL-32 form when its rows are short (stencils): room for the
@@ -133,7 +133,7 @@ int sstep_gmres_impl(const rbo_csr* A, const double* Mval, const double* b, doub
   c.seed = seed;
   c.sk_type = sk_type;
   c.d_inner = d_inner;
-  if ((e = orth_ctx_alloc(c, pmax, kmax, n))) return e;
+  if ((e = orth_ctx_alloc(c, pmax, kmax, s, n))) return e;
 
   CsrDev Araw{n, A->nnz, A->rowptr, A->col, A->val};
   CsrDev Ahat = Araw;

@@ -26,14 +26,14 @@ static void sched_shape(int type, int d, int d_inner, int zeta, int* ds, int* zs
   *zs = type == RBO_SKETCH_SPARSE_SIGN ? zeta : 1;
 }
 
-size_t orth_ctx_bytes(int pmax, int kmax, int d, int64_t n, int zeta, int type, int d_inner) {
+size_t orth_ctx_bytes(int pmax, int kmax, int ks, int d, int64_t n, int zeta, int type, int d_inner) {
   size_t pk = (size_t)std::max(pmax, 1) * kmax, kk = (size_t)kmax * kmax;
   size_t dd = (size_t)std::max(d, 1) * kmax;
   int ds = 0, zs = 0;
   sched_shape(type, d, d_inner, zeta, &ds, &zs);
   const size_t tab =
-      (d > 0 && ds > 0) ? sketch_sched_bytes(n, rowpass_sketch_T(pmax, kmax, ds, zs), ds, zs) + 256 : 0;
-  return (2 * pk + 6 * kk + 2 * dd + pk + kk) * 8 + 16 * 256 + tab;
+      (d > 0 && ds > 0) ? sketch_sched_bytes(n, rowpass_sketch_T(pmax, ks, ds, zs), ds, zs) + 256 : 0;
+  return (2 * pk + 8 * kk + 2 * dd + pk + kk) * 8 + 18 * 256 + tab;
 }
 
 void set_sketch(RowPass& r, const OrthCtx& c) {
@@ -53,7 +53,7 @@ int orth_max_L(int pmax, int kmax, int d) {
   return (pmax + kmax) * kmax + std::max(d, 0) * kmax;
 }
 
-int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int64_t n) {
+int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int ks, int64_t n) {
   c.pmax = pmax;
   c.kmax = kmax;
   size_t pk = (size_t)std::max(pmax, 1) * kmax, kk = (size_t)kmax * kmax;
@@ -65,16 +65,18 @@ int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int64_t n) {
   c.R2 = (double*)c.ar->take(kk * 8);
   c.T = (double*)c.ar->take(kk * 8);
   c.GB = (double*)c.ar->take(kk * 8);
+  c.RpInv = (double*)c.ar->take(kk * 8);
+  c.R2Inv = (double*)c.ar->take(kk * 8);
   c.qs = (double*)c.ar->take(dd * 8);
   c.tmp = (double*)c.ar->take((pk + kk + dd) * 8);
-  if (!c.C1 || !c.C2 || !c.Rh || !c.Rp || !c.R2 || !c.T || !c.GB || !c.qs || !c.tmp)
+  if (!c.C1 || !c.C2 || !c.Rh || !c.Rp || !c.R2 || !c.T || !c.GB || !c.RpInv || !c.R2Inv || !c.qs || !c.tmp)
     return RBO_ERR_NOMEM;
   c.sk = SketchSched();
   int ds = 0, zs = 0;
   sched_shape(c.sk_type, c.d, c.d_inner, c.zeta, &ds, &zs);
   if (c.d > 0 && ds > 0) {
     // the sparse sketch is a fixed operator for the call: hashed and transposed once
-    const int T = rowpass_sketch_T(pmax, kmax, ds, zs);
+    const int T = rowpass_sketch_T(pmax, ks, ds, zs);
     uint8_t* rec = (uint8_t*)c.ar->take(sketch_sched_bytes(n, T, ds, zs));
     if (!rec) return RBO_ERR_NOMEM;
     const int e = sketch_sched_launch(n, T, ds, zs, c.seed, rec, c.ar->status, c.st);
@@ -280,7 +282,7 @@ int bigpanel_add(OrthCtx& c, BigPanel& bp, int k) {
     r.write_y = 1; r.acc_y = 1;
     r.epi.op = EPI_GB; r.epi.GB = c.GB; r.epi.K = K; r.epi.poff = cols;
     r.epi.last = (cols + k == K) ? 1 : 0;
-    r.epi.out_rp = c.Rp; r.epi.block = bp.blk;
+    r.epi.out_rp = c.Rp; r.epi.out_inv = c.RpInv; r.epi.block = bp.blk;
     RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
   }
   bp.cols += k;
@@ -293,6 +295,7 @@ int bigpanel_finish(OrthCtx& c, BigPanel& bp, double* Rdev, int ldR, int col0, d
   if (bp.cols != K) return RBO_ERR_ARG;
   Epilogue fin;
   fin.op = EPI_CHOL; fin.out_r = c.R2; fin.stage = RBO_STAGE_FINAL; fin.block = bp.blk;
+  fin.out_inv = c.R2Inv;
   fin.asm_op = ASM_TWO_STAGE;
   fin.C1 = c.C1; fin.ldc1 = std::max(P, 1);
   fin.C2 = c.C2; fin.ldc2 = std::max(P, 1);
@@ -304,7 +307,7 @@ int bigpanel_finish(OrthCtx& c, BigPanel& bp, double* Rdev, int ldR, int col0, d
       RowPass r;
       r.df64 = c.df64; r.ozaki = c.ozaki; r.tag = 10;
       r.n = bp.n; r.X = bp.Q; r.ldx = bp.ldq; r.a = P; r.Y = bp.VB; r.ldy = bp.ldv; r.b = K;
-      r.Tri = c.Rp; r.write_y = 1; r.acc_x = 1;
+      r.Tri = c.Rp; r.Inv = c.RpInv; r.write_y = 1; r.acc_x = 1;
       r.epi.op = EPI_STORE; r.epi.out = c.C2; r.epi.out_ld = P;
       RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
     }
@@ -320,14 +323,14 @@ int bigpanel_finish(OrthCtx& c, BigPanel& bp, double* Rdev, int ldR, int col0, d
     RowPass r;
     r.df64 = c.df64; r.ozaki = c.ozaki; r.tag = 10;
     r.n = bp.n; r.Y = bp.VB; r.ldy = bp.ldv; r.b = K;
-    r.Tri = c.Rp; r.write_y = 1; r.acc_y = 1;
+    r.Tri = c.Rp; r.Inv = c.RpInv; r.write_y = 1; r.acc_y = 1;
     r.epi = fin;
     RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
   }
   RowPass r;
   r.df64 = c.df64; r.ozaki = c.ozaki; r.tag = 12;
   r.n = bp.n; r.Y = bp.VB; r.ldy = bp.ldv; r.b = K;
-  r.Tri = c.R2; r.write_y = 1;
+  r.Tri = c.R2; r.Inv = c.R2Inv; r.write_y = 1;
   return rowpass_launch(r, c.ar, c.st, &c.launches);
 }
 

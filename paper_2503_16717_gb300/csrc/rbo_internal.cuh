@@ -121,6 +121,7 @@ struct Epilogue {
   double* GB = nullptr;
   int last = 0;
   double* out_rp = nullptr;  // R' (K x K, ld K)
+  double* out_inv = nullptr; // EPI_CHOL / EPI_GB: inverse of the factor (same size), or null
   // assembly after a Cholesky (all device, column-major)
   int asm_op = ASM_NONE;
   const double* C1 = nullptr; int ldc1 = 0;   // p x k (or P x K)
@@ -145,6 +146,8 @@ struct RowPass {
   int ldc = 0;                   // 0 means a
   const double* Tri = nullptr;   // b x b (ld ldtri) upper triangular, null = none
   int ldtri = 0;                 // 0 means b
+  const double* Inv = nullptr;   // inverse of Tri (b x b), set where Tri is the factor of a
+                                 // nearly orthonormal Gram: y Tri^-1 may be formed as y Inv
   int tri_first = 0;             // 1: y' = y Tri^-1 - x C;  0: y' = (y - x C) Tri^-1
   int write_y = 0;
   int acc_x = 0;                 // accumulate X^T Y'
@@ -279,15 +282,17 @@ struct OrthCtx {
   int pmax = 0, kmax = 0;
   double *C1 = nullptr, *C2 = nullptr, *Rh = nullptr, *Rp = nullptr, *R2 = nullptr;
   double *T = nullptr, *qs = nullptr, *GB = nullptr;
+  double *RpInv = nullptr, *R2Inv = nullptr;  // inverses of Rp and R2 (two-stage)
   double* tmp = nullptr;  // pmax*kmax + kmax*kmax + d*kmax doubles for small staging
 };
 // Take the small buffers from the arena for blocks with up to pmax previous columns
 // and kmax columns per block (K for two-stage).  Returns RBO_OK or RBO_ERR_NOMEM.
-// With a sketch (c.d > 0) it also builds the sketch entry table of n rows.
-int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int64_t n);
+// With a sketch (c.d > 0) it also builds the sketch entry table of n rows, for sketched
+// panels of at most ks columns.
+int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int ks, int64_t n);
 // Arena bytes orth_ctx_alloc will need.
 // (d: rows of the final sketch; type RBO_SKETCH_*; d_inner: Count-Gauss Count stage)
-size_t orth_ctx_bytes(int pmax, int kmax, int d, int64_t n, int zeta, int type, int d_inner);
+size_t orth_ctx_bytes(int pmax, int kmax, int ks, int d, int64_t n, int zeta, int type, int d_inner);
 // Newton-basis shifts from the k x k upper Hessenberg H (ld ld): alpha, beta (s each).
 int newton_shifts(const double* H, int64_t ld, int k, int s, double* alpha, double* beta);
 int chebyshev_shifts(const double* H, int64_t ld, int k, int s, double* alpha, double* beta);

@@ -40,7 +40,7 @@ struct PassDev {
   int rec_off;            // sketch schedule record of the tile, offset inside a stage
   int kc, off_acc, off_ec;   // tensor-core pass: Gram chunk rows, item sums, C column scales
   int xblk, yblk;            // bytes of a 16-row block of X and of Y
-  int off_skf, c_digits;     // sketch tile values; whether C is held as digits
+  int off_skf, c_digits, inv_digits;  // sketch tile values; whether C / the inverse is held as digits
   int off_ys, ystage_bytes;  // sketch kernel: ring of Y stages (Y columns + record)
 };
 
@@ -195,6 +195,7 @@ static __device__ void run_epilogue(const PassDev& P, const double* red, double*
         for (int t = threadIdx.x; t < b * b; t += blockDim.x) e.out_r[t] = G[t];
       __syncthreads();
       assemble(e, G, b, sm + b * b, P.status);
+      if (e.out_inv != nullptr) cta_tri_inverse(G, b, sm + b * b, e.out_inv);
       break;
     }
     case EPI_PIP: {
@@ -310,6 +311,7 @@ static __device__ void run_epilogue(const PassDev& P, const double* red, double*
           return;
         }
         for (int t = threadIdx.x; t < Kc * Kc; t += blockDim.x) e.out_rp[t] = G[t];
+        if (e.out_inv != nullptr) cta_tri_inverse(G, Kc, sm + Kc * Kc, e.out_inv);
       }
       break;
     }
@@ -393,7 +395,7 @@ static inline size_t epilogue_doubles(const RowPass& rp) {
     case EPI_CHOL: need = (size_t)b * b * 2 + 64; break;
     case EPI_HH: need = (size_t)d * b + (size_t)b * b + 2 * b + 64; break;
     case EPI_SKB2: need = (size_t)3 * d * b + (size_t)2 * e.poff * b + (size_t)b * b + 2 * b + 64; break;
-    case EPI_GB: need = (size_t)(e.poff + b) * (e.poff + b) + 64; break;
+    case EPI_GB: need = (size_t)(e.poff + b) * (e.poff + b) * 2 + 64; break;
     case EPI_PIP: need = (size_t)b * b + 64; break;
     case EPI_SKETCH_OUT: need = (size_t)d * b + 64; break;
     default: break;
@@ -404,22 +406,30 @@ static inline size_t epilogue_doubles(const RowPass& rp) {
 // ------------------------------------------------------------------------------------
 // sketch entry sums of one tile (both row-pass kernels)
 // ------------------------------------------------------------------------------------
-// One sketch row over a tile: the sums of its entries' rows are added to the row's
-// accumulators (64-bit integers, float32 in mixed precision).  y holds the tile's values
-// and their negatives, entry byte e = local row << 1 | (sign < 0) at y + e * ldy.
+// Sketch sums of a tile: meta is its schedule record (mcap slot words, then the entry
+// bytes).  The thread that owns a slot adds the rows of its entries to the sketch row's
+// accumulators (64-bit integers, float32 in mixed precision; column stride d).  y holds the
+// tile's values and their negatives, entry byte e = local row << 1 | (sign < 0) at y + e * ldy.
 template <int CW, typename V>
-__device__ __forceinline__ void sketch_row_sum(V* acc, int d, const V* y, int ldy, const uint8_t* e, int cnt) {
-  V v[CW];
+__device__ __forceinline__ void sketch_tile_sums(const uint32_t* meta, int mcap, V* acc0, int d, const V* y, int ldy) {
+  const uint8_t* lst = reinterpret_cast<const uint8_t*>(meta + mcap);
+  for (int k = threadIdx.x; k < mcap; k += (int)blockDim.x) {
+    const uint32_t m = meta[k];
+    if (m == 0xFFFFFFFFu) break;
+    V* acc = acc0 + (m & 0xFFFu);
+    const uint8_t* e = lst + ((m >> 12) & 0x7FFu);
+    const uint8_t* end = e + (m >> 23);
+    V v[CW];
 #pragma unroll
-  for (int c = 0; c < CW; ++c) v[c] = acc[(size_t)c * d];
-#pragma unroll 2
-  for (int t = 0; t < cnt; ++t) {
-    const V* yr = y + (int)e[t] * ldy;
+    for (int c = 0; c < CW; ++c) v[c] = acc[(size_t)c * d];
+    for (; e < end; ++e) {
+      const V* yr = y + (int)*e * ldy;
 #pragma unroll
-    for (int c = 0; c < CW; ++c) v[c] += yr[c];
+      for (int c = 0; c < CW; ++c) v[c] += yr[c];
+    }
+#pragma unroll
+    for (int c = 0; c < CW; ++c) acc[(size_t)c * d] = v[c];
   }
-#pragma unroll
-  for (int c = 0; c < CW; ++c) acc[(size_t)c * d] = v[c];
 }
 #define RBO_CW_DISPATCH(fn, cw, ...)            \
   switch (cw) {                                 \

@@ -74,13 +74,17 @@ struct TcLayout {
   int xblk, yblk;
   size_t stage_bytes, off_c, off_acc, off_tri, off_dinv, off_ec, off_sk, off_skf, bytes;
 };
-static TcLayout tc_layout(int a, int b, int T, int items, bool has_c, bool digits, bool has_tri, int d, int rec) {
+// digits: B fragments of C (or, inv, of the inverse of Tri) are held in shared memory
+static TcLayout tc_layout(int a, int b, int T, int items, bool has_c, bool digits, bool has_tri, bool inv, int d,
+                          int rec, bool xs) {
   TcLayout l;
   l.xblk = tc_blk_bytes(a, has_c ? 16 : 8);
-  l.yblk = tc_blk_bytes(b, 8);
-  l.stage_bytes = (((size_t)(T / 16) * (l.xblk + l.yblk) + rec) + 1023) & ~size_t(1023);
-  size_t o = NST * l.stage_bytes;
-  const int NB = (b + 7) / 8, KS = (a + 15) / 16;
+  l.yblk = tc_blk_bytes(b, inv ? 16 : 8);
+  // per stage: X, Y, record; with one X stage (xs) X comes first and a stage is Y and record
+  const size_t xb = (size_t)(T / 16) * l.xblk;
+  l.stage_bytes = (((size_t)(T / 16) * l.yblk + (xs ? 0 : xb) + rec) + 1023) & ~size_t(1023);
+  size_t o = NST * l.stage_bytes + (xs ? xb : 0);
+  const int NB = (b + 7) / 8, KS = ((inv ? b : a) + 15) / 16;
   l.off_c = o; o += digits ? (size_t)NB * KS * 7 * 256 : 0;
   l.off_acc = o; o += (size_t)items * 1024;
   l.off_sk = o; o += (size_t)d * b * 8;
@@ -93,12 +97,12 @@ static TcLayout tc_layout(int a, int b, int T, int items, bool has_c, bool digit
 }
 
 // Tile height (64, 32 or 16) of the call's sketch schedule: the tallest for which a pass
-// of a_max X columns and b_max panel columns keeps its digits of C in shared memory (two
-// CTAs per SM for 64 rows), 16 rows otherwise.
+// of a_max X columns and b_max panel columns keeps its digits of C in shared memory, 16 rows
+// otherwise (a tile below 64 rows leaves warps without an update).
 int rowpass_sketch_T(int a_max, int b_max, int d, int zeta) {
   for (int T = 64; T > 16; T /= 2) {
-    const size_t need = tc_layout(a_max, b_max, T, 0, a_max > 0, true, false, d, sketch_sched_rec_bytes(T, d, zeta)).bytes;
-    if (need <= (T == 64 ? 110 : 220) * 1024) return T;
+    const size_t need = tc_layout(a_max, b_max, T, 0, a_max > 0, true, false, false, d, sketch_sched_rec_bytes(T, d, zeta), a_max > 0).bytes;
+    if (need <= 220 * 1024) return T;
   }
   return 16;
 }
@@ -131,8 +135,8 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     const int blk = tc_blk_bytes(a, rp.C ? 16 : 8) + tc_blk_bytes(b, 8);
     while (T < 256 && blk * (2 * T / 16) <= 20 * 1024) T *= 2;
   } else if (q == 1) {
-    const bool narrow = a + b <= 16;
-    T = narrow ? 256 : 128;
+    const bool narrow = a + b <= 16, upd = rp.C && ax == 0;  // (update + sym8: more CTAs)
+    T = upd ? 64 : (narrow ? 256 : 128);
     kc = narrow ? 64 : 32;
   } else if (q <= 3) {
     kc = 32;
@@ -145,10 +149,16 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   const size_t epi_bytes = ((size_t)L + 2) * 8 + epilogue_doubles(rp) * 8;
   TcLayout l;
   size_t smem = 0;
-  bool digits = rp.C != nullptr;
+  // Panels of more than 8 columns multiply by the inverse on the tensor cores where the
+  // caller vouches for the factor (2^22 rows, b = 30: 3717 -> see DESIGN us of substitution on
+  // the float64 pipe); narrow ones substitute
+  const bool xs = rp.C != nullptr && (q == 0 || (ax == 0 && b <= 8));  // as the kernels' XS
+  const bool want_inv = rp.Tri && rp.Inv && !rp.C && b > 8;
+  bool digits = rp.C != nullptr || want_inv;
   for (;;) {
-    kc = std::min(kc, T);
-    l = tc_layout(a, b, T, q * (T / kc), rp.C != nullptr, digits, rp.Tri != nullptr, d, d > 0 ? rp.sk.rec_bytes : 0);
+    kc = (ax == 0 && b <= 8) ? std::max(16, T / 4) : std::min(kc, T);  // sym8: the warps' own rows
+    l = tc_layout(a, b, T, q * (T / kc), rp.C != nullptr, digits, rp.Tri != nullptr, want_inv && digits, d,
+                  d > 0 ? rp.sk.rec_bytes : 0, xs);
     smem = std::max(l.bytes, epi_bytes) + 1024;  // + alignment slack of the base
     if ((long long)smem <= limit) break;
     if (T > 16 && d == 0) T /= 2;
@@ -199,7 +209,8 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   P.off_dinv = (int)l.off_dinv;
   P.off_sk = (int)l.off_sk;
   P.off_skf = (int)l.off_skf;
-  P.c_digits = digits ? 1 : 0;
+  P.c_digits = rp.C && digits ? 1 : 0;
+  P.inv_digits = want_inv && digits ? 1 : 0;
   P.off_red = 0;
   if (L > 0) {
     const size_t need = ((size_t)G * L + (size_t)ngroups * L) * 8;

@@ -11,12 +11,12 @@
 // with plain loads.  Per tile
 //   A  every warp updates its own 16-row blocks; triangular solve, one row per thread in
 //      registers; write-back;
-//   S  (sketch passes) the y' of the tile as 53-bit integers on one scale per column, and
+//   S  (sketch passes) the y' of the tile as 54-bit integers on one scale per column, and
 //      their signed sums per sketch row from the tile's schedule record: the thread that
 //      owns a slot of the record sums the slot's entries and adds them to the row's 64-bit
 //      integer accumulators.  A column's scale only grows (the accumulators are shifted
 //      when a tile raises it) and the accumulators enter the CTA's float64 partial every
-//      512 rows, so that a tile costs no float64 operation per sketch row;
+//      384 rows, so that a tile costs no float64 operation per sketch row;
 //   B  the Gram items, (16 Z columns) x (8 Y' columns) x (a chunk of kc rows), are dealt
 //      to the warps; an item always goes to the same warp, which keeps its float64 sums
 //      in its own shared-memory slots.
@@ -53,7 +53,11 @@ struct TcDev {
 template <bool HC, bool HT, int G, bool SK>
 __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_constant__ TcDev D) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bars[NST];
+  // X is read by the update alone when the pass has no general Gram: one X stage then, its
+  // next tile copied in once every warp has updated its rows (Y keeps two stages), which
+  // leaves room for four CTAs per SM
+  constexpr bool XS = HC && G != 1;
+  __shared__ __align__(8) uint64_t bars[NST], barx;
   __shared__ int s_flag;
   __shared__ int s_last;
   __shared__ int s_bad;
@@ -80,38 +84,48 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
 
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) mbar_init(&bars[s], 1);
+    mbar_init(&barx, 1);
     fence_mbar_init();
   }
   __syncthreads();
 
-  auto stage_X = [&](int s) { return smem + (size_t)s * P.stage_bytes; };
-  auto stage_Y = [&](int s) { return smem + (size_t)s * P.stage_bytes + (size_t)nblk16 * xblk; };
-  auto stage_R = [&](int s) { return smem + (size_t)s * P.stage_bytes + (size_t)nblk16 * (xblk + yblk); };
+  auto stage_X = [&](int s) { return smem + (XS ? 0 : (size_t)s * P.stage_bytes); };
+  auto stage_Y = [&](int s) { return smem + (size_t)nblk16 * xblk + (size_t)s * P.stage_bytes; };
+  auto stage_R = [&](int s) { return stage_Y(s) + (size_t)nblk16 * yblk; };
   // one thread copies a tile into stage s
   auto issue_tile = [&](int tile, int s) {
     const int r0 = tile * T;
-    mbar_arrive_expect_tx(&bars[s], (uint32_t)(T * 8) * (uint32_t)(a + b) + (uint32_t)rec_n);
+    mbar_arrive_expect_tx(&bars[s], (uint32_t)(T * 8) * (uint32_t)((XS ? 0 : a) + b) + (uint32_t)rec_n);
     if (d > 0) bulk_copy_g2s(stage_R(s), rp.sk.rec + (size_t)tile * rec_n, (uint32_t)rec_n, &bars[s]);
     for (int k = 0; k < nblk16; ++k) {
-      if (a > 0) tma_load_rows(stage_X(s) + k * xblk, &D.tmX, r0 + 16 * k, &bars[s]);
+      if (!XS && a > 0) tma_load_rows(stage_X(s) + k * xblk, &D.tmX, r0 + 16 * k, &bars[s]);
       tma_load_rows(stage_Y(s) + k * yblk, &D.tmY, r0 + 16 * k, &bars[s]);
     }
   };
+  auto issue_x = [&](int tile) {  // XS: the tile's X alone
+    mbar_arrive_expect_tx(&barx, (uint32_t)(T * 8) * (uint32_t)a);
+    for (int k = 0; k < nblk16; ++k) tma_load_rows(smem + k * xblk, &D.tmX, tile * T + 16 * k, &barx);
+  };
 
   // the first tile is in flight while the small matrices are prepared
-  uint32_t phase[NST] = {0u, 0u};
+  uint32_t phase[NST] = {0u, 0u}, phx = 0u;
   const int first = blockIdx.x;
-  if (tid == 0 && P.use_bulk && first < P.ntiles) issue_tile(first, 0);
+  if (tid == 0 && P.use_bulk && first < P.ntiles) {
+    issue_tile(first, 0);
+    if (XS) issue_x(first);
+  }
   // the padding columns of every block hold zeros (the copies do not touch them)
   for (int s = 0; s < NST; ++s) {
     const int pa = (xblk >> 7) - a, pb = (yblk >> 7) - b;
     for (int t = tid; t < nblk16 * (pa + pb) * 8; t += TC_NT) {
       const int k = t / ((pa + pb) * 8), u = t - k * (pa + pb) * 8, c = u >> 3;
+      if (XS && s > 0 && c < pa) continue;  // (the first X tile is in flight around its padding)
       unsigned char* p = c < pa ? stage_X(s) + k * xblk + (a + c) * 128 : stage_Y(s) + k * yblk + (b + c - pa) * 128;
       *reinterpret_cast<uint4*>(p + 16 * (u & 7)) = make_uint4(0u, 0u, 0u, 0u);
     }
   }
-  if constexpr (HT) {
+  const bool inv = HT && !HC && P.inv_digits;  // y' = y Inv as digit products (wide panels)
+  if (HT && !inv) {
     const int ldt = rp.ldtri > 0 ? rp.ldtri : b;
     for (int t = tid; t < b * b; t += TC_NT) {
       const int i = t % b, c = t / b;
@@ -127,8 +141,11 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
     if (tid == 0) s_rescale = 0;
   }
   if (HC && P.c_digits) tc_build_c(rp.C, ldc, a, b, cf, ec, &s_bad);
+  if (inv) tc_build_c(rp.Inv, b, b, b, cf, ec, &s_bad);
   __syncthreads();
-  const int bad_c = HC ? (P.c_digits ? s_bad : 1) : 0;
+  const int bad_c = HC ? (P.c_digits ? s_bad : 1) : (inv ? s_bad : 0);
+  // rows of a tile a warp owns from the update to the sums of a chunk: rpw from rw
+  const int rpw = max(16, T >> 2), rw = warp * rpw, re = min(rw + rpw, T);
   double* mypart = P.L > 0 ? P.partials + (size_t)blockIdx.x * P.L : nullptr;
   const bool mixed = SK && rp.mixed;  // float32 values and sums of the sketch
   // sketch sums into the partial: mypart = / += (each thread its own entries)
@@ -140,7 +157,10 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
         mypart[t] = (double)reinterpret_cast<const float*>(ska)[t];
         continue;
       }
-      const double v = s_nan[c] ? __longlong_as_double(0x7FF8000000000000LL) : scalbn((double)ska[t], s_scale[c] - 1075);
+      const int sc = s_scale[c];
+      double v = (double)ska[t];
+      v = sc >= 60 ? v * __hiloint2double((sc - 53) << 20, 0) : scalbn(v, sc - 1076);
+      if (s_nan[c]) v = __longlong_as_double(0x7FF8000000000000LL);
       mypart[t] = sk_first ? v : mypart[t] + v;
       ska[t] = 0;
     }
@@ -157,11 +177,14 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
     unsigned char* xs = stage_X(s);
     unsigned char* ys = stage_Y(s);
     if (P.use_bulk) {
-      if (__syncthreads_or(!mbar_wait_bounded(&bars[s], phase[s]))) {
+      bool ok = mbar_wait_bounded(&bars[s], phase[s]);
+      if (XS) ok = mbar_wait_bounded(&barx, phx) && ok;
+      if (__syncthreads_or(!ok)) {
         if (tid == 0) set_error(P.status, RBO_ERR_TIMEOUT, 1);
         return;
       }
       phase[s] ^= 1u;
+      phx ^= 1u;
       // prefetch the next tile into the other stage (its readers passed the barrier)
       const int nxt = tile + gridDim.x;
       if (tid == 0 && nxt < P.ntiles) {
@@ -184,10 +207,20 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
     }
 
     // ---- A: y' in place in the Y stage -------------------------------------------
-    // one row per thread, column blocks of 8 in registers; each entry subtracts its terms
-    // in column order, as an unblocked row-by-row substitution would
+    // Each warp works on its own rows, without a block barrier.  Triangular solve: one row
+    // per lane, column blocks of 8 in registers; each entry subtracts its terms in column
+    // order, as an unblocked row-by-row substitution would.
+    bool synced = false;  // the last step ended with a block barrier
     auto tri_solve = [&]() {
-      for (int r = tid; r < T; r += TC_NT) {
+      if (inv) {
+        for (int k = rw >> 4; k < re >> 4; ++k) tc_trmul_rows(ys + k * yblk, b, cf, ec, bad_c, rp.Inv);
+        __syncwarp();
+        return;
+      }
+      // (a warp with fewer than 32 rows would leave lanes idle: rows over the block then)
+      const bool own = rpw >= 32;
+      if (!own && HC) __syncthreads();
+      for (int r = own ? rw + lane : tid; r < (own ? re : T); r += own ? 32 : TC_NT) {
         for (int c0 = 0; c0 < b; c0 += 8) {
           const int cw = min(8, b - c0);
           double v[8];
@@ -210,19 +243,31 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
             }
         }
       }
-      __syncthreads();
+      if (own) __syncwarp();
+      else __syncthreads();
+      synced = !own;
     };
     if (HT && rp.tri_first) tri_solve();
     if constexpr (HC) {
-      for (int k = warp; k < nblk16; k += TC_NW)
+      for (int k = rw >> 4; k < re >> 4; ++k)
         tc_update_rows(xs + k * xblk, ys + k * yblk, a, b, cf, ec, bad_c, rp.C, ldc);
-      __syncthreads();
+      synced = false;
+      if (XS && !SK) {
+        __syncthreads();  // every warp is done with X (sketch passes: at their own barrier)
+        if (tid == 0 && P.use_bulk && tile + (int)gridDim.x < P.ntiles) {
+          fence_proxy_async();
+          issue_x(tile + gridDim.x);
+        }
+      } else {
+        __syncwarp();
+      }
     }
     if (HT && !rp.tri_first) tri_solve();
     if (rp.write_y) {
-      if (P.use_bulk) {  // two rows per thread
-        for (int t = tid; t < b * (T >> 1); t += TC_NT) {
-          const int c = t >> (tsh - 1), r = (t & ((T >> 1) - 1)) * 2;
+      if (P.use_bulk) {  // two rows per lane
+        const int h = (re - rw) >> 1, hsh = 31 - __clz(max(h, 1));
+        for (int t = lane; t < b * h; t += 32) {
+          const int c = t >> hsh, r = rw + (t & (h - 1)) * 2;
           const double2 v = tc_ld2(ys + TcTile::off(yblk, r, c));
           double* dst = rp.Y + c * rp.ldy + r0 + r;
           if (r + 1 < rows)
@@ -231,83 +276,91 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
             *dst = v.x;
         }
       } else {
-        for (int t = tid; t < b * T; t += TC_NT) {
-          const int c = t >> tsh, r = t & (T - 1);
-          if (r < rows) rp.Y[c * rp.ldy + r0 + r] = tc_ld(ys + TcTile::off(yblk, r, c));
-        }
+        for (int c = 0; c < b; ++c)
+          for (int r = rw + lane; r < min(re, rows); r += 32)
+            rp.Y[c * rp.ldy + r0 + r] = tc_ld(ys + TcTile::off(yblk, r, c));
       }
     }
 
     // ---- S: sketch sums ---------------------------------------------------------------
     if constexpr (SK) {
-      if (!mixed && sk_rows + T > 512) {  // 2^53 * 512 < 2^63
-        sk_flush();
-        sk_rows = 0;
-        __syncthreads();  // the scales are read above, raised below
-      }
-      sk_rows += T;
-      if (mixed) {
-        for (int t = tid; t < T * b; t += TC_NT) {
-          const int c = t >> tsh, r = t & (T - 1);
-          const float f = f64_to_f32_int(tc_ld(ys + TcTile::off(yblk, r, c)));
+      // every warp converts its rows with the columns' current scales; only a tile with a
+      // value past a scale (or not finite) takes the block-wide path below
+      bool past = false;
+      for (int t = lane; t < (re - rw) * b; t += 32) {
+        const int r = rw + (t & (rpw - 1)), c = t / rpw;
+        const double v = tc_ld(ys + TcTile::off(yblk, r, c));
+        if (mixed) {
+          const float f = f64_to_f32_int(v);
           reinterpret_cast<float*>(skf)[2 * r * b + c] = f;
           reinterpret_cast<float*>(skf)[(2 * r + 1) * b + c] = -f;
+        } else {
+          const int sc = s_scale[c];
+          past = past || ((__double2hiint(v) >> 20) & 0x7FF) > sc;
+          const long long f = fx_round54(v, sc);
+          skf[2 * r * b + c] = f;
+          skf[(2 * r + 1) * b + c] = -f;
         }
-        __syncthreads();
-      } else {
-        for (int c = warp; c < b; c += TC_NW) {
-          int ex = 0;
-          for (int r = lane; r < T; r += 32)
-            ex = max(ex, (__double2hiint(tc_ld(ys + TcTile::off(yblk, r, c))) >> 20) & 0x7FF);
-          ex = __reduce_max_sync(0xffffffffu, ex);
-          if (lane == 0) {
-            const int old = s_scale[c];
-            if (ex == 0x7FF) s_nan[c] = 1;
-            s_shift[c] = 0;
-            if (ex > old && ex != 0x7FF) {
-              s_shift[c] = min(ex - old, 63);
-              s_scale[c] = ex;
-              s_rescale = 1;
+      }
+      if (__any_sync(0xffffffffu, past) && lane == 0) s_rescale = 1;
+      __syncthreads();
+      if (XS && tid == 0 && P.use_bulk && tile + (int)gridDim.x < P.ntiles) {
+        fence_proxy_async();
+        issue_x(tile + gridDim.x);
+      }
+      if (!mixed) {
+        const bool rescale = s_rescale != 0, full = sk_rows + T > 384;  // 2^54 * 384 < 2^63
+        if (full) {
+          sk_flush();
+          sk_rows = 0;
+        }
+        sk_rows += T;
+        if (rescale) {
+          __syncthreads();  // scales read by the flush and the conversion
+          for (int c = warp; c < b; c += TC_NW) {
+            int ex = 0;
+            for (int r = lane; r < T; r += 32)
+              ex = max(ex, (__double2hiint(tc_ld(ys + TcTile::off(yblk, r, c))) >> 20) & 0x7FF);
+            ex = __reduce_max_sync(0xffffffffu, ex);
+            if (lane == 0) {
+              if (ex == 0x7FF) s_nan[c] = 1;
+              const int old = s_scale[c], now = (ex > old && ex != 0x7FF) ? ex + 1 : old;  // room to grow
+              s_shift[c] = min(now - old, 63);
+              s_scale[c] = now;
             }
           }
-        }
-        __syncthreads();
-        if (s_rescale) {
+          __syncthreads();
           for (int t = tid; t < d * b; t += TC_NT) {
             const int k = s_shift[t / d];
             if (k > 0) ska[t] = k >= 63 ? 0 : (ska[t] + (1LL << (k - 1))) >> k;
           }
+          for (int t = tid; t < T * b; t += TC_NT) {
+            const int c = t >> tsh, r = t & (T - 1);
+            const double v = tc_ld(ys + TcTile::off(yblk, r, c));
+            const long long f = s_nan[c] ? 0 : fx_round54(v, s_scale[c]);
+            skf[2 * r * b + c] = f;
+            skf[(2 * r + 1) * b + c] = -f;
+          }
+          if (tid == 0) s_rescale = 0;
         }
-        for (int t = tid; t < T * b; t += TC_NT) {
-          const int c = t >> tsh, r = t & (T - 1);
-          const double v = tc_ld(ys + TcTile::off(yblk, r, c));
-          const long long f = s_nan[c] ? 0 : fx_round53(v, s_scale[c]);
-          skf[2 * r * b + c] = f;
-          skf[(2 * r + 1) * b + c] = -f;
-        }
-        __syncthreads();
-        if (tid == 0) s_rescale = 0;
+        if (rescale || full) __syncthreads();
       }
       const uint32_t* meta = reinterpret_cast<const uint32_t*>(stage_R(s));
-      const uint8_t* lst = reinterpret_cast<const uint8_t*>(meta + rp.sk.mcap);
-      for (int k = tid; k < rp.sk.mcap; k += TC_NT) {
-        const uint32_t m = meta[k];
-        if (m == 0xFFFFFFFFu) break;
-        const int i = (int)(m & 0xFFFu), o = (int)((m >> 12) & 0x7FFu), cnt = (int)(m >> 23);
-        for (int c0 = 0; c0 < b; c0 += CB) {
-          const int cw = min(CB, b - c0);
-          if (mixed) {
-            RBO_CW_DISPATCH(sketch_row_sum, cw, reinterpret_cast<float*>(ska) + i + (size_t)c0 * d, d,
-                            reinterpret_cast<const float*>(skf) + c0, b, lst + o, cnt)
-          } else {
-            RBO_CW_DISPATCH(sketch_row_sum, cw, ska + i + (size_t)c0 * d, d, skf + c0, b, lst + o, cnt)
-          }
+      for (int c0 = 0; c0 < b; c0 += CB) {
+        const int cw = min(CB, b - c0);
+        if (mixed) {
+          RBO_CW_DISPATCH(sketch_tile_sums, cw, meta, rp.sk.mcap, reinterpret_cast<float*>(ska) + (size_t)c0 * d, d,
+                          reinterpret_cast<const float*>(skf) + c0, b)
+        } else {
+          RBO_CW_DISPATCH(sketch_tile_sums, cw, meta, rp.sk.mcap, ska + (size_t)c0 * d, d, skf + c0, b)
         }
       }
     }
 
     // ---- B: Z += [x, y']^T y' ------------------------------------------------------
     if constexpr (G != 0) {
+      // the chunks of sym8 items are the warps' own rows; general items read other warps'
+      if (G == 1 && (HC || HT) && !synced) __syncthreads();
       const TcTile xt{xs, xblk}, yt{ys, yblk};
       for (int item = warp; item < P.items; item += TC_NW) {
         if constexpr (G == 2) {

@@ -45,6 +45,28 @@ static __device__ int cta_cholesky(double* G, int b, int* s_flag) {
   return -1;
 }
 
+// Inverse of the b x b upper triangular R (shared memory, ld b) into out (global, ld b,
+// zero below the diagonal); `w` holds b * b doubles.  One column per thread, by back
+// substitution.
+static __device__ void cta_tri_inverse(const double* R, int b, double* w, double* out) {
+  __syncthreads();
+  for (int c = threadIdx.x; c < b; c += blockDim.x) {
+    w[c + c * b] = 1.0 / R[c + c * b];
+    for (int i = c - 1; i >= 0; --i) {
+      double s0 = 0.0, s1 = 0.0;
+      int l = i + 1;
+      for (; l + 1 <= c; l += 2) {
+        s0 = fma(R[i + l * b], w[l + c * b], s0);
+        s1 = fma(R[i + (l + 1) * b], w[l + 1 + c * b], s1);
+      }
+      if (l <= c) s0 = fma(R[i + l * b], w[l + c * b], s0);
+      w[i + c * b] = -(s0 + s1) / R[i + i * b];
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < b * b; t += blockDim.x) out[t] = (t % b <= t / b) ? w[t] : 0.0;
+}
+
 // First column j whose diagonal entry R_jj of the k x k triangular factor (ld k) is
 // not finite or within k * 2^-53 of the largest |R_ii|: the factored block is rank
 // deficient to working precision.  -1 if none.  Call from one thread.

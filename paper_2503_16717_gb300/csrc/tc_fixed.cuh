@@ -75,16 +75,17 @@ __device__ __forceinline__ FxScale fx_scale(int E) {
   return FxScale{((uint32_t)E << 21) | 0x1FFFFFu, (1u - (uint32_t)E) << 22};
 }
 
-// A value as an integer below 2^53 on the scale of exponent field E (unit 2^(E - 1075)),
-// rounded to nearest, ties away from zero; zero and subnormal values give 0
-__device__ __forceinline__ long long fx_round53(double v, int E) {
+// A value as an integer of at most 2^54 on the scale of exponent field E (unit
+// 2^(E - 1076)), rounded to nearest, ties away from zero; zero and subnormal values give 0
+// (values past the scale give garbage)
+__device__ __forceinline__ long long fx_round54(double v, int E) {
   const uint32_t l = (uint32_t)__double2loint(v), h = (uint32_t)__double2hiint(v);
   const uint32_t e = (h >> 20) & 0x7FFu;
-  const uint32_t m = (__funnelshift_l(l, h, 1) & 0x1FFFFFu) | 0x200000u;  // high word of 2 M
+  const uint32_t m = (__funnelshift_l(l, h, 2) & 0x3FFFFFu) | 0x400000u;  // high word of 4 M
   uint64_t F;
   asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tshr.u64 t, t, %3;\n\tadd.u64 t, t, 1;\n\tshr.u64 %0, t, 1;\n\t}"
       : "=l"(F)
-      : "r"(l << 1), "r"(m), "r"(e == 0u ? 64u : (uint32_t)E - e));
+      : "r"(l << 2), "r"(m), "r"(e == 0u ? 64u : (uint32_t)E - e));
   return (h >> 31) ? -(long long)F : (long long)F;
 }
 

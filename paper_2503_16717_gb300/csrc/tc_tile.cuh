@@ -6,8 +6,8 @@
 // (two rows) permuted by the column: chunk j of column c sits at j ^ (c % 8).  This is
 // what a tensor copy of a (16 rows x columns) box with the 128-byte swizzle writes, and
 // both access patterns below are free of bank conflicts in it.  Columns are padded with
-// zeros to a multiple of 8 (blocks of a multiple of 1024 bytes), those of an update's X to
-// a multiple of 16.
+// zeros to a multiple of 8 (blocks of a multiple of 1024 bytes), the left operand of a
+// product with digits of C to a multiple of 16.
 #pragma once
 
 #include "tc_fixed.cuh"
@@ -282,6 +282,70 @@ static __device__ __forceinline__ void tc_update_rows(const unsigned char* xb, u
         double* yp = reinterpret_cast<double*>(yt + (((o & 1) ? o1 : o0) ^ ((o >> 1) * 64)));
         *yp = fma(-v, fx_weight(o >> 1 ? E1 : E0, ec[c]), *yp);
       }
+    }
+  }
+}
+
+// y = y Inv for the 16 tile rows of one block (yb: b columns padded with zeros to a multiple
+// of 16), Inv upper triangular as B fragments (tc_build_c).  Column tiles are finished from
+// the right: tile nt reads columns up to 8 nt + 7 only.
+static __device__ __forceinline__ void tc_trmul_rows(unsigned char* yb, int b, const uint2* cf, const int* ec, int bad,
+                                                     const double* Inv) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int KS = (b + 15) >> 4, NB = (b + 7) >> 3;
+  const int o0 = 2 * t * 128 + (((g >> 1) ^ (2 * t)) << 4) + ((g & 1) << 3);
+  const int o1 = (2 * t + 1) * 128 + (((g >> 1) ^ (2 * t + 1)) << 4) + ((g & 1) << 3);
+  FxMax m0, m1;
+  for (int k8 = 0; k8 < b; k8 += 8) {
+    const unsigned char* p = yb + k8 * 128;
+    m0.add(tc_ld(p + o0), tc_ld(p + o1));
+    m1.add(tc_ld(p + (o0 ^ 64)), tc_ld(p + (o1 ^ 64)));
+  }
+  m0.reduce4();
+  m1.reduce4();
+  const int E0 = m0.scale(), E1 = m1.scale();
+  if (__any_sync(0xffffffffu, E0 == 0 || E1 == 0) || bad) {
+    if (lane < 16)
+      for (int c = b - 1; c >= 0; --c) {
+        double v = 0.0;
+        for (int i = 0; i <= c; ++i) v = fma(tc_ld(yb + TcTile::off(0, lane, i)), Inv[i + (size_t)c * b], v);
+        *reinterpret_cast<double*>(yb + TcTile::off(0, lane, c)) = v;
+      }
+    return;
+  }
+  const FxScale k0 = fx_scale(E0), k1 = fx_scale(E1);
+  const FxMask km = fx_masks();
+  for (int nt = NB - 1; nt >= 0; --nt) {
+    const int ks_end = min(KS, (nt >> 1) + 1);
+    const bool small = ks_end <= 2;
+    float acc[7][4];
+    fx_clear(acc, small);
+#pragma unroll 1
+    for (int ks = 0; ks < ks_end; ++ks) {
+      const unsigned char* p = yb + ks * 2048;
+      FxPair p00 = fx_pair(tc_ld(p + o0), tc_ld(p + o1), k0, km);
+      FxPair p10 = fx_pair(tc_ld(p + (o0 ^ 64)), tc_ld(p + (o1 ^ 64)), k1, km);
+      FxPair p01 = fx_pair(tc_ld(p + 1024 + o0), tc_ld(p + 1024 + o1), k0, km);
+      FxPair p11 = fx_pair(tc_ld(p + 1024 + (o0 ^ 64)), tc_ld(p + 1024 + (o1 ^ 64)), k1, km);
+      uint32_t bd[7][2];
+#pragma unroll
+      for (int J = 0; J < 7; ++J) {
+        const uint2 u = cf[((size_t)(nt * KS + ks) * 7 + J) * 32 + lane];
+        bd[J][0] = u.x;
+        bd[J][1] = u.y;
+      }
+      fx_step(acc, p00, p10, p01, p11, bd, km);
+    }
+    fx_ints(acc, small);
+    __syncwarp();  // every lane has read this tile's columns
+    unsigned char* yt = yb + nt * 1024;
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      const int c = 8 * nt + 2 * t + (o & 1);
+      const double v = fx_join(acc, o);
+      if (c < b)
+        *reinterpret_cast<double*>(yt + (((o & 1) ? o1 : o0) ^ ((o >> 1) * 64))) =
+            v * fx_weight(o >> 1 ? E1 : E0, ec[c]);
     }
   }
 }
