@@ -33,7 +33,7 @@ size_t orth_ctx_bytes(int pmax, int kmax, int ks, int d, int64_t n, int zeta, in
   sched_shape(type, d, d_inner, zeta, &ds, &zs);
   const size_t tab =
       (d > 0 && ds > 0) ? sketch_sched_bytes(n, rowpass_sketch_T(pmax, ks, ds, zs), ds, zs) + 256 : 0;
-  return (2 * pk + 8 * kk + 2 * dd + pk + kk) * 8 + 18 * 256 + tab;
+  return (2 * pk + 8 * kk + dd + pk + kk) * 8 + 18 * 256 + tab;
 }
 
 void set_sketch(RowPass& r, const OrthCtx& c) {
@@ -68,7 +68,7 @@ int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int ks, int64_t n) {
   c.RpInv = (double*)c.ar->take(kk * 8);
   c.R2Inv = (double*)c.ar->take(kk * 8);
   c.qs = (double*)c.ar->take(dd * 8);
-  c.tmp = (double*)c.ar->take((pk + kk + dd) * 8);
+  c.tmp = (double*)c.ar->take((pk + kk) * 8);
   if (!c.C1 || !c.C2 || !c.Rh || !c.Rp || !c.R2 || !c.T || !c.GB || !c.RpInv || !c.R2Inv || !c.qs || !c.tmp)
     return RBO_ERR_NOMEM;
   c.sk = SketchSched();
@@ -145,6 +145,7 @@ int one_stage_block(OrthCtx& c, int64_t n, const double* Q, int64_t ldq, int p, 
     RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
   }
   // P2: W = W - Q C1, then sketch -> R_hat (or Gram -> chol for CholQR2)
+  bool cluster = false;  // the Householder factor in its own cluster kernel
   {
     RowPass r;
     r.df64 = c.df64; r.ozaki = c.ozaki; r.tag = 2;
@@ -153,13 +154,18 @@ int one_stage_block(OrthCtx& c, int64_t n, const double* Q, int64_t ldq, int p, 
     if (rand) {
       set_sketch(r, c);
       r.mixed = c.mixed;
-      r.epi.op = EPI_HH; r.epi.out_r = c.Rh; r.epi.stage = RBO_STAGE_INTRA; r.epi.block = blk;
+      cluster = c.sk_type == RBO_SKETCH_SPARSE_SIGN && skb2_supported(c.d, k, 0);
+      r.epi.op = cluster ? EPI_GROUPS : EPI_HH;
+      r.epi.out_r = c.Rh; r.epi.stage = RBO_STAGE_INTRA; r.epi.block = blk;
     } else {
       r.acc_y = 1;
       r.epi.op = EPI_CHOL; r.epi.out_r = c.Rh; r.epi.stage = RBO_STAGE_INTRA; r.epi.block = blk;
     }
     RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
   }
+  if (cluster)
+    RBO_TRY(skb2_launch(c.ar->gpart, c.ar->ngroups, (int64_t)c.d * k, nullptr, c.Rh, c.d, k, k, 0, RBO_STAGE_INTRA,
+                        blk, c.ar->status, c.st, &c.launches));
   // P3: W = W R_hat^{-1}; R' = chol(W^T W)
   {
     RowPass r;
@@ -261,17 +267,17 @@ int bigpanel_add(OrthCtx& c, BigPanel& bp, int k) {
     if (P > 0) { r.C = c.C1 + (size_t)cols * P; r.ldc = P; r.write_y = 1; }
     set_sketch(r, c);
     r.mixed = c.mixed;
-    const bool cluster = skb2_supported(c.d, k, cols);
+    const bool cluster = c.sk_type == RBO_SKETCH_SPARSE_SIGN && skb2_supported(c.d, k, cols);
     if (cluster) {
-      r.epi.op = EPI_SKETCH_OUT; r.epi.out_sk = c.tmp;
+      r.epi.op = EPI_GROUPS;
     } else {
       r.epi.op = EPI_SKB2; r.epi.qs = c.qs; r.epi.T = c.T; r.epi.K = K; r.epi.poff = cols;
     }
     r.epi.stage = RBO_STAGE_BIGPANEL; r.epi.block = bp.blk;
     RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
     if (cluster)
-      RBO_TRY(skb2_launch(c.tmp, c.qs, c.T, c.d, k, K, cols, RBO_STAGE_BIGPANEL, bp.blk, c.ar->status, c.st,
-                          &c.launches));
+      RBO_TRY(skb2_launch(c.ar->gpart, c.ar->ngroups, (int64_t)c.d * k, c.qs, c.T, c.d, k, K, cols,
+                          RBO_STAGE_BIGPANEL, bp.blk, c.ar->status, c.st, &c.launches));
   }
   {
     RowPass r;

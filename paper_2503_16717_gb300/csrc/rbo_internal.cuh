@@ -62,6 +62,8 @@ struct Arena {
   int n_tickets = 0;
   double* red = nullptr;         // cross-CTA reduction scratch of the current call
   size_t red_bytes = 0;
+  const double* gpart = nullptr; // EPI_GROUPS: the last pass's group partials, L apart
+  int ngroups = 0;
   void reset() { used = 256; red = nullptr; red_bytes = 0; }
   // bump allocation, 256-byte aligned; returns nullptr when `cap` is too small
   void* take(size_t bytes) {
@@ -94,6 +96,7 @@ enum EpiOp : int {
   EPI_STORE_ALL = 6,  // write all of Z (zr x b, ld zr) to out and the sketch (d x b) to out_sk
   EPI_PIP = 7,        // two-stage BCGS-PIP: Z = [Qbar_{<j} Vh]^T Vh; T_jj = chol(G - P^T P);
                       // T(0:poff, poff:poff+b) = P, T(poff:, poff:) = T_jj
+  EPI_GROUPS = 9,     // leave the group partials in the arena (gpart, ngroups) for a later kernel
   EPI_SKETCH_OUT = 8, // write the sketch S Y' (rows x b, column-major) to out_sk
 };
 
@@ -184,11 +187,12 @@ int rowpass_launch(const RowPass& rp, Arena* ar, cudaStream_t st, int* launches)
 // called by rowpass_launch once the common checks passed; RBO_ERR_ARG when the pass does
 // not fit its shared memory.
 int rowpass_tc_launch(const RowPass& rp, Arena* ar, cudaStream_t st, int* launches, int num_sms);
-// Sketched BCGS2-HH of a panel on a cluster of CTAs (skb2.cu): v (d x k, the reduced sketch)
-// against qs(:, :poff); writes qs(:, poff:poff+k) and T(:poff+k, poff:poff+k) (ld K).
+// Householder R of a panel's sketch (qs null: T is k x k, poff 0), or its sketched BCGS2-HH
+// against qs(:, :poff): writes qs(:, poff:poff+k) and T(:poff+k, poff:poff+k) (ld K); on a
+// cluster of CTAs (skb2.cu).  v: nparts partial sketches (d x k), `stride` doubles apart.
 bool skb2_supported(int d, int k, int poff);
-int skb2_launch(const double* v, double* qs, double* T, int d, int k, int K, int poff, int stage, int block,
-                DevStatus* status, cudaStream_t st, int* launches);
+int skb2_launch(const double* v, int nparts, int64_t stride, double* qs, double* T, int d, int k, int K, int poff,
+                int stage, int block, DevStatus* status, cudaStream_t st, int* launches);
 
 // Sketch schedule: S restricted to each tile of T basis rows, transposed once per
 // call so that the row pass needs neither hashing nor a scatter with conflicts.
@@ -283,7 +287,7 @@ struct OrthCtx {
   double *C1 = nullptr, *C2 = nullptr, *Rh = nullptr, *Rp = nullptr, *R2 = nullptr;
   double *T = nullptr, *qs = nullptr, *GB = nullptr;
   double *RpInv = nullptr, *R2Inv = nullptr;  // inverses of Rp and R2 (two-stage)
-  double* tmp = nullptr;  // pmax*kmax + kmax*kmax + d*kmax doubles for small staging
+  double* tmp = nullptr;  // pmax*kmax + kmax*kmax doubles for small staging
 };
 // Take the small buffers from the arena for blocks with up to pmax previous columns
 // and kmax columns per block (K for two-stage).  Returns RBO_OK or RBO_ERR_NOMEM.

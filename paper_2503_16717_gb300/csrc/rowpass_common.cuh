@@ -342,21 +342,33 @@ __device__ __forceinline__ void tree_reduce_epilogue(const PassDev& P, unsigned 
   __syncthreads();
   if (!s_last) return;
   __threadfence();
+  // two outputs per thread at a time: a reduction step costs an L2 latency, and the wide
+  // results (d b values of a sketch) would otherwise pay it many times in sequence
+  const int nt = (int)blockDim.x;
   {
     const double* base = P.partials + (size_t)g * GROUP * P.L;
     double* gout = P.gpart + (size_t)g * P.L;
-    for (int t = tid; t < P.L; t += (int)blockDim.x) {
-      double s = 0.0;
-      double v[GROUP];
+    for (int t = tid; t < P.L; t += 2 * nt) {
+      const bool two = t + nt < P.L;
+      double v[GROUP], w[GROUP];
 #pragma unroll
-      for (int i = 0; i < GROUP; ++i) v[i] = i < gsize ? __ldcg(base + (size_t)i * P.L + t) : 0.0;
+      for (int i = 0; i < GROUP; ++i) {
+        v[i] = i < gsize ? __ldcg(base + (size_t)i * P.L + t) : 0.0;
+        w[i] = i < gsize && two ? __ldcg(base + (size_t)i * P.L + t + nt) : 0.0;
+      }
+      double s = 0.0, u = 0.0;
 #pragma unroll
       for (int i = 0; i < GROUP; ++i)
-        if (i < gsize) s += v[i];
+        if (i < gsize) {
+          s += v[i];
+          u += w[i];
+        }
       gout[t] = s;
+      if (two) gout[t + nt] = u;
     }
   }
   if (tid == 0) P.tickets[g] = 0u;
+  if (P.p.epi.op == EPI_GROUPS) return;
   __threadfence();
   __syncthreads();
   if (tid == 0) {
@@ -367,18 +379,26 @@ __device__ __forceinline__ void tree_reduce_epilogue(const PassDev& P, unsigned 
   if (!s_last) return;
   __threadfence();
   double* red = reinterpret_cast<double*>(smem + P.off_red);
-  for (int t = tid; t < P.L; t += (int)blockDim.x) {
-    double s = 0.0;
-    for (int i0 = 0; i0 < P.ngroups; i0 += 8) {
-      double v[8];
+  for (int t = tid; t < P.L; t += 2 * nt) {
+    const bool two = t + nt < P.L;
+    double s = 0.0, u = 0.0;
+    for (int i0 = 0; i0 < P.ngroups; i0 += 16) {
+      double v[16], w[16];
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-        v[i] = i0 + i < P.ngroups ? __ldcg(P.gpart + (size_t)(i0 + i) * P.L + t) : 0.0;
+      for (int i = 0; i < 16; ++i) {
+        const bool in = i0 + i < P.ngroups;
+        v[i] = in ? __ldcg(P.gpart + (size_t)(i0 + i) * P.L + t) : 0.0;
+        w[i] = in && two ? __ldcg(P.gpart + (size_t)(i0 + i) * P.L + t + nt) : 0.0;
+      }
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (i0 + i < P.ngroups) s += v[i];
+      for (int i = 0; i < 16; ++i)
+        if (i0 + i < P.ngroups) {
+          s += v[i];
+          u += w[i];
+        }
     }
     red[t] = s;
+    if (two) red[t + nt] = u;
   }
   if (tid == 0) P.tickets[P.ngroups] = 0u;
   __syncthreads();

@@ -219,6 +219,8 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     P.partials = ar->red;
     P.gpart = ar->red + (size_t)G * L;
     P.tickets = ar->tickets;
+    ar->gpart = P.gpart;
+    ar->ngroups = ngroups;
   }
   ProfToken tok = prof_start(st);
   kern<<<G, TC_NT, smem, st>>>(D);

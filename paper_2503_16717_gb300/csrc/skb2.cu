@@ -1,7 +1,8 @@
-// The sketched BCGS2 with Householder intra step of the two-stage preprocessing
-// (Section 7.2) on a cluster of 8 CTAs: v (d x k, the reduced sketch of the panel) against
-// the sketched basis qs (d x poff) of the big panel, giving T(:, panel) and the panel's
-// sketched basis columns.
+// The small dense work on a panel's sketch, on a cluster of 8 CTAs: the Householder factor
+// R of RandHH (one-stage, Section 5.2), or the sketched BCGS2 with Householder intra step of
+// the two-stage preprocessing (Section 7.2): v (d x k) against the sketched basis qs
+// (d x poff) of the big panel, giving T(:, panel) and the panel's sketched basis columns.
+// v is the sum of the sketch pass's group partials (fixed order).
 //
 // The work is small but float64, and one SM does 2 float64 FMAs per cycle: the four
 // products with qs take 4 d poff k of them, 160 us of one SM at d = 404, poff = 40,
@@ -27,8 +28,10 @@ constexpr int SKB2_CTAS = 8;
 constexpr int SKB2_NT = 256;
 
 struct Skb2Dev {
-  const double* v;   // d x k
-  double* qs;        // d x K sketched basis, columns poff.. written
+  const double* v;   // nparts partials of d x k, `stride` apart
+  int nparts;
+  int64_t stride;
+  double* qs;        // d x K sketched basis, columns poff.. written; null: R only
   double* T;         // K x K
   int d, k, K, poff, m;  // m: rows per CTA
   int stage, block;
@@ -56,7 +59,19 @@ __global__ void __cluster_dims__(SKB2_CTAS, 1, 1) __launch_bounds__(SKB2_NT) skb
   double* W = G + k * k;                   // k x k
   double* beta = W + k * k;                // k
 
-  for (int e = tid; e < nr * k; e += SKB2_NT) a[(e % nr) + (e / nr) * m] = P.v[r0 + e % nr + (size_t)(e / nr) * d];
+  for (int e = tid; e < nr * k; e += SKB2_NT) {
+    const double* v = P.v + r0 + e % nr + (size_t)(e / nr) * d;
+    double s = 0.0;
+    for (int g0 = 0; g0 < P.nparts; g0 += 16) {  // 16 loads in flight, summed in order
+      double t[16];
+#pragma unroll
+      for (int g = 0; g < 16; ++g) t[g] = g0 + g < P.nparts ? __ldcg(v + (int64_t)(g0 + g) * P.stride) : 0.0;
+#pragma unroll
+      for (int g = 0; g < 16; ++g)
+        if (g0 + g < P.nparts) s += t[g];
+    }
+    a[(e % nr) + (e / nr) * m] = s;
+  }
   for (int e = tid; e < nr * pp; e += SKB2_NT) q[(e % nr) + (e / nr) * m] = P.qs[r0 + e % nr + (size_t)(e / nr) * d];
   for (int e = tid; e < k * k; e += SKB2_NT) R[e] = 0.0;
   for (int e = tid; e < np; e += SKB2_NT) cs[e] = 0.0;
@@ -145,40 +160,42 @@ __global__ void __cluster_dims__(SKB2_CTAS, 1, 1) __launch_bounds__(SKB2_NT) skb
         a[(j - r0) + c * m] = c == j ? v0 : c1[k + c] - (c1[c] + v0 * c1[k + c]) * bj * v0;
     __syncthreads();
   }
-  // V^T V (strict upper triangle), V(i, j) = 0 above row j
-  for (int t = warp; t < k * k; t += SKB2_NT / 32) {
-    const int i = t % k, c = t / k;
-    double s = 0.0;
-    if (i < c)
-      for (int r = min(max(c - r0, 0), nr) + lane; r < nr; r += 32) s = fma(a[r + i * m], a[r + c * m], s);
-    s = warp_sum(s);
-    if (lane == 0) part[buf * np + t] = s;
-  }
-  exchange(G, k * k);
-  // T of the WY form in place of G: T_jj = beta_j, T(:j, j) = -beta_j T(:j, :j) (V^T v_j)(:j)
-  for (int j = 0; j < k; ++j) {
-    double t = 0.0;
-    if (tid < j)
-      for (int l = tid; l < j; ++l) t = fma(G[tid + l * k], G[l + j * k], t);
+  if (P.qs != nullptr) {
+    // V^T V (strict upper triangle), V(i, j) = 0 above row j
+    for (int t = warp; t < k * k; t += SKB2_NT / 32) {
+      const int i = t % k, c = t / k;
+      double s = 0.0;
+      if (i < c)
+        for (int r = min(max(c - r0, 0), nr) + lane; r < nr; r += 32) s = fma(a[r + i * m], a[r + c * m], s);
+      s = warp_sum(s);
+      if (lane == 0) part[buf * np + t] = s;
+    }
+    exchange(G, k * k);
+    // T of the WY form in place of G: T_jj = beta_j, T(:j, j) = -beta_j T(:j, :j) (V^T v_j)(:j)
+    for (int j = 0; j < k; ++j) {
+      double t = 0.0;
+      if (tid < j)
+        for (int l = tid; l < j; ++l) t = fma(G[tid + l * k], G[l + j * k], t);
+      __syncthreads();
+      if (tid < j) G[tid + j * k] = -beta[j] * t;
+      if (tid == j) G[j + j * k] = beta[j];
+      __syncthreads();
+    }
+    // W = T Vt^T (Vt lower triangular)
+    for (int e = tid; e < k * k; e += SKB2_NT) {
+      const int i = e % k, c = e / k;
+      double s = 0.0;
+      for (int l = i; l <= c; ++l) s = fma(G[i + l * k], Vt[c + l * k], s);
+      W[e] = s;
+    }
     __syncthreads();
-    if (tid < j) G[tid + j * k] = -beta[j] * t;
-    if (tid == j) G[j + j * k] = beta[j];
-    __syncthreads();
-  }
-  // W = T Vt^T (Vt lower triangular)
-  for (int e = tid; e < k * k; e += SKB2_NT) {
-    const int i = e % k, c = e / k;
-    double s = 0.0;
-    for (int l = i; l <= c; ++l) s = fma(G[i + l * k], Vt[c + l * k], s);
-    W[e] = s;
-  }
-  __syncthreads();
-  // Q = I - V W with the signs that make diag(R) >= 0
-  for (int e = tid; e < nr * k; e += SKB2_NT) {
-    const int r = e % nr, c = e / nr, gr = r0 + r;
-    double s = gr == c ? 1.0 : 0.0;
-    for (int l = 0; l < k && l <= gr; ++l) s = fma(-a[r + l * m], W[l + c * k], s);
-    P.qs[gr + (size_t)(pp + c) * d] = R[c + c * k] < 0.0 ? -s : s;
+    // Q = I - V W with the signs that make diag(R) >= 0
+    for (int e = tid; e < nr * k; e += SKB2_NT) {
+      const int r = e % nr, c = e / nr, gr = r0 + r;
+      double s = gr == c ? 1.0 : 0.0;
+      for (int l = 0; l < k && l <= gr; ++l) s = fma(-a[r + l * m], W[l + c * k], s);
+      P.qs[gr + (size_t)(pp + c) * d] = R[c + c * k] < 0.0 ? -s : s;
+    }
   }
   if (rank == 0) {
     for (int e = tid; e < pp * k; e += SKB2_NT) P.T[e % pp + (size_t)(pp + e / pp) * K] = cs[e];
@@ -200,10 +217,10 @@ static int g_skb2_set[64] = {};
 // Whether the cluster kernel serves this shape (otherwise the epilogue of the pass does)
 bool skb2_supported(int d, int k, int poff) { return k <= 16 && d >= k && poff <= 64 && d <= 1024; }
 
-int skb2_launch(const double* v, double* qs, double* T, int d, int k, int K, int poff, int stage, int block,
-                DevStatus* status, cudaStream_t st, int* launches) {
+int skb2_launch(const double* v, int nparts, int64_t stride, double* qs, double* T, int d, int k, int K, int poff,
+                int stage, int block, DevStatus* status, cudaStream_t st, int* launches) {
   if (!skb2_supported(d, k, poff)) return RBO_ERR_ARG;
-  Skb2Dev P{v, qs, T, d, k, K, poff, (d + SKB2_CTAS - 1) / SKB2_CTAS, stage, block, status};
+  Skb2Dev P{v, nparts, stride, qs, T, d, k, K, poff, (d + SKB2_CTAS - 1) / SKB2_CTAS, stage, block, status};
   const int np = std::max(std::max(poff, k), 2) * k;
   const size_t smem = ((size_t)P.m * (k + poff) + 4 * (size_t)np + 4 * (size_t)k * k + k) * 8;
   int dev = 0;
