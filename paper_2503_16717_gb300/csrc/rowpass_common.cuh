@@ -78,18 +78,16 @@ static __device__ void assemble(const Epilogue& e, const double* R2, int k, doub
   // A large deviation means that step failed (the block is numerically rank
   // deficient at the working precision) and the final CholQR cannot repair it;
   // report instead of returning a non-orthogonal Q.
-  if (threadIdx.x == 0) {
-    double dev = 0.0;
-    for (int t = 0; t < k * k; ++t) {
-      const int i = t % k, c = t / k;
-      if (i <= c) dev = fmax(dev, fabs(R2[t] - (i == c ? 1.0 : 0.0)));
-    }
-    if (!(dev <= 0.5)) {
-      if (atomicCAS(&status->code, 0, RBO_ERR_LOST_ORTHOGONALITY) == 0) {
-        status->block = e.block;
-        status->column = -1;
-        status->stage = RBO_STAGE_FINAL;
-      }
+  bool lost = false;
+  for (int t = threadIdx.x; t < k * k; t += blockDim.x) {
+    const int i = t % k, c = t / k;
+    if (i <= c) lost = lost || !(fabs(R2[t] - (i == c ? 1.0 : 0.0)) <= 0.5);
+  }
+  if (__syncthreads_or(lost) && threadIdx.x == 0) {
+    if (atomicCAS(&status->code, 0, RBO_ERR_LOST_ORTHOGONALITY) == 0) {
+      status->block = e.block;
+      status->column = -1;
+      status->stage = RBO_STAGE_FINAL;
     }
   }
   // M = R' * (R_hat or T)
@@ -322,6 +320,55 @@ static __device__ void run_epilogue(const PassDev& P, const double* red, double*
 }
 
 
+// sum of 16 values by pairs (a short chain: float64 additions take long on this GPU)
+__device__ __forceinline__ double pair_sum16(const double (&v)[16]) {
+  double s[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) s[i] = v[i] + v[i + 8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s[i] += s[i + 4];
+  return (s[0] + s[2]) + (s[1] + s[3]);
+}
+
+// out[t] = sum over i < cnt of part[i * L + t], t < L, by the whole block in a fixed order.
+// A step costs an L2 latency: short results take several lanes per output, long ones two
+// outputs per thread, with 16 loads of each in flight.
+__device__ __forceinline__ void sum_partials(const double* part, int cnt, int L, double* out) {
+  const int tid = threadIdx.x, nt = (int)blockDim.x;
+  int S = 8;
+  while (S > 1 && L * S > nt) S >>= 1;
+  if (S > 1) {
+    const int t = tid / S, sub = tid % S;
+    double s = 0.0;
+    for (int i0 = sub; i0 < cnt && t < L; i0 += 16 * S) {
+      double v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = i0 + i * S < cnt ? __ldcg(part + (size_t)(i0 + i * S) * L + t) : 0.0;
+      s += pair_sum16(v);
+    }
+    for (int o = S >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (t < L && sub == 0) out[t] = s;
+    return;
+  }
+  for (int t = tid; t < L; t += 2 * nt) {
+    const bool two = t + nt < L;
+    double s = 0.0, u = 0.0;
+    for (int i0 = 0; i0 < cnt; i0 += 16) {
+      double v[16], w[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const bool in = i0 + i < cnt;
+        v[i] = in ? __ldcg(part + (size_t)(i0 + i) * L + t) : 0.0;
+        w[i] = in && two ? __ldcg(part + (size_t)(i0 + i) * L + t + nt) : 0.0;
+      }
+      s += pair_sum16(v);
+      u += pair_sum16(w);
+    }
+    out[t] = s;
+    if (two) out[t + nt] = u;
+  }
+}
+
 // Fixed-order two-level tree over the per-CTA partials (each CTA has written its L
 // values to P.partials + blockIdx.x * L): groups of GROUP CTAs are summed by the
 // group's last CTA (ticket), then the last group summer sums the group partials into
@@ -342,31 +389,7 @@ __device__ __forceinline__ void tree_reduce_epilogue(const PassDev& P, unsigned 
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  // two outputs per thread at a time: a reduction step costs an L2 latency, and the wide
-  // results (d b values of a sketch) would otherwise pay it many times in sequence
-  const int nt = (int)blockDim.x;
-  {
-    const double* base = P.partials + (size_t)g * GROUP * P.L;
-    double* gout = P.gpart + (size_t)g * P.L;
-    for (int t = tid; t < P.L; t += 2 * nt) {
-      const bool two = t + nt < P.L;
-      double v[GROUP], w[GROUP];
-#pragma unroll
-      for (int i = 0; i < GROUP; ++i) {
-        v[i] = i < gsize ? __ldcg(base + (size_t)i * P.L + t) : 0.0;
-        w[i] = i < gsize && two ? __ldcg(base + (size_t)i * P.L + t + nt) : 0.0;
-      }
-      double s = 0.0, u = 0.0;
-#pragma unroll
-      for (int i = 0; i < GROUP; ++i)
-        if (i < gsize) {
-          s += v[i];
-          u += w[i];
-        }
-      gout[t] = s;
-      if (two) gout[t + nt] = u;
-    }
-  }
+  sum_partials(P.partials + (size_t)g * GROUP * P.L, gsize, P.L, P.gpart + (size_t)g * P.L);
   if (tid == 0) P.tickets[g] = 0u;
   if (P.p.epi.op == EPI_GROUPS) return;
   __threadfence();
@@ -379,27 +402,7 @@ __device__ __forceinline__ void tree_reduce_epilogue(const PassDev& P, unsigned 
   if (!s_last) return;
   __threadfence();
   double* red = reinterpret_cast<double*>(smem + P.off_red);
-  for (int t = tid; t < P.L; t += 2 * nt) {
-    const bool two = t + nt < P.L;
-    double s = 0.0, u = 0.0;
-    for (int i0 = 0; i0 < P.ngroups; i0 += 16) {
-      double v[16], w[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const bool in = i0 + i < P.ngroups;
-        v[i] = in ? __ldcg(P.gpart + (size_t)(i0 + i) * P.L + t) : 0.0;
-        w[i] = in && two ? __ldcg(P.gpart + (size_t)(i0 + i) * P.L + t + nt) : 0.0;
-      }
-#pragma unroll
-      for (int i = 0; i < 16; ++i)
-        if (i0 + i < P.ngroups) {
-          s += v[i];
-          u += w[i];
-        }
-    }
-    red[t] = s;
-    if (two) red[t + nt] = u;
-  }
+  sum_partials(P.gpart, P.ngroups, P.L, red);
   if (tid == 0) P.tickets[P.ngroups] = 0u;
   __syncthreads();
   double* sm = red + ((P.L + 1) & ~1);

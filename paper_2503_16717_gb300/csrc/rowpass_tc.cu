@@ -141,6 +141,11 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   } else if (q <= 3) {
     kc = 32;
   }
+  // few rows: shorter tiles while they leave SMs without one
+  while (d == 0 && T > 64 && (rp.n + T - 1) / T < 2 * (int64_t)num_sms) {
+    T /= 2;
+    kc = std::max(16, kc / 2);
+  }
   const bool hc = rp.C != nullptr, ht = rp.Tri != nullptr;
   const TcKernel kern = q == 0 ? tc_kernel_g0(hc, ht, d > 0)
                                : (ax == 0 && b <= 8 ? tc_kernel_g2(hc, ht) : tc_kernel_g1(hc, ht));

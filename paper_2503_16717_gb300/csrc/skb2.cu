@@ -24,7 +24,7 @@
 namespace rbo {
 namespace cg = cooperative_groups;
 
-constexpr int SKB2_CTAS = 8;
+constexpr int SKB2_CTAS = 8;  // (the exchange sums eight partials)
 constexpr int SKB2_NT = 256;
 
 struct Skb2Dev {
@@ -82,10 +82,10 @@ __global__ void __cluster_dims__(SKB2_CTAS, 1, 1) __launch_bounds__(SKB2_NT) skb
   auto exchange = [&](double* out, int cnt) {
     cl.sync();
     for (int e = tid; e < cnt; e += SKB2_NT) {
-      double s = 0.0;
+      double v[SKB2_CTAS];
 #pragma unroll
-      for (int r = 0; r < SKB2_CTAS; ++r) s += cl.map_shared_rank(part, r)[buf * np + e];
-      out[e] = s;
+      for (int r = 0; r < SKB2_CTAS; ++r) v[r] = cl.map_shared_rank(part, r)[buf * np + e];
+      out[e] = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
     }
     buf ^= 1;
     __syncthreads();
@@ -138,9 +138,21 @@ __global__ void __cluster_dims__(SKB2_CTAS, 1, 1) __launch_bounds__(SKB2_NT) skb
     exchange(c1, 2 * k);
     if (tid == 0) {
       const double rest = c1[j], x0 = c1[k + j];
-      const double alpha = sqrt(rest + x0 * x0), s = x0 >= 0.0 ? 1.0 : -1.0;
-      const double v0 = x0 + s * alpha, vtv = rest + v0 * v0;
-      s_col[0] = beta[j] = alpha == 0.0 ? 0.0 : 2.0 / vtv;
+      const double sq = rest + x0 * x0, s = x0 >= 0.0 ? 1.0 : -1.0;
+      // 2 / v^T v = 1 / (alpha (alpha + |x0|)); the fast forms inside the range where that
+      // product is normal
+      double alpha, v0, b2;
+      if (sq > 1e-280 && sq < 1e280) {
+        double inva;
+        sqrt_and_inverse(sq, alpha, inva);
+        v0 = x0 + s * alpha;
+        b2 = fast_reciprocal(alpha * fabs(v0));
+      } else {
+        alpha = sqrt(sq);
+        v0 = x0 + s * alpha;
+        b2 = alpha == 0.0 ? 0.0 : 1.0 / alpha / fabs(v0);
+      }
+      s_col[0] = beta[j] = b2;
       s_col[1] = v0;
       R[j + j * k] = -s * alpha;
     }

@@ -8,12 +8,95 @@
 
 namespace rbo {
 
+// 2^e for -1022 <= e <= 1023
+static __device__ __forceinline__ double pow2i(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+
+// sqrt(p) and 1 / sqrt(p) of a positive finite normal p: a float32 estimate of 1 / sqrt(m),
+// m = p 4^-q in [1, 4), refined by one step of the cubically convergent iteration
+// y (1 + r / 2 + 3 r^2 / 8), r = 1 - m y^2 (the binomial series of (1 - r)^(-1/2)), and one
+// Newton correction of m y.  The float64 operations of this GPU take long, so that the
+// depth of the chain (7 of them) is what a small factorisation costs.
+static __device__ __forceinline__ void sqrt_and_inverse(double p, double& r, double& inv) {
+  const int hi = __double2hiint(p);
+  const int q = ((hi >> 20) - 1023) >> 1;
+  const double m = __hiloint2double(hi - (q << 21), __double2loint(p));
+  const double y0 = f32_to_f64_int(rsqrtf(f64_to_f32_int(m)));
+  const double e = fma(-m, y0 * y0, 1.0);
+  const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);
+  double s = m * y;
+  s = fma(0.5 * y, fma(-s, s, m), s);
+  r = s * pow2i(q);
+  inv = y * pow2i(-q);
+}
+// 1 / z of a positive finite z with 2^-1000 < z < 2^1000: a float32 estimate y refined by
+// y (1 + e + e^2), e = 1 - z y
+static __device__ __forceinline__ double fast_reciprocal(double z) {
+  const int hi = __double2hiint(z), q = (hi >> 20) - 1023;
+  const double m = __hiloint2double(hi - (q << 20), __double2loint(z));
+  const double y0 = f32_to_f64_int(1.0f / f64_to_f32_int(m));
+  const double e = fma(-m, y0, 1.0);
+  return fma(y0, fma(e, e, e), y0) * pow2i(-q);
+}
+// positive, finite and normal, by its bits
+static __device__ __forceinline__ bool pos_normal(double p) {
+  const unsigned h = (unsigned)__double2hiint(p);
+  return h >= 0x00100000u && h < 0x7FF00000u;
+}
+
+// Cholesky of at most 8 columns by one warp, lane c holding column c in registers: the
+// dependent chain of float64 operations bounds it, so there are no block barriers inside
+// and every update of a column is independent.
+static __device__ int warp_cholesky8(double* G, int b) {
+  const int lane = threadIdx.x & 31;
+  double a[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = (i < b && lane < b && i <= lane) ? G[i + lane * b] : 0.0;
+  int bad = -1;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if (j >= b || bad >= 0) continue;  // (uniform over the warp)
+    const double piv = __shfl_sync(0xffffffffu, a[j], j);
+    double r, inv;
+    if (pos_normal(piv)) {
+      sqrt_and_inverse(piv, r, inv);
+    } else if (!(piv > 0.0) || !isfinite(piv)) {
+      bad = j;
+      continue;
+    } else {  // subnormal
+      r = sqrt(piv);
+      inv = 1.0 / r;
+    }
+    a[j] = lane == j ? r : a[j] * inv;
+#pragma unroll
+    for (int i = j + 1; i < 8; ++i) {
+      const double rji = __shfl_sync(0xffffffffu, a[j], i);  // R(j, i)
+      if (i < b) a[i] = fma(-rji, a[j], a[i]);
+    }
+  }
+  if (bad < 0 && lane < b) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < b) G[i + lane * b] = i <= lane ? a[i] : 0.0;
+  }
+  return bad;
+}
+
 // In-place upper Cholesky of the b x b symmetric matrix G (column-major, ld b, only
 // the upper triangle is read).  On exit the upper triangle holds R (G = R^T R) and
 // the strict lower triangle is zeroed.  Returns -1, or the first column whose pivot
 // is not positive / not finite (Section 5.1: "non-positive pivots").
 static __device__ int cta_cholesky(double* G, int b, int* s_flag) {
   const int tid = threadIdx.x;
+  if (b <= 8) {
+    if (tid < 32) {
+      const int bad = warp_cholesky8(G, b);
+      if (tid == 0) *s_flag = bad;
+    }
+    __syncthreads();
+    const int bad = *s_flag;
+    __syncthreads();
+    return bad;
+  }
   for (int j = 0; j < b; ++j) {
     if (tid == 0) {
       double piv = G[j + j * b];
