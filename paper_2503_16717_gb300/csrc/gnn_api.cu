@@ -22,12 +22,13 @@ __global__ void graph_features_kernel(int64_t, const int32_t*, const int32_t*, c
                                       const int32_t*, const double*, float*, float*);
 __global__ void encode_kernel(int64_t, int, const float*, const __nv_bfloat16*, int, int, float*);
 // tensor-core message and node-update layers (gnn_tc.cu)
-int message_tc_launch(int64_t nnz, int64_t n, const int32_t* col, const float* ein, const float* x,
-                      float* e0out, const float* h, const __nv_bfloat16* w, int l, float* m,
-                      float* eout, float* pe, DevStatus* status, cudaStream_t st);
-int node_update_tc_launch(int64_t n, const int32_t* rowptr, const float* m, const float* hin,
-                          const __nv_bfloat16* w, int l, float* agg, float* rh, float* hout,
-                          float* sdec, float* tdec, DevStatus* status, cudaStream_t st);
+int message_tc_launch(bool train, int64_t nnz, int64_t n, const int32_t* rowptr, const int32_t* erow,
+                      const int32_t* col, const float* ein, const float* x, float* e0out, const float* h,
+                      const float* f, const __nv_bfloat16* w, int l, float* agg, float* m, float* eout, float* pe,
+                      DevStatus* status, cudaStream_t st);
+int node_update_tc_launch(int64_t n, const int32_t* rowptr, float* agg, int keep_agg, const float* hin,
+                          const float* f, const __nv_bfloat16* w, int l, float* rh, float* hout, float* sdec,
+                          float* tdec, DevStatus* status, cudaStream_t st);
 __global__ void decode_terms_kernel(int64_t, const int32_t*, const int32_t*, const float*, const float*,
                                     const float*, const __nv_bfloat16*, const double*, double*);
 __global__ void spmm_kernel(int64_t, int, const int32_t*, const int32_t*, const double*,
@@ -188,7 +189,8 @@ static size_t work_bytes(int64_t n, int64_t nnz, int nr, bool train) {
   b += (size_t)nnz * 8 + (size_t)n * 8 + (size_t)nnz * 12 + (size_t)n * 8;
   const int ne = train ? NL + 1 : 2, nm = train ? NL : 1;
   b += (size_t)ne * nnz * W * 4 + (size_t)ne * n * W * 4;
-  b += (size_t)nm * nnz * W * 4 + (size_t)2 * nm * n * W * 4;
+  b += (size_t)nm * (n + 2 * ((nnz + 31) / 32)) * W * 4;
+  if (train) b += (size_t)nm * nnz * W * 4 + (size_t)nm * n * W * 4;
   b += (size_t)nnz * 8;
   b += (size_t)nnz * 4 + (size_t)2 * n * 4;
   if (train) {
@@ -215,9 +217,11 @@ static int work_take(Arena* ar, Work& w, int64_t n, int64_t nnz, int nr, bool tr
     w.h[l] = (float*)T(n * W * 4);
   }
   for (int l = 0; l < nm; ++l) {
-    w.m[l] = (float*)T(nnz * W * 4);
-    w.agg[l] = (float*)T(n * W * 4);
-    w.rh[l] = (float*)T(n * W * 4);
+    w.agg[l] = (float*)T((n + 2 * ((nnz + 31) / 32)) * W * 4);  // row sums, then pieces of cut rows
+    if (train) {
+      w.m[l] = (float*)T(nnz * W * 4);
+      w.rh[l] = (float*)T(n * W * 4);
+    }
   }
   w.Mval = (double*)T(nnz * 8);
   w.pe = (float*)T(nnz * 4);
@@ -246,7 +250,7 @@ static int work_take(Arena* ar, Work& w, int64_t n, int64_t nnz, int nr, bool tr
   for (int l = 0; l < ne; ++l)
     if (!w.e[l] || !w.h[l]) return RBO_ERR_NOMEM;
   for (int l = 0; l < nm; ++l)
-    if (!w.m[l] || !w.agg[l] || !w.rh[l]) return RBO_ERR_NOMEM;
+    if (!w.agg[l] || (train && (!w.m[l] || !w.rh[l]))) return RBO_ERR_NOMEM;
   return RBO_OK;
 }
 
@@ -265,22 +269,24 @@ static int forward(rbo_gnn_s* g, const rbo_csr* A, Work& w, Arena* ar, cudaStrea
                                                ar->status);
   graph_features_kernel<<<grid1(n), 256, 0, st>>>(n, A->rowptr, A->col, A->val, w.tpos, w.dinv, w.x,
                                                   w.f);
-  encode_kernel<<<grid1(n * W), 256, 0, st>>>(n, 2, w.f, g->wbf, OFF_WN, OFF_BN, w.h[0]);
-  *launches += 3;
+  // (inference computes h_0 from the features inside the first layer)
+  if (train) encode_kernel<<<grid1(n * W), 256, 0, st>>>(n, 2, w.f, g->wbf, OFF_WN, OFF_BN, w.h[0]);
+  *launches += train ? 3 : 2;
   for (int l = 0; l < NL; ++l) {
     const int a = train ? l : (l & 1), b = train ? l + 1 : ((l + 1) & 1);
     const bool last = l == NL - 1;
-    float* mm = train ? w.m[l] : w.m[0];
-    float* ag = train ? w.agg[l] : nullptr;
+    float* mm = train ? w.m[l] : nullptr;
+    float* ag = train ? w.agg[l] : w.agg[0];
     float* rr = train ? w.rh[l] : nullptr;
     float* eo = (train || !last) ? w.e[b] : nullptr;
     float* ho = (train || !last) ? w.h[b] : nullptr;
-    int rc = message_tc_launch(nnz, n, A->col, l == 0 ? nullptr : w.e[a], w.x,
-                               (l == 0 && train) ? w.e[0] : nullptr, w.h[a], g->wbf, l, mm, eo,
+    int rc = message_tc_launch(train, nnz, n, A->rowptr, w.erow, A->col, l == 0 ? nullptr : w.e[a], w.x,
+                               (l == 0 && train) ? w.e[0] : nullptr, w.h[a], w.f, g->wbf, l, ag, mm, eo,
                                last ? w.pe : nullptr, ar->status, st);
     if (rc == RBO_OK)
-      rc = node_update_tc_launch(n, A->rowptr, mm, w.h[a], g->wbf, l, ag, rr, ho,
-                                 last ? w.sdec : nullptr, last ? w.tdec : nullptr, ar->status, st);
+      rc = node_update_tc_launch(n, A->rowptr, ag, train ? 1 : 0, (l == 0 && !train) ? nullptr : w.h[a], w.f,
+                                 g->wbf, l, rr, ho, last ? w.sdec : nullptr, last ? w.tdec : nullptr, ar->status,
+                                 st);
     if (rc != RBO_OK) return rc;
     *launches += 2;
   }

@@ -242,18 +242,30 @@ struct MsgArgs {
   const float* ein;          // e_l per edge; null: e_0 from x
   const float* x;            // edge features, 3 per edge (used when ein is null)
   float* e0out;              // e_0 written here when computed and non-null
-  const float* h;            // h_l per node (gathered by column)
+  const float* h;            // h_l per node (gathered by column; not used where h_0 comes from f)
+  const float* f;            // node features, 2 per node (first layer of inference)
   const __nv_bfloat16* w;    // bfloat16 parameters
   int l;                     // layer
-  float* m;                  // m_l per edge
+  const int32_t* rowptr;     // row starts
+  const int32_t* erow;       // row i of edge q
+  float* agg;                // row sums of m (n rows of 32), then 2 rows of pieces per 32 edges
+  float* m;                  // m_l per edge, or null
   float* eout;               // e_{l+1} = e_l + m_l per edge, or null
   float* pe;                 // decoder edge term wo[0:32] . e_{l+1} per edge, or null
   DevStatus* status;
 };
 
 // message layer l over all edges (see the file header); edge q = (row i, col[q] = j).
-// ENC: e_0 from the edge features (first layer); PE: the decoder's edge term (last layer)
-template <bool ENC, bool PE>
+// The row sums are formed here: a warp owns 32 consecutive edges, 32 w .. 32 w + 31, and adds
+// the messages of each row in order.  A row i whose edges all belong to the warp goes to
+// agg[i]; the piece of a row that began before the warp's edges goes to agg[n + 2 w], the
+// piece of a row that begins among them and goes on behind them to agg[n + 2 w + 1]; the
+// node update adds the pieces in order.  m itself (128 bytes an edge written here and read
+// back there) is only stored for the backward.
+// ENC: e_0 from the edge features and, in inference, h_0 from the node features (first
+// layer); PE: the decoder's edge term (last layer); TRAIN: every activation is stored,
+// otherwise only e_{l+1} of the layers before the last
+template <bool ENC, bool PE, bool TRAIN>
 __global__ void __launch_bounds__(TNT, TCTAS) message_tc_kernel(const __grid_constant__ MsgArgs P) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
@@ -279,26 +291,67 @@ __global__ void __launch_bounds__(TNT, TCTAS) message_tc_kernel(const __grid_con
     for (int k = 0; k < 3; ++k) s_we[32 * k + lane] = __bfloat162float(P.w[OFF_WE + 32 * k + lane]);
   }
   __syncthreads();
+  constexpr bool HF = ENC && !TRAIN;  // h_0 = relu(Wn f + bn) of the column's node, lane = channel
+  float wn0 = 0.f, wn1 = 0.f, bn = 0.f;
+  if (HF) {
+    wn0 = __bfloat162float(P.w[OFF_WN + 2 * lane]);
+    wn1 = __bfloat162float(P.w[OFF_WN + 2 * lane + 1]);
+    bn = __bfloat162float(P.w[OFF_BN + lane]);
+  }
   const int64_t nnz = P.nnz;
   const int64_t ntiles = (nnz + TT - 1) / TT;
   bool bad = false;
   int it = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
     const int64_t e0 = tile * TT + warp * 32;
-    int cj = -1;
-    if (e0 + lane < nnz) {
+    const bool full = e0 + 32 <= nnz;  // (no bounds checks in the loops below)
+    const int nv = (int)std::min<int64_t>(32, std::max<int64_t>(0, nnz - e0));  // valid edges
+    int cj = 0, ri = -1;
+    if (lane < nv) {
       cj = P.col[e0 + lane];
+      ri = P.erow[e0 + lane];
       if (cj < 0 || (int64_t)cj >= P.n) {
-        bad = true;
-        cj = -1;
+        bad = true;  // reported; the row read instead does not matter
+        cj = 0;
       }
     }
+    // rows of the warp's edges: where this lane's edge ends a row's piece, the row of agg it
+    // goes to
+    const int rn = __shfl_down_sync(0xffffffffu, ri, 1);
+    const bool end = lane < nv && (lane + 1 == nv || rn != ri);
+    const unsigned ends = __ballot_sync(0xffffffffu, end);
+    uint32_t slot = (uint32_t)ri;
+    if (end) {
+      const bool first = (ends & ((1u << lane) - 1u)) == 0u;
+      const int rs = P.rowptr[ri], re = P.rowptr[ri + 1];
+      if (first && (int64_t)rs < e0) slot = (uint32_t)P.n + 2u * (uint32_t)(e0 >> 5);
+      else if ((int64_t)re > e0 + nv) slot = (uint32_t)P.n + 2u * (uint32_t)(e0 >> 5) + 1u;
+    }
     float ev[32], hv[32];
+    if constexpr (!ENC) {
+      const float* el = P.ein + e0 * W + lane;
+      if (full) {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const int c = __shfl_sync(0xffffffffu, cj, j);
-      if constexpr (!ENC) ev[j] = e0 + j < nnz ? P.ein[(e0 + j) * W + lane] : 0.f;
-      hv[j] = c >= 0 ? P.h[(int64_t)c * W + lane] : 0.f;
+        for (int j = 0; j < 32; ++j) ev[j] = el[j * W];
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) ev[j] = j < nv ? el[j * W] : 0.f;
+      }
+    }
+    if constexpr (HF) {
+      const float2 fj = lane < nv ? *reinterpret_cast<const float2*>(P.f + 2 * (int64_t)cj) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const float f0 = __shfl_sync(0xffffffffu, fj.x, j), f1 = __shfl_sync(0xffffffffu, fj.y, j);
+        hv[j] = relu_tc(fmaf(wn1, f1, fmaf(wn0, f0, bn)));
+      }
+    } else {
+      const float* hl = P.h + lane;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const int64_t c = __shfl_sync(0xffffffffu, cj, j);  // (0 past the last edge)
+        hv[j] = hl[c * W];
+      }
     }
     float x0 = 0.f, x1 = 0.f, x2 = 0.f;  // first layer: this thread's edge features
     if (ENC && e0 + lane < nnz) {
@@ -343,28 +396,43 @@ __global__ void __launch_bounds__(TNT, TCTAS) message_tc_kernel(const __grid_con
       }
       if (e0 + lane < nnz) P.pe[e0 + lane] = t;
     }
-    float* __restrict__ eout = P.eout;
-#pragma unroll 8
-    for (int j = 0; j < 32; ++j) {
-      if (e0 + j < nnz) {
-        const float mv = relu_tc(buf[j * TLD + 32 + lane] + bias);
-        P.m[(e0 + j) * W + lane] = mv;
-        if (eout) eout[(e0 + j) * W + lane] = buf[j * TLD + lane] + mv;
-      }
+    float run = 0.f;
+    float* aggl = P.agg + lane;
+    float* eo = P.eout + e0 * W + lane;
+    float* mo = P.m + e0 * W + lane;
+    auto store = [&](int j) {
+      const float mv = relu_tc(buf[j * TLD + 32 + lane] + bias);
+      if constexpr (TRAIN) mo[j * W] = mv;
+      if constexpr (TRAIN || !PE) eo[j * W] = (ENC ? buf[j * TLD + lane] : ev[j]) + mv;
+      run += mv;
+      const uint32_t sj = __shfl_sync(0xffffffffu, slot, j);
+      const bool ej = (ends >> j) & 1u;
+      if (ej) aggl[(int64_t)sj * W] = run;
+      run = ej ? 0.f : run;
+    };
+    if (full) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) store(j);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (j < nv) store(j);
     }
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) set_error(P.status, RBO_ERR_ARG, 41);
   tc_teardown(&s_fin, tbase);
 }
 
-// aggregation + node update of layer l over all nodes (see the file header)
-// agg, rh and hout may be null (inference keeps only what the next layer reads); sdec
-// and tdec, when non-null, receive the decoder's node terms wo[32:64] . h' and
+// node update of layer l over all nodes (see the file header); agg holds the row sums as the
+// message layer left them, rows in pieces are completed here (and stored in agg
+// with keep_agg, for the backward).  hin null: h_0 from the node features f.  rh and hout may be null (inference keeps only
+// what the next layer reads); sdec and tdec, when non-null, receive the decoder's node terms wo[32:64] . h' and
 // wo[64:96] . h' (the last layer)
 __global__ void __launch_bounds__(TNT, TCTAS)
-    node_update_tc_kernel(int64_t n, const int32_t* __restrict__ rowptr, const float* __restrict__ m,
-                          const float* __restrict__ hin, const __nv_bfloat16* __restrict__ w, int l,
-                          float* __restrict__ agg, float* __restrict__ rh, float* __restrict__ hout,
+    node_update_tc_kernel(int64_t n, const int32_t* __restrict__ rowptr, float* __restrict__ agg,
+                          int keep_agg, const float* __restrict__ hin, const float* __restrict__ f,
+                          const __nv_bfloat16* __restrict__ w, int l,
+                          float* __restrict__ rh, float* __restrict__ hout,
                           float* __restrict__ sdec, float* __restrict__ tdec, DevStatus* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
@@ -389,56 +457,63 @@ __global__ void __launch_bounds__(TNT, TCTAS)
     s_woj[lane] = __bfloat162float(w[OFF_WO + 2 * W + lane]);
   }
   __syncthreads();
+  const float wn0 = __bfloat162float(w[OFF_WN + 2 * lane]), wn1 = __bfloat162float(w[OFF_WN + 2 * lane + 1]),
+              bn = __bfloat162float(w[OFF_BN + lane]);
+  const float* bpart = agg + n * W;  // pieces of rows cut by a warp's edge range
   const int64_t ntiles = (n + TT - 1) / TT;
   int it = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
     const int64_t i0 = tile * TT + warp * 32;
-    // row starts of the warp's 32 nodes (lanes past the last node: rowptr[n], above every
-    // edge of the range) and the end of the warp's edge range
-    const int rs = rowptr[std::min<int64_t>(i0 + lane, n)];
-    const int E0 = __shfl_sync(0xffffffffu, rs, 0);
-    const int E1 = rowptr[std::min<int64_t>(i0 + 32, n)];
+    // this lane's node: its first and last edge warps (w0 < 0: no edges)
+    int w0 = -1, w1 = -1;
+    if (i0 + lane < n) {
+      const int rs = rowptr[i0 + lane], re = rowptr[i0 + lane + 1];
+      if (re > rs) {
+        w0 = rs >> 5;
+        w1 = (re - 1) >> 5;
+      }
+    }
+    const unsigned pieces = __ballot_sync(0xffffffffu, w1 > w0);
     {
-      float hv[32];
+      float hv[32], av[32];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) hv[j] = i0 + j < n ? hin[(i0 + j) * W + lane] : 0.f;
+      for (int j = 0; j < 32; ++j) {
+        const int a = __shfl_sync(0xffffffffu, w0, j);
+        const bool cut = (pieces >> j) & 1u;
+        const float* p = cut ? bpart + ((int64_t)a * 2 + 1) * W + lane : agg + (i0 + j) * W + lane;
+        if (hin) hv[j] = i0 + j < n ? hin[(i0 + j) * W + lane] : 0.f;
+        av[j] = a >= 0 ? *p : 0.f;
+      }
+      if (!hin) {  // first layer of inference: h_0 from the node features
+        const float2 fj = i0 + lane < n ? *reinterpret_cast<const float2*>(f + 2 * (i0 + lane)) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const float f0 = __shfl_sync(0xffffffffu, fj.x, j), f1 = __shfl_sync(0xffffffffu, fj.y, j);
+          hv[j] = relu_tc(fmaf(wn1, f1, fmaf(wn0, f0, bn)));
+        }
+      }
       __syncwarp();  // the previous tile's reads of the buffer are done
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         buf[j * TLD + lane] = hv[j];
-        buf[j * TLD + 32 + lane] = 0.f;  // nodes without edges
+        buf[j * TLD + 32 + lane] = av[j];
       }
     }
-    // incoming messages in CSR order, 32 edges in flight; an edge belongs to the last node
-    // whose row starts at or before it; each node's sum starts from 0 and adds its edges
-    // in order
-    int cur = -1;
-    float run = 0.f;
-    for (int e = E0; e < E1; e += 32) {
-      float v[32];
-#pragma unroll
-      for (int u = 0; u < 32; ++u) v[u] = e + u < E1 ? m[(int64_t)(e + u) * W + lane] : 0.f;
-#pragma unroll
-      for (int u = 0; u < 32; ++u) {
-        // branch-free: a new node stores the previous node's sum and restarts from this
-        // edge (0 + v = v, the same value as an explicit restart); edges past the range
-        // keep the node and add 0
-        const unsigned mask = __ballot_sync(0xffffffffu, rs <= e + u);
-        const int j = e + u < E1 ? 31 - __clz((int)mask) : cur;
-        const bool fresh = j != cur;
-        if (fresh && cur >= 0) buf[cur * TLD + 32 + lane] = run;
-        run = fresh ? v[u] : run + v[u];
-        cur = j;
-      }
+    // the rows in pieces: the remaining pieces in order
+    for (unsigned p = pieces; p != 0u; p &= p - 1u) {
+      const int j = __ffs((int)p) - 1;
+      const int a = __shfl_sync(0xffffffffu, w0, j), e = __shfl_sync(0xffffffffu, w1, j);
+      float s = buf[j * TLD + 32 + lane];
+      for (int k = a + 1; k <= e; ++k) s += bpart[(int64_t)k * 2 * W + lane];
+      buf[j * TLD + 32 + lane] = s;
+      if (keep_agg) agg[(i0 + j) * W + lane] = s;
     }
-    if (cur >= 0) buf[cur * TLD + 32 + lane] = run;
-    __syncwarp();
-    if (agg) {
+    if (keep_agg) {  // nodes without edges
 #pragma unroll 8
       for (int j = 0; j < 32; ++j)
-        if (i0 + j < n) agg[(i0 + j) * W + lane] = buf[j * TLD + 32 + lane];
+        if (i0 + j < n && __shfl_sync(0xffffffffu, w0, j) < 0) agg[(i0 + j) * W + lane] = 0.f;
     }
-    __syncwarp();  // agg read before tile_products overwrites the columns with outputs
+    __syncwarp();
     if (!tile_products(buf, tbase, tlane, Bs, &s_mma, it)) {
       if (tid == 0) set_error(status, RBO_ERR_TIMEOUT, 42);
       break;
@@ -749,29 +824,30 @@ static int tc_grid(int64_t items) {
   return (int)std::min<int64_t>(tiles, (int64_t)TCTAS * std::max(sms, 1));
 }
 
-int message_tc_launch(int64_t nnz, int64_t n, const int32_t* col, const float* ein, const float* x,
-                      float* e0out, const float* h, const __nv_bfloat16* w, int l, float* m,
-                      float* eout, float* pe, DevStatus* status, cudaStream_t st) {
+int message_tc_launch(bool train, int64_t nnz, int64_t n, const int32_t* rowptr, const int32_t* erow,
+                      const int32_t* col, const float* ein, const float* x, float* e0out, const float* h,
+                      const float* f, const __nv_bfloat16* w, int l, float* agg, float* m, float* eout, float* pe,
+                      DevStatus* status, cudaStream_t st) {
   if (nnz <= 0) return RBO_OK;
-  const MsgArgs P{nnz, n, col, ein, x, e0out, h, w, l, m, eout, pe, status};
-  const int G = tc_grid(nnz);
-  if (!ein && pe)
-    message_tc_kernel<true, true><<<G, TNT, TSMEM, st>>>(P);
-  else if (!ein)
-    message_tc_kernel<true, false><<<G, TNT, TSMEM, st>>>(P);
-  else if (pe)
-    message_tc_kernel<false, true><<<G, TNT, TSMEM, st>>>(P);
+  const MsgArgs P{nnz, n, col, ein, x, e0out, h, f, w, l, rowptr, erow, agg, m, eout, pe, status};
+  void (*k)(MsgArgs) = nullptr;
+  const bool enc = ein == nullptr, dec = pe != nullptr;
+  if (train)
+    k = enc ? (dec ? message_tc_kernel<true, true, true> : message_tc_kernel<true, false, true>)
+            : (dec ? message_tc_kernel<false, true, true> : message_tc_kernel<false, false, true>);
   else
-    message_tc_kernel<false, false><<<G, TNT, TSMEM, st>>>(P);
+    k = enc ? (dec ? message_tc_kernel<true, true, false> : message_tc_kernel<true, false, false>)
+            : (dec ? message_tc_kernel<false, true, false> : message_tc_kernel<false, false, false>);
+  k<<<tc_grid(nnz), TNT, TSMEM, st>>>(P);
   return note_cuda(cudaGetLastError());
 }
 
-int node_update_tc_launch(int64_t n, const int32_t* rowptr, const float* m, const float* hin,
-                          const __nv_bfloat16* w, int l, float* agg, float* rh, float* hout,
-                          float* sdec, float* tdec, DevStatus* status, cudaStream_t st) {
+int node_update_tc_launch(int64_t n, const int32_t* rowptr, float* agg, int keep_agg, const float* hin,
+                          const float* f, const __nv_bfloat16* w, int l, float* rh, float* hout, float* sdec,
+                          float* tdec, DevStatus* status, cudaStream_t st) {
   if (n <= 0) return RBO_OK;
-  node_update_tc_kernel<<<tc_grid(n), TNT, TSMEM, st>>>(n, rowptr, m, hin, w, l, agg, rh, hout, sdec,
-                                                        tdec, status);
+  node_update_tc_kernel<<<tc_grid(n), TNT, TSMEM, st>>>(n, rowptr, agg, keep_agg, hin, f, w, l, rh, hout,
+                                                        sdec, tdec, status);
   return note_cuda(cudaGetLastError());
 }
 
