@@ -63,104 +63,97 @@ __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, int64_t nnz,
 }
 
 
-// Short rows: each warp takes groups of 32 consecutive rows (persistent grid of 4
-// blocks per SM; the row pointers of the warp's next group are loaded while the
-// current group is processed).  The warp stages the entries of its rows in chunks of
-// SCH (coalesced index and value loads, the x gathers issued by the same lanes), then
-// every lane runs the multiply-adds of its own row from shared memory, as two
-// interleaved chains (even and odd entries) added at the end.  No cross-lane float64
-// reduction is needed: each float64 operation costs a slot of this GPU's narrow
-// float64 pipe.
-constexpr int SCH = 256;
-__global__ void __launch_bounds__(256) spmv_stream_kernel(int64_t n, int64_t nnz,
-                                                          const int32_t* __restrict__ rowptr,
-                                                          const int32_t* __restrict__ col,
-                                                          const double* __restrict__ val,
-                                                          const double* __restrict__ dscale,
-                                                          const double* __restrict__ x,
-                                                          const double* __restrict__ bvec,
-                                                          double* __restrict__ y, DevStatus* status,
-                                                          SpmvShift sh) {
-  __shared__ double sv[8][SCH], sx[8][SCH];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t ngroups = (n + 31) / 32;
-  const int64_t gstride = (int64_t)gridDim.x * 8;
-  int64_t g = (int64_t)blockIdx.x * 8 + warp;
-  int beg = 0, end = 0;
-  if (g < ngroups && g * 32 + lane < n) {
-    beg = __ldg(rowptr + g * 32 + lane);
-    end = __ldg(rowptr + g * 32 + lane + 1);
-  }
-  for (; g < ngroups; g += gstride) {
-    // row pointers of this warp's next group, in flight during this group
-    const int64_t gn = g + gstride;
-    int nbeg = 0, nend = 0;
-    if (gn < ngroups && gn * 32 + lane < n) {
-      nbeg = __ldg(rowptr + gn * 32 + lane);
-      nend = __ldg(rowptr + gn * 32 + lane + 1);
+// Short rows: a block takes 256 consecutive rows, whose indices and values are two
+// contiguous pieces of the CSR arrays; the bulk-copy engine brings them into shared memory
+// (no load instructions and no registers for the bytes in flight, which bound an earlier
+// form that staged 32 rows per warp with plain loads), then every thread walks its own row,
+// the x gathers of 8 entries in flight.  Two interleaved chains per row (even and odd
+// entries) added at the end, a fixed order; no cross-lane float64 reduction.  Blocks with
+// more entries than the staging holds (`cap`), malformed row pointers or unaligned arrays
+// read them from global memory instead.  SCALE is a template argument because the float64
+// pipe (2 operations per SM and cycle) bounds the kernel: a multiplication by a scale that
+// is not there would be half of its work.
+constexpr int SPR = 256;  // rows (threads) per block
+template <bool SCALE>
+__global__ void __launch_bounds__(SPR, 6) spmv_block_kernel(int64_t n, int64_t nnz, int cap,
+                                                         const int32_t* __restrict__ rowptr,
+                                                         const int32_t* __restrict__ col,
+                                                         const double* __restrict__ val,
+                                                         const double* __restrict__ dscale,
+                                                         const double* __restrict__ x,
+                                                         const double* __restrict__ bvec,
+                                                         double* __restrict__ y, DevStatus* status,
+                                                         SpmvShift sh) {
+  extern __shared__ __align__(16) unsigned char sm_sp[];
+  __shared__ __align__(8) uint64_t bar;
+  double* sval = reinterpret_cast<double*>(sm_sp);                 // cap + 2 values
+  int32_t* scol = reinterpret_cast<int32_t*>(sval + cap + 2);       // cap + 4 indices
+  const int tid = threadIdx.x;
+  const int64_t r0 = blockIdx.x * (int64_t)SPR, r = r0 + tid;
+  const int64_t rl = r0 + SPR < n ? r0 + SPR : n;
+  const int e0 = __ldg(rowptr + r0), e1 = __ldg(rowptr + rl);
+  const bool staged = cap > 0 && e0 >= 0 && e1 >= e0 && (int64_t)e1 <= nnz && e1 - e0 <= cap;
+  // 16-byte aligned starts at or before e0, whole 16-byte pieces before e1
+  const int v0 = e0 & ~1, c0 = e0 & ~3;
+  if (staged) {
+    const uint32_t bv = (uint32_t)(e1 - v0) * 8u & ~15u, bc = (uint32_t)(e1 - c0) * 4u & ~15u;
+    if (tid == 0) {
+      mbar_init(&bar, 1);
+      fence_mbar_init();
+      mbar_arrive_expect_tx(&bar, bv + bc);
+      if (bv) bulk_copy_g2s(sval, val + v0, bv, &bar);
+      if (bc) bulk_copy_g2s(scol, col + c0, bc, &bar);
     }
-    const int64_t r0 = g * 32, r = r0 + lane;
-    const int nr = (int)((n - r0) < 32 ? (n - r0) : 32);
-    const int e0 = __shfl_sync(0xffffffffu, beg, 0);
-    const int e1 = __shfl_sync(0xffffffffu, end, nr - 1);
-    const bool range_ok = e0 >= 0 && e1 >= e0 && (int64_t)e1 <= nnz;
-    if (r < n && (!range_ok || beg < e0 || end < beg || end > e1)) {
+    // what is left after the whole pieces
+    for (int e = v0 + (int)(bv / 8) + tid; e < e1; e += SPR) sval[e - v0] = __ldg(val + e);
+    for (int e = c0 + (int)(bc / 4) + tid; e < e1; e += SPR) scol[e - c0] = __ldg(col + e);
+  }
+  int beg = 0, end = 0;
+  if (r < n) {
+    beg = __ldg(rowptr + r);
+    end = __ldg(rowptr + r + 1);
+    const bool bad = staged ? (beg < e0 || end < beg || end > e1) : (beg < 0 || end < beg || (int64_t)end > nnz);
+    if (bad) {
       if (status) set_error(status, RBO_ERR_ARG, 11);
       end = beg;
     }
-    double s = 0.0, s2 = 0.0;
-    if (range_ok) {
-      for (int c0 = e0; c0 < e1; c0 += SCH) {
-        const int cn = (e1 - c0) < SCH ? (e1 - c0) : SCH;
-        int cj[SCH / 32];
-        double v[SCH / 32], xv[SCH / 32];
+  }
+  __syncthreads();
+  if (staged && !mbar_wait_bounded(&bar, 0u)) {
+    if (status) set_error(status, RBO_ERR_TIMEOUT, 13);
+    return;
+  }
+  if (r >= n) return;
+  double s0 = 0.0, s1 = 0.0;
+  bool bad = false;
+  auto walk = [&](const int32_t* cp, const double* vp, int len) {
+    for (int e = 0; e < len; e += 8) {
+      const int k = len - e;  // entries left
+      int c[8];
+      double v[8], xv[8];
 #pragma unroll
-        for (int u = 0; u < SCH / 32; ++u) {
-          const int t = u * 32 + lane;
-          cj[u] = -1;
-          v[u] = 0.0;
-          if (t < cn) {
-            cj[u] = __ldg(col + c0 + t);
-            v[u] = __ldg(val + c0 + t);
-          }
-        }
+      for (int j = 0; j < 8; ++j) c[j] = j < k ? cp[e + j] : 0;
 #pragma unroll
-        for (int u = 0; u < SCH / 32; ++u) {
-          const int t = u * 32 + lane;
-          xv[u] = 0.0;
-          if (t < cn) {
-            if (cj[u] < 0 || (int64_t)cj[u] >= n) {
-              if (status) set_error(status, RBO_ERR_ARG, 12);
-              v[u] = 0.0;
-            } else {
-              xv[u] = dscale ? __ldg(dscale + cj[u]) * __ldg(x + cj[u]) : __ldg(x + cj[u]);
-            }
-          }
-        }
+      for (int j = 0; j < 8; ++j) {
+        const bool ok = (uint64_t)(int64_t)c[j] < (uint64_t)n;
+        bad = bad || !ok;
+        const int cj = ok ? c[j] : 0;
+        xv[j] = __ldg(x + cj);
+        if (SCALE) xv[j] *= __ldg(dscale + cj);
+        v[j] = ok && j < k ? vp[e + j] : 0.0;
+      }
 #pragma unroll
-        for (int u = 0; u < SCH / 32; ++u) {
-          const int t = u * 32 + lane;
-          if (t < cn) {
-            sv[warp][t] = v[u];
-            sx[warp][t] = xv[u];
-          }
-        }
-        __syncwarp();
-        const int lo = beg > c0 ? beg : c0, hi = end < c0 + cn ? end : c0 + cn;
-        int e = lo;
-        for (; e + 1 < hi; e += 2) {
-          s = fma(sv[warp][e - c0], sx[warp][e - c0], s);
-          s2 = fma(sv[warp][e + 1 - c0], sx[warp][e + 1 - c0], s2);
-        }
-        if (e < hi) s = fma(sv[warp][e - c0], sx[warp][e - c0], s);
-        __syncwarp();
+      for (int j = 0; j < 8; j += 2) {
+        if (j < k) s0 = fma(v[j], xv[j], s0);
+        if (j + 1 < k) s1 = fma(v[j + 1], xv[j + 1], s1);
       }
     }
-    s += s2;
-    if (r < n) y[r] = bvec ? (bvec[r] - s) : shifted(s, sh, r);
-    beg = nbeg;
-    end = nend;
-  }
+  };
+  if (staged) walk(scol + (beg - c0), sval + (beg - v0), end - beg);
+  else walk(col + beg, val + beg, end - beg);
+  if (bad && status) set_error(status, RBO_ERR_ARG, 12);
+  const double s = s0 + s1;
+  y[r] = bvec ? (bvec[r] - s) : shifted(s, sh, r);
 }
 
 static int spmv_dispatch_inner(const CsrDev& A, const double* dscale, const double* x,
@@ -200,12 +193,18 @@ static int spmv_dispatch_inner(const CsrDev& A, const double* dscale, const doub
                                const SpmvShift& sh) {
   const double avg = A.n > 0 ? (double)A.nnz / (double)A.n : 0.0;
   if (avg <= 12.0) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t blocks = std::min<int64_t>((A.n + 255) / 256, (int64_t)std::max(sms, 1) * 4);
-    spmv_stream_kernel<<<(unsigned)blocks, 256, 0, st>>>(A.n, A.nnz, A.rowptr, A.col, A.val, dscale,
-                                                          x, b, y, status, sh);
+    const int64_t blocks = (A.n + SPR - 1) / SPR;
+    if (blocks > 0x7FFFFFFFLL) return RBO_ERR_ARG;
+    // staging for a quarter more entries than the average block has (at most 3840: 46 KB)
+    const bool aligned = ((uintptr_t)A.col & 15) == 0 && ((uintptr_t)A.val & 15) == 0;
+    const int cap = aligned ? ((int)(avg * SPR * 1.25) + 67) & ~3 : 0;
+    const size_t smem = (size_t)(cap + 2) * 8 + (size_t)(cap + 4) * 4;
+    if (dscale)
+      spmv_block_kernel<true><<<(unsigned)blocks, SPR, smem, st>>>(A.n, A.nnz, cap, A.rowptr, A.col, A.val, dscale,
+                                                                   x, b, y, status, sh);
+    else
+      spmv_block_kernel<false><<<(unsigned)blocks, SPR, smem, st>>>(A.n, A.nnz, cap, A.rowptr, A.col, A.val, dscale,
+                                                                    x, b, y, status, sh);
   } else if (avg <= 24.0)
     spmv_go<8>(A, dscale, x, b, y, status, st, sh);
   else
