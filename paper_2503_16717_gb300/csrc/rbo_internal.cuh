@@ -198,7 +198,7 @@ int skb2_launch(const double* v, int nparts, int64_t stride, double* qs, double*
 // call so that the row pass needs neither hashing nor a scatter with conflicts.
 // Record of a tile (rec_bytes, a 16-byte multiple):
 //   meta[mcap] (uint32): one per non-empty sketch row i of the tile, sorted by the
-//       number of entries (descending, then i): i | offset << 12 | count << 23;
+//       number of entries (descending): i | offset << 12 | count << 23;
 //       0xFFFFFFFF past the last;
 //   list[T * zeta] (uint8): the tile's entries grouped by sketch row (rows in
 //       increasing order within a group): local row << 1 | (sign < 0).

@@ -684,108 +684,104 @@ size_t sketch_sched_bytes(int64_t n, int T, int d, int zeta) {
   return (size_t)((n + T - 1) / T) * (size_t)sketch_sched_rec_bytes(T, d, zeta);
 }
 
-static int next_pow2(int v) {
-  int p = 1;
-  while (p < v) p <<= 1;
-  return p;
-}
-
-// ascending bitonic sort of N (a power of two) keys in shared memory, whole block
-template <typename K>
-__device__ void block_bitonic_sort(K* key, int N) {
-  for (int k = 2; k <= N; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const int l = i ^ j;
-        if (l > i) {
-          const K x = key[i], y = key[l];
-          if ((x > y) == ((i & k) == 0)) {
-            key[i] = y;
-            key[l] = x;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-// One CTA per tile: hash the tile's rows (SplitMix64 sparse-sign columns), sort the
-// (sketch row, pair) keys, then sort the non-empty sketch rows by entry count.
-// Keys are unique, so the result does not depend on thread timing.
-__global__ void sketch_sched_kernel(int64_t n, int T, int d, int zeta, uint64_t seed, int np2,
-                                    int mp2, int mcap, int rec_bytes, uint8_t* out,
-                                    DevStatus* status) {
+// One CTA of 64 threads per tile of T <= 64 rows.  Every thread hashes one row (SplitMix64
+// sparse-sign column) and sets its bit in the row and sign masks of the sketch rows it
+// hits: the masks are the transposed tile, entries already in increasing row.  Then the
+// non-empty sketch rows are placed by entry count: a histogram of the counts and a scan
+// over it give the first slot and list position of every count, an atomic the place among
+// equal counts (the order of equal slots does not affect any sum).  (An earlier form sorted
+// keys with a bitonic network: 403 us for 10^6 rows, d = 244, zeta = 8.)
+constexpr int SCHED_NT = 64;
+__global__ void __launch_bounds__(SCHED_NT) sketch_sched_kernel(int64_t n, int T, int d, int zeta, uint64_t seed,
+                                                                int mcap, int rec_bytes, uint8_t* out,
+                                                                DevStatus* status) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  unsigned long long* rkey = reinterpret_cast<unsigned long long*>(sm_raw);  // mp2
-  uint32_t* key = reinterpret_cast<uint32_t*>(rkey + mp2);                    // np2
-  __shared__ int s_nrow;
-  const int tile = blockIdx.x, tid = threadIdx.x;
-  const int64_t r0 = (int64_t)tile * T;
+  uint32_t* meta = reinterpret_cast<uint32_t*>(sm_raw);              // the record: mcap words
+  uint8_t* lst = reinterpret_cast<uint8_t*>(meta + mcap);             // and T * zeta bytes
+  uint32_t* mask = reinterpret_cast<uint32_t*>(sm_raw + rec_bytes);   // d x (rows lo, hi, signs lo, hi)
+  __shared__ int hist[66], slot0[66], off0[66], s_scan[4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t tile = blockIdx.x, r0 = tile * T;
   const int rows = (int)std::min<int64_t>((int64_t)T, n - r0);
-  const int np = T * zeta;
-  if (tid == 0) s_nrow = 0;
-  for (int t = tid; t < np2; t += blockDim.x) key[t] = 0xFFFFFFFFu;
-  for (int t = tid; t < mp2; t += blockDim.x) rkey[t] = ~0ull;
+  for (int t = tid; t < 4 * d; t += SCHED_NT) mask[t] = 0u;
+  for (int t = tid; t < rec_bytes / 4; t += SCHED_NT) meta[t] = t < mcap ? 0xFFFFFFFFu : 0u;
+  for (int t = tid; t < 66; t += SCHED_NT) hist[t] = 0;
   __syncthreads();
-  for (int r = tid; r < rows; r += blockDim.x) {
+  if (tid < rows) {
     int ix[ZMAX], ng[ZMAX];
 #pragma unroll
     for (int t = 0; t < ZMAX; ++t) { ix[t] = 0; ng[t] = 0; }
-    if (!sketch_column(seed, (uint64_t)(r0 + r), d, zeta, ix, ng)) set_error(status, RBO_ERR_SKETCH, 2);
+    if (!sketch_column(seed, (uint64_t)(r0 + tid), d, zeta, ix, ng)) set_error(status, RBO_ERR_SKETCH, 2);
 #pragma unroll
     for (int t = 0; t < ZMAX; ++t) {
       if (t < zeta) {
-        const uint32_t p = (uint32_t)(r * zeta + t);
-        key[p] = ((uint32_t)ix[t] << 12) | (p << 1) | (uint32_t)ng[t];
+        atomicOr(&mask[4 * ix[t] + warp], 1u << lane);
+        if (ng[t]) atomicOr(&mask[4 * ix[t] + 2 + warp], 1u << lane);
       }
     }
   }
   __syncthreads();
-  block_bitonic_sort(key, np2);
-  uint8_t* rec = out + (size_t)tile * rec_bytes;
-  uint32_t* meta = reinterpret_cast<uint32_t*>(rec);
-  uint8_t* lst = rec + (size_t)mcap * 4;
-  const int nvalid = rows * zeta;
-  for (int q = tid; q < np; q += blockDim.x) {
-    uint8_t v = 0;
-    if (q < nvalid) {
-      const uint32_t kq = key[q];
-      const int p = (int)((kq >> 1) & 0x7FFu);
-      v = (uint8_t)(((p / zeta) << 1) | (int)(kq & 1u));
-      const uint32_t i = kq >> 12;
-      if (q == 0 || (key[q - 1] >> 12) != i) {  // first entry of sketch row i
-        int e = q + 1;
-        while (e < nvalid && (key[e] >> 12) == i) ++e;
-        const uint32_t cnt = (uint32_t)(e - q);
-        const uint32_t m = i | ((uint32_t)q << 12) | (cnt << 23);
-        const unsigned long long sk = ((unsigned long long)(511u - cnt) << 12) | i;
-        const int slot = atomicAdd(&s_nrow, 1);
-        rkey[slot] = (sk << 32) | m;
-      }
-    }
-    lst[q] = v;
+  for (int i = tid; i < d; i += SCHED_NT) {
+    const int c = __popc(mask[4 * i]) + __popc(mask[4 * i + 1]);
+    if (c) atomicAdd(&hist[c], 1);
   }
   __syncthreads();
-  block_bitonic_sort(rkey, mp2);
-  for (int q = tid; q < mcap; q += blockDim.x)
-    meta[q] = q < s_nrow ? (uint32_t)(rkey[q] & 0xFFFFFFFFull) : 0xFFFFFFFFu;
-  // zero the record's padding
-  for (int t = mcap * 4 + np + tid; t < rec_bytes; t += blockDim.x) rec[t] = 0;
+  {  // exclusive scans over the counts 64, 63, .., 1 (thread t: count 64 - t)
+    const int c = 64 - tid, h = hist[c], w = h * c;
+    int a = h, b = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, a, o), y = __shfl_up_sync(0xffffffffu, b, o);
+      if (lane >= o) {
+        a += x;
+        b += y;
+      }
+    }
+    if (lane == 31) {
+      s_scan[2 * warp] = a;
+      s_scan[2 * warp + 1] = b;
+    }
+    __syncthreads();
+    slot0[c] = a - h + (warp ? s_scan[0] : 0);
+    off0[c] = b - w + (warp ? s_scan[1] : 0);
+    hist[c] = 0;  // now: places taken among the rows of this count
+  }
+  __syncthreads();
+  for (int i = tid; i < d; i += SCHED_NT) {
+    const uint32_t lo = mask[4 * i], hi = mask[4 * i + 1], sl = mask[4 * i + 2], sh = mask[4 * i + 3];
+    const int c = __popc(lo) + __popc(hi);
+    if (!c) continue;
+    const int k = atomicAdd(&hist[c], 1);
+    int o = off0[c] + k * c;
+    meta[slot0[c] + k] = (uint32_t)i | ((uint32_t)o << 12) | ((uint32_t)c << 23);
+    for (uint32_t m = lo; m; m &= m - 1u) {
+      const int r = __ffs((int)m) - 1;
+      lst[o++] = (uint8_t)((r << 1) | ((sl >> r) & 1u));
+    }
+    for (uint32_t m = hi; m; m &= m - 1u) {
+      const int r = __ffs((int)m) - 1;
+      lst[o++] = (uint8_t)(((r + 32) << 1) | ((sh >> r) & 1u));
+    }
+  }
+  __syncthreads();
+  uint4* rec = reinterpret_cast<uint4*>(out + (size_t)tile * rec_bytes);
+  for (int t = tid; t < rec_bytes / 16; t += SCHED_NT) rec[t] = reinterpret_cast<const uint4*>(sm_raw)[t];
 }
 
 int sketch_sched_launch(int64_t n, int T, int d, int zeta, uint64_t seed, uint8_t* out,
                         DevStatus* status, cudaStream_t st) {
-  if (n <= 0 || (T != 16 && T != 32 && T != 64 && T != 128) || d < 1 || d > DMAX || zeta < 1 ||
-      zeta > ZMAX || zeta > d || !out)
+  if (n <= 0 || (T != 16 && T != 32 && T != 64) || d < 1 || d > DMAX || zeta < 1 || zeta > ZMAX || zeta > d || !out)
     return RBO_ERR_ARG;
-  const int np2 = next_pow2(T * zeta), mcap = sketch_sched_mcap(T, d, zeta);
-  const int mp2 = next_pow2(mcap);
-  const size_t smem = (size_t)mp2 * 8 + (size_t)np2 * 4;
+  const int mcap = sketch_sched_mcap(T, d, zeta), rec = sketch_sched_rec_bytes(T, d, zeta);
+  const size_t smem = (size_t)rec + (size_t)d * 16;  // at most 17 KB + 64 KB
   const int64_t ntiles = (n + T - 1) / T;
-  sketch_sched_kernel<<<(unsigned)ntiles, NT, smem, st>>>(n, T, d, zeta, seed, np2, mp2, mcap,
-                                                          sketch_sched_rec_bytes(T, d, zeta), out,
-                                                          status);
+  if (ntiles > 0x7FFFFFFFLL) return RBO_ERR_ARG;
+  if (smem > 48 * 1024) {
+    const int e = note_cuda(cudaFuncSetAttribute(sketch_sched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 96 * 1024));
+    if (e != RBO_OK) return e;
+  }
+  sketch_sched_kernel<<<(unsigned)ntiles, SCHED_NT, smem, st>>>(n, T, d, zeta, seed, mcap, rec, out, status);
   return cudaGetLastError() == cudaSuccess ? RBO_OK : RBO_ERR_CUDA;
 }
 
