@@ -169,29 +169,45 @@ __device__ __forceinline__ void fx_mma(float (&d)[4], uint32_t a0, uint32_t a1, 
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// the same with another addend: d = A B + c
+__device__ __forceinline__ void fx_mma_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                             uint32_t b0, uint32_t b1, const float (&c)[4]) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%10, %11, %12, %13};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+
 // All pairs I + J <= 6 of one K step: A = four pairs of values, p[row half][K half] (rows
 // g / g + 8), B = digits bd[J][K half]
-template <int I>
+// FIRST: the first step of a sum, which starts from `init` instead of the accumulators.
+template <int I, bool FIRST>
 __device__ __forceinline__ void fx_level(float (&acc)[7][4], const FxPair& p00, const FxPair& p10,
                                          const FxPair& p01, const FxPair& p11, const uint32_t (&bd)[7][2],
-                                         const FxMask& k) {
-  const uint32_t a0 = fx_digit<I>(p00, k), a1 = fx_digit<I>(p10, k), a2 = fx_digit<I>(p01, k), a3 = fx_digit<I>(p11, k);
+                                         const FxMask& k, const float (&init)[4]) {
+  const uint32_t a0 = fx_digit<I>(p00, k), a1 = fx_digit<I>(p10, k), a2 = fx_digit<I>(p01, k),
+                 a3 = fx_digit<I>(p11, k);
 #pragma unroll
-  for (int J = 0; J + I <= 6; ++J) fx_mma(acc[I + J], a0, a1, a2, a3, bd[J][0], bd[J][1]);
+  for (int J = 0; J + I <= 6; ++J) {
+    if (FIRST && I == 0) fx_mma_first(acc[J], a0, a1, a2, a3, bd[J][0], bd[J][1], init);
+    else fx_mma(acc[I + J], a0, a1, a2, a3, bd[J][0], bd[J][1]);
+  }
 }
+template <bool FIRST>
 __device__ __forceinline__ void fx_step(float (&acc)[7][4], FxPair& p00, FxPair& p10, FxPair& p01,
-                                        FxPair& p11, const uint32_t (&bd)[7][2], const FxMask& k) {
-  fx_level<0>(acc, p00, p10, p01, p11, bd, k);
-  fx_level<1>(acc, p00, p10, p01, p11, bd, k);
-  fx_level<2>(acc, p00, p10, p01, p11, bd, k);
-  fx_level<3>(acc, p00, p10, p01, p11, bd, k);
+                                        FxPair& p11, const uint32_t (&bd)[7][2], const FxMask& k,
+                                        const float (&init)[4]) {
+  fx_level<0, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<1, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<2, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<3, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
   fx_mask_low(p00, k);
   fx_mask_low(p10, k);
   fx_mask_low(p01, k);
   fx_mask_low(p11, k);
-  fx_level<4>(acc, p00, p10, p01, p11, bd, k);
-  fx_level<5>(acc, p00, p10, p01, p11, bd, k);
-  fx_level<6>(acc, p00, p10, p01, p11, bd, k);
+  fx_level<4, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<5, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<6, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
 }
 // digits of a B fragment (K pairs q0: 2t, 2t+1 and q1: 2t+8, 2t+9 of column g)
 __device__ __forceinline__ void fx_bdigits(FxPair& q0, FxPair& q1, uint32_t (&bd)[7][2], const FxMask& k) {
@@ -208,12 +224,10 @@ __device__ __forceinline__ void fx_bdigits(FxPair& q0, FxPair& q1, uint32_t (&bd
 
 // Accumulators start at 1.5 * 2^23 while the sums stay below 2^22 (at most 32 terms), so
 // that the integer is the bit difference; otherwise at 0, converted.
-__device__ __forceinline__ void fx_clear(float (&acc)[7][4], bool small) {
+__device__ __forceinline__ void fx_init(float (&c)[4], bool small) {
   const float v = small ? __uint_as_float(FX_MAGIC) : 0.0f;
 #pragma unroll
-  for (int l = 0; l < 7; ++l)
-#pragma unroll
-    for (int o = 0; o < 4; ++o) acc[l][o] = v;
+  for (int o = 0; o < 4; ++o) c[o] = v;
 }
 // the sums as integers, in place
 __device__ __forceinline__ void fx_ints(float (&acc)[7][4], bool small) {
