@@ -26,8 +26,8 @@ int message_tc_launch(bool train, int64_t nnz, int64_t n, const int32_t* rowptr,
                       const int32_t* col, const float* ein, const float* x, float* e0out, const float* h,
                       const float* f, const __nv_bfloat16* w, int l, float* agg, float* m, float* eout, float* pe,
                       DevStatus* status, cudaStream_t st);
-int node_update_tc_launch(int64_t n, const int32_t* rowptr, float* agg, int keep_agg, const float* hin,
-                          const float* f, const __nv_bfloat16* w, int l, float* rh, float* hout, float* sdec,
+int node_update_tc_launch(int64_t n, const int32_t* rowptr, float* agg, const float* m, int keep_agg,
+                          const float* hin, const float* f, const __nv_bfloat16* w, int l, float* rh, float* hout, float* sdec,
                           float* tdec, DevStatus* status, cudaStream_t st);
 __global__ void decode_terms_kernel(int64_t, const int32_t*, const int32_t*, const float*, const float*,
                                     const float*, const __nv_bfloat16*, const double*, double*);
@@ -189,8 +189,8 @@ static size_t work_bytes(int64_t n, int64_t nnz, int nr, bool train) {
   b += (size_t)nnz * 8 + (size_t)n * 8 + (size_t)nnz * 12 + (size_t)n * 8;
   const int ne = train ? NL + 1 : 2, nm = train ? NL : 1;
   b += (size_t)ne * nnz * W * 4 + (size_t)ne * n * W * 4;
-  b += (size_t)nm * (n + 2 * ((nnz + 31) / 32)) * W * 4;
-  if (train) b += (size_t)nm * nnz * W * 4 + (size_t)nm * n * W * 4;
+  b += (size_t)nm * nnz * W * 4 + (size_t)nm * n * W * 4;
+  if (train) b += (size_t)nm * n * W * 4;
   b += (size_t)nnz * 8;
   b += (size_t)nnz * 4 + (size_t)2 * n * 4;
   if (train) {
@@ -217,11 +217,9 @@ static int work_take(Arena* ar, Work& w, int64_t n, int64_t nnz, int nr, bool tr
     w.h[l] = (float*)T(n * W * 4);
   }
   for (int l = 0; l < nm; ++l) {
-    w.agg[l] = (float*)T((n + 2 * ((nnz + 31) / 32)) * W * 4);  // row sums, then pieces of cut rows
-    if (train) {
-      w.m[l] = (float*)T(nnz * W * 4);
-      w.rh[l] = (float*)T(n * W * 4);
-    }
+    w.m[l] = (float*)T(nnz * W * 4);
+    w.agg[l] = (float*)T(n * W * 4);
+    if (train) w.rh[l] = (float*)T(n * W * 4);
   }
   w.Mval = (double*)T(nnz * 8);
   w.pe = (float*)T(nnz * 4);
@@ -250,7 +248,7 @@ static int work_take(Arena* ar, Work& w, int64_t n, int64_t nnz, int nr, bool tr
   for (int l = 0; l < ne; ++l)
     if (!w.e[l] || !w.h[l]) return RBO_ERR_NOMEM;
   for (int l = 0; l < nm; ++l)
-    if (!w.agg[l] || (train && (!w.m[l] || !w.rh[l]))) return RBO_ERR_NOMEM;
+    if (!w.m[l] || !w.agg[l] || (train && !w.rh[l])) return RBO_ERR_NOMEM;
   return RBO_OK;
 }
 
@@ -275,7 +273,7 @@ static int forward(rbo_gnn_s* g, const rbo_csr* A, Work& w, Arena* ar, cudaStrea
   for (int l = 0; l < NL; ++l) {
     const int a = train ? l : (l & 1), b = train ? l + 1 : ((l + 1) & 1);
     const bool last = l == NL - 1;
-    float* mm = train ? w.m[l] : nullptr;
+    float* mm = train ? w.m[l] : w.m[0];
     float* ag = train ? w.agg[l] : w.agg[0];
     float* rr = train ? w.rh[l] : nullptr;
     float* eo = (train || !last) ? w.e[b] : nullptr;
@@ -284,7 +282,7 @@ static int forward(rbo_gnn_s* g, const rbo_csr* A, Work& w, Arena* ar, cudaStrea
                                (l == 0 && train) ? w.e[0] : nullptr, w.h[a], w.f, g->wbf, l, ag, mm, eo,
                                last ? w.pe : nullptr, ar->status, st);
     if (rc == RBO_OK)
-      rc = node_update_tc_launch(n, A->rowptr, ag, train ? 1 : 0, (l == 0 && !train) ? nullptr : w.h[a], w.f,
+      rc = node_update_tc_launch(n, A->rowptr, ag, mm, train ? 1 : 0, (l == 0 && !train) ? nullptr : w.h[a], w.f,
                                  g->wbf, l, rr, ho, last ? w.sdec : nullptr, last ? w.tdec : nullptr, ar->status,
                                  st);
     if (rc != RBO_OK) return rc;

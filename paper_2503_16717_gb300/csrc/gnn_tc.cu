@@ -248,8 +248,8 @@ struct MsgArgs {
   int l;                     // layer
   const int32_t* rowptr;     // row starts
   const int32_t* erow;       // row i of edge q
-  float* agg;                // row sums of m (n rows of 32), then 2 rows of pieces per 32 edges
-  float* m;                  // m_l per edge, or null
+  float* agg;                // row sums of m (n rows of 32; of cut rows, their first part)
+  float* m;                  // m_l per edge (without TRAIN: of the edges behind a cut alone)
   float* eout;               // e_{l+1} = e_l + m_l per edge, or null
   float* pe;                 // decoder edge term wo[0:32] . e_{l+1} per edge, or null
   DevStatus* status;
@@ -257,11 +257,11 @@ struct MsgArgs {
 
 // message layer l over all edges (see the file header); edge q = (row i, col[q] = j).
 // The row sums are formed here: a warp owns 32 consecutive edges, 32 w .. 32 w + 31, and adds
-// the messages of each row in order.  A row i whose edges all belong to the warp goes to
-// agg[i]; the piece of a row that began before the warp's edges goes to agg[n + 2 w], the
-// piece of a row that begins among them and goes on behind them to agg[n + 2 w + 1]; the
-// node update adds the pieces in order.  m itself (128 bytes an edge written here and read
-// back there) is only stored for the backward.
+// the messages of each row in order into agg[i].  Where a row goes on past its warp's edges,
+// agg[i] is the sum of its first part and the messages behind the cut are stored one by one:
+// the node update adds them in order, so that every sum runs over its row's edges from the
+// first to the last wherever the cuts fall.  Other messages (128 bytes an edge written here
+// and read back there) are only stored for the backward.
 // ENC: e_0 from the edge features and, in inference, h_0 from the node features (first
 // layer); PE: the decoder's edge term (last layer); TRAIN: every activation is stored,
 // otherwise only e_{l+1} of the layers before the last
@@ -315,18 +315,13 @@ __global__ void __launch_bounds__(TNT, TCTAS) message_tc_kernel(const __grid_con
         cj = 0;
       }
     }
-    // rows of the warp's edges: where this lane's edge ends a row's piece, the row of agg it
-    // goes to
+    // rows of the warp's edges: `ends` marks the last edge of each, `tail` the edges of a row
+    // that began before the warp's first edge
     const int rn = __shfl_down_sync(0xffffffffu, ri, 1);
-    const bool end = lane < nv && (lane + 1 == nv || rn != ri);
-    const unsigned ends = __ballot_sync(0xffffffffu, end);
-    uint32_t slot = (uint32_t)ri;
-    if (end) {
-      const bool first = (ends & ((1u << lane) - 1u)) == 0u;
-      const int rs = P.rowptr[ri], re = P.rowptr[ri + 1];
-      if (first && (int64_t)rs < e0) slot = (uint32_t)P.n + 2u * (uint32_t)(e0 >> 5);
-      else if ((int64_t)re > e0 + nv) slot = (uint32_t)P.n + 2u * (uint32_t)(e0 >> 5) + 1u;
-    }
+    const unsigned ends = __ballot_sync(0xffffffffu, lane < nv && (lane + 1 == nv || rn != ri));
+    const int r0 = __shfl_sync(0xffffffffu, ri, 0);
+    const unsigned tail = r0 >= 0 && (int64_t)P.rowptr[r0] < e0 ? (ends ^ (ends - 1u)) : 0u;
+    const unsigned outs = ends & ~tail;
     float ev[32], hv[32];
     if constexpr (!ENC) {
       const float* el = P.ein + e0 * W + lane;
@@ -402,13 +397,12 @@ __global__ void __launch_bounds__(TNT, TCTAS) message_tc_kernel(const __grid_con
     float* mo = P.m + e0 * W + lane;
     auto store = [&](int j) {
       const float mv = relu_tc(buf[j * TLD + 32 + lane] + bias);
-      if constexpr (TRAIN) mo[j * W] = mv;
+      if (TRAIN || ((tail >> j) & 1u)) mo[j * W] = mv;
       if constexpr (TRAIN || !PE) eo[j * W] = (ENC ? buf[j * TLD + lane] : ev[j]) + mv;
       run += mv;
-      const uint32_t sj = __shfl_sync(0xffffffffu, slot, j);
-      const bool ej = (ends >> j) & 1u;
-      if (ej) aggl[(int64_t)sj * W] = run;
-      run = ej ? 0.f : run;
+      const int64_t sj = __shfl_sync(0xffffffffu, ri, j);
+      if ((outs >> j) & 1u) aggl[sj * W] = run;
+      run = (ends >> j) & 1u ? 0.f : run;
     };
     if (full) {
 #pragma unroll
@@ -424,13 +418,14 @@ __global__ void __launch_bounds__(TNT, TCTAS) message_tc_kernel(const __grid_con
 }
 
 // node update of layer l over all nodes (see the file header); agg holds the row sums as the
-// message layer left them, rows in pieces are completed here (and stored in agg
-// with keep_agg, for the backward).  hin null: h_0 from the node features f.  rh and hout may be null (inference keeps only
-// what the next layer reads); sdec and tdec, when non-null, receive the decoder's node terms wo[32:64] . h' and
-// wo[64:96] . h' (the last layer)
+// message layer left them; cut rows are completed here with the messages m behind the cut
+// (and stored in agg with keep_agg, for the backward).  hin null: h_0 from the node features
+// f.  rh and hout may be null (inference keeps only what the next layer reads); sdec and tdec,
+// when non-null, receive the decoder's node terms wo[32:64] . h' and wo[64:96] . h' (the last
+// layer)
 __global__ void __launch_bounds__(TNT, TCTAS)
     node_update_tc_kernel(int64_t n, const int32_t* __restrict__ rowptr, float* __restrict__ agg,
-                          int keep_agg, const float* __restrict__ hin, const float* __restrict__ f,
+                          const float* __restrict__ m, int keep_agg, const float* __restrict__ hin, const float* __restrict__ f,
                           const __nv_bfloat16* __restrict__ w, int l,
                           float* __restrict__ rh, float* __restrict__ hout,
                           float* __restrict__ sdec, float* __restrict__ tdec, DevStatus* status) {
@@ -459,30 +454,26 @@ __global__ void __launch_bounds__(TNT, TCTAS)
   __syncthreads();
   const float wn0 = __bfloat162float(w[OFF_WN + 2 * lane]), wn1 = __bfloat162float(w[OFF_WN + 2 * lane + 1]),
               bn = __bfloat162float(w[OFF_BN + lane]);
-  const float* bpart = agg + n * W;  // pieces of rows cut by a warp's edge range
   const int64_t ntiles = (n + TT - 1) / TT;
   int it = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
     const int64_t i0 = tile * TT + warp * 32;
-    // this lane's node: its first and last edge warps (w0 < 0: no edges)
-    int w0 = -1, w1 = -1;
+    // this lane's node: the edges behind the cut after its first edge's warp, if any
+    int te = 0, tn = 0;
+    bool any = false;
     if (i0 + lane < n) {
       const int rs = rowptr[i0 + lane], re = rowptr[i0 + lane + 1];
-      if (re > rs) {
-        w0 = rs >> 5;
-        w1 = (re - 1) >> 5;
-      }
+      any = re > rs;
+      te = (rs | 31) + 1;
+      tn = any ? max(re - te, 0) : 0;
     }
-    const unsigned pieces = __ballot_sync(0xffffffffu, w1 > w0);
+    const unsigned some = __ballot_sync(0xffffffffu, any), cut = __ballot_sync(0xffffffffu, tn > 0);
     {
       float hv[32], av[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        const int a = __shfl_sync(0xffffffffu, w0, j);
-        const bool cut = (pieces >> j) & 1u;
-        const float* p = cut ? bpart + ((int64_t)a * 2 + 1) * W + lane : agg + (i0 + j) * W + lane;
         if (hin) hv[j] = i0 + j < n ? hin[(i0 + j) * W + lane] : 0.f;
-        av[j] = a >= 0 ? *p : 0.f;
+        av[j] = (some >> j) & 1u ? agg[(i0 + j) * W + lane] : 0.f;
       }
       if (!hin) {  // first layer of inference: h_0 from the node features
         const float2 fj = i0 + lane < n ? *reinterpret_cast<const float2*>(f + 2 * (i0 + lane)) : make_float2(0.f, 0.f);
@@ -499,19 +490,39 @@ __global__ void __launch_bounds__(TNT, TCTAS)
         buf[j * TLD + 32 + lane] = av[j];
       }
     }
-    // the rows in pieces: the remaining pieces in order
-    for (unsigned p = pieces; p != 0u; p &= p - 1u) {
-      const int j = __ffs((int)p) - 1;
-      const int a = __shfl_sync(0xffffffffu, w0, j), e = __shfl_sync(0xffffffffu, w1, j);
-      float s = buf[j * TLD + 32 + lane];
-      for (int k = a + 1; k <= e; ++k) s += bpart[(int64_t)k * 2 * W + lane];
-      buf[j * TLD + 32 + lane] = s;
-      if (keep_agg) agg[(i0 + j) * W + lane] = s;
+    // the messages behind the cuts, in order, 16 loads in flight: the k-th belongs to the node
+    // whose count range holds k
+    if (cut) {
+      int upto = tn;  // counts up to and including this lane's node
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += u;
+      }
+      const int total = __shfl_sync(0xffffffffu, upto, 31);
+      for (int k0 = 0; k0 < total; k0 += 16) {
+        int node = 0;  // lane k: node of message k0 + k
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if (__shfl_sync(0xffffffffu, upto, node + o - 1) <= k0 + lane) node += o;
+        const int edge = __shfl_sync(0xffffffffu, te - (upto - tn), node) + k0 + lane;
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const int64_t q = __shfl_sync(0xffffffffu, edge, u);
+          v[u] = k0 + u < total ? m[q * W + lane] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const int j = __shfl_sync(0xffffffffu, node, u);
+          if (k0 + u < total) buf[j * TLD + 32 + lane] += v[u];
+        }
+      }
     }
-    if (keep_agg) {  // nodes without edges
+    if (keep_agg) {  // cut rows, and nodes without edges
 #pragma unroll 8
       for (int j = 0; j < 32; ++j)
-        if (i0 + j < n && __shfl_sync(0xffffffffu, w0, j) < 0) agg[(i0 + j) * W + lane] = 0.f;
+        if (i0 + j < n && (((cut | ~some) >> j) & 1u)) agg[(i0 + j) * W + lane] = buf[j * TLD + 32 + lane];
     }
     __syncwarp();
     if (!tile_products(buf, tbase, tlane, Bs, &s_mma, it)) {
@@ -842,11 +853,11 @@ int message_tc_launch(bool train, int64_t nnz, int64_t n, const int32_t* rowptr,
   return note_cuda(cudaGetLastError());
 }
 
-int node_update_tc_launch(int64_t n, const int32_t* rowptr, float* agg, int keep_agg, const float* hin,
+int node_update_tc_launch(int64_t n, const int32_t* rowptr, float* agg, const float* m, int keep_agg, const float* hin,
                           const float* f, const __nv_bfloat16* w, int l, float* rh, float* hout, float* sdec,
                           float* tdec, DevStatus* status, cudaStream_t st) {
   if (n <= 0) return RBO_OK;
-  node_update_tc_kernel<<<tc_grid(n), TNT, TSMEM, st>>>(n, rowptr, agg, keep_agg, hin, f, w, l, rh, hout,
+  node_update_tc_kernel<<<tc_grid(n), TNT, TSMEM, st>>>(n, rowptr, agg, m, keep_agg, hin, f, w, l, rh, hout,
                                                         sdec, tdec, status);
   return note_cuda(cudaGetLastError());
 }
