@@ -40,7 +40,7 @@ struct PassDev {
   int rec_off;            // sketch schedule record of the tile, offset inside a stage
   int kc, off_acc, off_ec;   // tensor-core pass: Gram chunk rows, item sums, C column scales
   int xblk, yblk;            // bytes of a 16-row block of X and of Y
-  int off_skf, c_digits, inv_digits;  // sketch tile values; whether C / the inverse is held as digits
+  int off_skf, c_digits;  // sketch tile values; whether C is held as digits
   int off_ys, ystage_bytes;  // sketch kernel: ring of Y stages (Y columns + record)
 };
 

@@ -125,20 +125,28 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     blk_start[k + 1] = blk_start[k] + (need + 15) / 16;
   }
   const int q = blk_start[nblk];
-  // Tile height and chunk: at least four items per tile for the four warps, chunks of 32
-  // rows where that takes them (their sums need no conversion), 64 otherwise; passes
-  // without a Gram take tiles of about 20 KB; sketch passes those of the schedule
+  // Tile height and chunk.  Four items a tile keep the four warps busy in one turn, and long
+  // chunks spare scans, conversions and joins of the sums (2^22 x 61, chunks of 32 -> 64 rows
+  // at q = 3: 484 -> 470 us; more turns of shorter chunks, q = 1 in 64-row tiles: 494 us); a
+  // chunk of 32 needs no conversion of its sums.  Solve + general Gram (XL: no second X stage)
+  // takes the tallest tiles: 128-row chunks there, 674 -> 572 us (their sums stay below
+  // 7 * 128 * 2^14 < 2^24).  Passes without a Gram take tiles of about 20 KB; sketch passes
+  // those of the schedule.
   int T = 64, kc = 64;
+  const bool narrow_gram = ax > 0 && b <= 8 && !rp.C;
   if (d > 0) {
     T = rp.sk.T;
   } else if (q == 0) {
     const int blk = tc_blk_bytes(a, rp.C ? 16 : 8) + tc_blk_bytes(b, 8);
     while (T < 256 && blk * (2 * T / 16) <= 20 * 1024) T *= 2;
+  } else if (narrow_gram && rp.Tri) {
+    T = q == 1 ? 256 : 128;
+    kc = q <= 2 ? 64 : 128;
   } else if (q == 1) {
     const bool narrow = a + b <= 16, upd = rp.C && ax == 0;  // (update + sym8: more CTAs)
     T = upd ? 64 : (narrow ? 256 : 128);
     kc = narrow ? 64 : 32;
-  } else if (q <= 3) {
+  } else if (q <= (narrow_gram ? 2 : 3)) {
     kc = 32;
   }
   // few rows: shorter tiles while they leave SMs without one
@@ -146,19 +154,23 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     T /= 2;
     kc = std::max(16, kc / 2);
   }
-  const bool hc = rp.C != nullptr, ht = rp.Tri != nullptr;
-  const TcKernel kern = q == 0 ? tc_kernel_g0(hc, ht, d > 0)
-                               : (ax == 0 && b <= 8 ? tc_kernel_g2(hc, ht) : tc_kernel_g1(hc, ht));
+  const bool hc = rp.C != nullptr;
+  auto kernel_of = [&](int tri) {
+    return q == 0 ? tc_kernel_g0(hc, tri, d > 0) : (ax == 0 && b <= 8 ? tc_kernel_g2(hc, tri) : tc_kernel_g1(hc, tri));
+  };
+  bool want_inv = rp.Tri && rp.Inv && !rp.C && b > 8;
+  TcKernel kern = kernel_of(want_inv ? 2 : (rp.Tri ? 1 : 0));
   if (!kern) return RBO_ERR_ARG;
   const int limit = tc_smem_limit((const void*)kern);
   const size_t epi_bytes = ((size_t)L + 2) * 8 + epilogue_doubles(rp) * 8;
   TcLayout l;
   size_t smem = 0;
   // Panels of more than 8 columns multiply by the inverse on the tensor cores where the
-  // caller vouches for the factor (2^22 rows, b = 30: 3717 -> see DESIGN us of substitution on
-  // the float64 pipe); narrow ones substitute
-  const bool xs = rp.C != nullptr && (q == 0 || (ax == 0 && b <= 8));  // as the kernels' XS
-  const bool want_inv = rp.Tri && rp.Inv && !rp.C && b > 8;
+  // caller vouches for the factor (2^22 rows, b = 30, alone: 3717 us of substitution on the
+  // float64 pipe, 1059 us); narrow ones substitute (2^22 x 61, b = 5, with the Gram: 674 us
+  // against 897 by the inverse)
+  const bool gen = q > 0 && !(ax == 0 && b <= 8);  // general Gram
+  const bool xs = rp.C ? !gen : (rp.Tri && gen);   // as the kernels' XS
   bool digits = rp.C != nullptr || want_inv;
   for (;;) {
     kc = (ax == 0 && b <= 8) ? std::max(16, T / 4) : std::min(kc, T);  // sym8: the warps' own rows
@@ -167,8 +179,13 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     smem = std::max(l.bytes, epi_bytes) + 1024;  // + alignment slack of the base
     if ((long long)smem <= limit) break;
     if (T > 16 && d == 0) T /= 2;
-    else if (digits) digits = false;  // C stays float64
-    else return RBO_ERR_ARG;
+    else if (digits) {  // C stays float64, a factor is substituted
+      digits = false;
+      if (want_inv) {
+        want_inv = false;
+        kern = kernel_of(1);
+      }
+    } else return RBO_ERR_ARG;
   }
   const int ntiles = (int)((rp.n + T - 1) / T);
   int occ = 0;
@@ -215,7 +232,6 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   P.off_sk = (int)l.off_sk;
   P.off_skf = (int)l.off_skf;
   P.c_digits = rp.C && digits ? 1 : 0;
-  P.inv_digits = want_inv && digits ? 1 : 0;
   P.off_red = 0;
   if (L > 0) {
     const size_t need = ((size_t)G * L + (size_t)ngroups * L) * 8;

@@ -47,16 +47,28 @@ struct TcDev {
   PassDev P;
 };
 
-// HC: projection (C digits); HT: triangular solve; G: Gram, 0 none, 1 general, 2 of at most
+// CTAs per SM the registers are bounded for: the substitution alone waits for the float64 pipe
+// and wants warps (2^22 rows, b = 5: 153 us at 4, 138 at 8 with spills, 135 at 6); with the
+// Gram of 8 columns 5 (251 -> 246 us); everything else needs its 128 registers.
+constexpr int tc_min_ctas(bool hc, int tri, int g) {
+  return tri == 1 && !hc ? (g == 0 ? 6 : (g == 2 ? 5 : 4)) : 4;
+}
+
+// HC: projection (C digits); TRI: triangular factor, 0 none, 1 substitution, 2 product with its
+// inverse (digits); G: Gram, 0 none, 1 general, 2 of at most
 // 8 columns of Y' alone; SK: sparse sketch (no triangle, no Gram).  Each kind of pass is its
 // own kernel: fewer live registers and less code than one kernel with all phases.
-template <bool HC, bool HT, int G, bool SK>
-__global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_constant__ TcDev D) {
+template <bool HC, int TRI, int G, bool SK>
+__global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_kernel(const __grid_constant__ TcDev D) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // X is read by the update alone when the pass has no general Gram: one X stage then, its
   // next tile copied in once every warp has updated its rows (Y keeps two stages), which
-  // leaves room for four CTAs per SM
-  constexpr bool XS = HC && G != 1;
+  // leaves room for four CTAs per SM.  With a triangle and a general Gram (XL) X is read by
+  // the Gram alone and comes in while the panel's rows are solved: one stage again, and tiles
+  // of 128 rows in the same shared memory, whose four warps each have 32 rows to solve (64
+  // rows: two warps idle, 2^22 x 61: 742 -> 674 us; b = 30 with the inverse 2683 -> 2393 us).
+  constexpr bool HT = TRI != 0, inv = TRI == 2;
+  constexpr bool XL = HT && !HC && G == 1, XS = (HC && G != 1) || XL;
   __shared__ __align__(8) uint64_t bars[NST], barx;
   __shared__ int s_flag;
   __shared__ int s_last;
@@ -104,7 +116,8 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
   };
   auto issue_x = [&](int tile) {  // XS: the tile's X alone
     mbar_arrive_expect_tx(&barx, (uint32_t)(T * 8) * (uint32_t)a);
-    for (int k = 0; k < nblk16; ++k) tma_load_rows(smem + k * xblk, &D.tmX, tile * T + 16 * k, &barx);
+    if (a > 0)
+      for (int k = 0; k < nblk16; ++k) tma_load_rows(smem + k * xblk, &D.tmX, tile * T + 16 * k, &barx);
   };
 
   // the first tile is in flight while the small matrices are prepared
@@ -124,7 +137,6 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
       *reinterpret_cast<uint4*>(p + 16 * (u & 7)) = make_uint4(0u, 0u, 0u, 0u);
     }
   }
-  const bool inv = HT && !HC && P.inv_digits;  // y' = y Inv as digit products (wide panels)
   if (HT && !inv) {
     const int ldt = rp.ldtri > 0 ? rp.ldtri : b;
     for (int t = tid; t < b * b; t += TC_NT) {
@@ -178,18 +190,19 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
     unsigned char* ys = stage_Y(s);
     if (P.use_bulk) {
       bool ok = mbar_wait_bounded(&bars[s], phase[s]);
-      if (XS) ok = mbar_wait_bounded(&barx, phx) && ok;
+      if (XS && !XL) ok = mbar_wait_bounded(&barx, phx) && ok;
       if (__syncthreads_or(!ok)) {
         if (tid == 0) set_error(P.status, RBO_ERR_TIMEOUT, 1);
         return;
       }
       phase[s] ^= 1u;
-      phx ^= 1u;
+      if (!XL) phx ^= 1u;
       // prefetch the next tile into the other stage (its readers passed the barrier)
       const int nxt = tile + gridDim.x;
-      if (tid == 0 && nxt < P.ntiles) {
+      if (tid == 0) {
         fence_proxy_async();
-        issue_tile(nxt, s ^ 1);
+        if (XL && it > 0) issue_x(tile);
+        if (nxt < P.ntiles) issue_tile(nxt, s ^ 1);
       }
     } else {
       __syncthreads();  // the previous tile's readers are done
@@ -212,7 +225,7 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
     // order, as an unblocked row-by-row substitution would.
     bool synced = false;  // the last step ended with a block barrier
     auto tri_solve = [&]() {
-      if (inv) {
+      if constexpr (inv) {
         for (int k = rw >> 4; k < re >> 4; ++k) tc_trmul_rows(ys + k * yblk, b, cf, ec, bad_c, rp.Inv);
         __syncwarp();
         return;
@@ -360,7 +373,15 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
     // ---- B: Z += [x, y']^T y' ------------------------------------------------------
     if constexpr (G != 0) {
       // the chunks of sym8 items are the warps' own rows; general items read other warps'
-      if (G == 1 && (HC || HT) && !synced) __syncthreads();
+      if (XL && P.use_bulk) {
+        if (__syncthreads_or(!mbar_wait_bounded(&barx, phx))) {
+          if (tid == 0) set_error(P.status, RBO_ERR_TIMEOUT, 1);
+          return;
+        }
+        phx ^= 1u;
+      } else if (G == 1 && (HC || HT) && !synced) {
+        __syncthreads();
+      }
       const TcTile xt{xs, xblk}, yt{ys, yblk};
       for (int item = warp; item < P.items; item += TC_NW) {
         if constexpr (G == 2) {
@@ -402,8 +423,8 @@ __global__ void __launch_bounds__(TC_NT, 4) rowpass_tc_kernel(const __grid_const
 
 // The kernel of a kind of pass; null for a combination no pass uses
 typedef void (*TcKernel)(TcDev);
-TcKernel tc_kernel_g0(bool hc, bool ht, bool sk);  // no Gram   (rowpass_tc_g0.cu)
-TcKernel tc_kernel_g1(bool hc, bool ht);           // general   (rowpass_tc_g1.cu)
-TcKernel tc_kernel_g2(bool hc, bool ht);           // Y'^T Y', at most 8 columns (rowpass_tc_g2.cu)
+TcKernel tc_kernel_g0(bool hc, int tri, bool sk);  // no Gram   (rowpass_tc_g0.cu)
+TcKernel tc_kernel_g1(bool hc, int tri);            // general   (rowpass_tc_g1.cu)
+TcKernel tc_kernel_g2(bool hc, int tri);            // Y'^T Y', at most 8 columns (rowpass_tc_g2.cu)
 
 }  // namespace rbo

@@ -2,9 +2,10 @@
 #include "rowpass_tc.cuh"
 
 namespace rbo {
-TcKernel tc_kernel_g0(bool hc, bool ht, bool sk) {
-  if (sk) return ht ? nullptr : (hc ? rowpass_tc_kernel<true, false, 0, true> : rowpass_tc_kernel<false, false, 0, true>);
-  if (ht) return hc ? rowpass_tc_kernel<true, true, 0, false> : rowpass_tc_kernel<false, true, 0, false>;
-  return hc ? rowpass_tc_kernel<true, false, 0, false> : rowpass_tc_kernel<false, false, 0, false>;
+TcKernel tc_kernel_g0(bool hc, int tri, bool sk) {
+  if (sk) return tri ? nullptr : (hc ? rowpass_tc_kernel<true, 0, 0, true> : rowpass_tc_kernel<false, 0, 0, true>);
+  if (hc) return tri ? rowpass_tc_kernel<true, 1, 0, false> : rowpass_tc_kernel<true, 0, 0, false>;
+  if (tri) return tri == 2 ? rowpass_tc_kernel<false, 2, 0, false> : rowpass_tc_kernel<false, 1, 0, false>;
+  return rowpass_tc_kernel<false, 0, 0, false>;
 }
 }  // namespace rbo

@@ -2,8 +2,9 @@
 #include "rowpass_tc.cuh"
 
 namespace rbo {
-TcKernel tc_kernel_g1(bool hc, bool ht) {
-  if (ht) return hc ? rowpass_tc_kernel<true, true, 1, false> : rowpass_tc_kernel<false, true, 1, false>;
-  return hc ? rowpass_tc_kernel<true, false, 1, false> : rowpass_tc_kernel<false, false, 1, false>;
+TcKernel tc_kernel_g1(bool hc, int tri) {
+  if (hc) return tri ? rowpass_tc_kernel<true, 1, 1, false> : rowpass_tc_kernel<true, 0, 1, false>;
+  if (tri) return tri == 2 ? rowpass_tc_kernel<false, 2, 1, false> : rowpass_tc_kernel<false, 1, 1, false>;
+  return rowpass_tc_kernel<false, 0, 1, false>;
 }
 }  // namespace rbo

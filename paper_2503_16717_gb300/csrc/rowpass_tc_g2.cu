@@ -2,8 +2,9 @@
 #include "rowpass_tc.cuh"
 
 namespace rbo {
-TcKernel tc_kernel_g2(bool hc, bool ht) {
-  if (ht) return hc ? rowpass_tc_kernel<true, true, 2, false> : rowpass_tc_kernel<false, true, 2, false>;
-  return hc ? rowpass_tc_kernel<true, false, 2, false> : rowpass_tc_kernel<false, false, 2, false>;
+TcKernel tc_kernel_g2(bool hc, int tri) {
+  if (hc) return tri ? rowpass_tc_kernel<true, 1, 2, false> : rowpass_tc_kernel<true, 0, 2, false>;
+  if (tri) return tri == 2 ? rowpass_tc_kernel<false, 2, 2, false> : rowpass_tc_kernel<false, 1, 2, false>;
+  return rowpass_tc_kernel<false, 0, 2, false>;
 }
 }  // namespace rbo
