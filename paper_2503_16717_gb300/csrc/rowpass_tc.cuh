@@ -15,8 +15,9 @@
 //      their signed sums per sketch row from the tile's schedule record: the thread that
 //      owns a slot of the record sums the slot's entries and adds them to the row's 64-bit
 //      integer accumulators.  A column's scale only grows (the accumulators are shifted
-//      when a tile raises it) and the accumulators enter the CTA's float64 partial every
-//      384 rows, so that a tile costs no float64 operation per sketch row;
+//      when a tile raises it) and the accumulators enter the CTA's float64 partial before a
+//      sketch row can have summed 384 entries (a few thousand rows, by the tiles' largest
+//      counts), so that a tile costs no float64 operation per sketch row;
 //   B  the Gram items, (16 Z columns) x (8 Y' columns) x (a chunk of kc rows), are dealt
 //      to the warps; an item always goes to the same warp, which keeps its float64 sums
 //      in its own shared-memory slots.
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   };
 
   // the first tile is in flight while the small matrices are prepared
-  uint32_t phase[NST] = {0u, 0u}, phx = 0u;
+  uint32_t phx = 0u;  // (a stage's phase: the parity of the tiles it held)
   const int first = blockIdx.x;
   if (tid == 0 && P.use_bulk && first < P.ntiles) {
     issue_tile(first, 0);
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   __syncthreads();
   const int bad_c = HC ? (P.c_digits ? s_bad : 1) : (inv ? s_bad : 0);
   // rows of a tile a warp owns from the update to the sums of a chunk: rpw from rw
-  const int rpw = max(16, T >> 2), rw = warp * rpw, re = min(rw + rpw, T);
+  const int rsh = max(4, tsh - 2), rpw = 1 << rsh, rw = warp * rpw, re = min(rw + rpw, T);
   double* mypart = P.L > 0 ? P.partials + (size_t)blockIdx.x * P.L : nullptr;
   const bool mixed = SK && rp.mixed;  // float32 values and sums of the sketch
   // sketch sums into the partial: mypart = / += (each thread its own entries)
@@ -178,7 +179,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
     }
     sk_first = false;
   };
-  int sk_rows = 0;  // rows summed since the last flush
+  int sk_cnt = 0;  // entries a sketch row can have summed since the last flush
   const int q = P.blk_start[P.nblk];  // Gram items per chunk
 
   int it = 0;
@@ -189,13 +190,12 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
     unsigned char* xs = stage_X(s);
     unsigned char* ys = stage_Y(s);
     if (P.use_bulk) {
-      bool ok = mbar_wait_bounded(&bars[s], phase[s]);
+      bool ok = mbar_wait_bounded(&bars[s], (uint32_t)(it >> 1) & 1u);
       if (XS && !XL) ok = mbar_wait_bounded(&barx, phx) && ok;
       if (__syncthreads_or(!ok)) {
         if (tid == 0) set_error(P.status, RBO_ERR_TIMEOUT, 1);
         return;
       }
-      phase[s] ^= 1u;
       if (!XL) phx ^= 1u;
       // prefetch the next tile into the other stage (its readers passed the barrier)
       const int nxt = tile + gridDim.x;
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       // value past a scale (or not finite) takes the block-wide path below
       bool past = false;
       for (int t = lane; t < (re - rw) * b; t += 32) {
-        const int r = rw + (t & (rpw - 1)), c = t / rpw;
+        const int r = rw + (t & (rpw - 1)), c = t >> rsh;
         const double v = tc_ld(ys + TcTile::off(yblk, r, c));
         if (mixed) {
           const float f = f64_to_f32_int(v);
@@ -322,12 +322,15 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
         issue_x(tile + gridDim.x);
       }
       if (!mixed) {
-        const bool rescale = s_rescale != 0, full = sk_rows + T > 384;  // 2^54 * 384 < 2^63
+        // the record's first slot has the tile's most entries in one sketch row
+        const uint32_t m0 = *reinterpret_cast<const uint32_t*>(stage_R(s));
+        const int most = m0 == 0xFFFFFFFFu ? 0 : (int)(m0 >> 23);
+        const bool rescale = s_rescale != 0, full = sk_cnt + most > 384;  // 2^54 * 384 < 2^63
         if (full) {
           sk_flush();
-          sk_rows = 0;
+          sk_cnt = 0;
         }
-        sk_rows += T;
+        sk_cnt += most;
         if (rescale) {
           __syncthreads();  // scales read by the flush and the conversion
           for (int c = warp; c < b; c += TC_NW) {
