@@ -116,15 +116,26 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   const int a = rp.a, b = rp.b;
   const int ax = rp.acc_x ? a : 0;
   const int zr = ax + (rp.acc_y ? b : 0), no = zr * b, L = no + d * b;
-  // Gram items of a chunk: for every 8 columns of Y', the 16-column groups of Z down to
-  // the block's diagonal
-  const int nblk = (b + 7) / 8;
-  int blk_start[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (int k = 0; k < nblk; ++k) {
-    const int need = zr == 0 ? 0 : ax + (rp.acc_y ? std::min(b, 8 * k + 8) : 0);
-    blk_start[k + 1] = blk_start[k] + (need + 15) / 16;
-  }
-  const int q = blk_start[nblk];
+  const bool hc = rp.C != nullptr;
+  // Panels of more than 8 columns multiply by the inverse on the tensor cores where the
+  // caller vouches for the factor (2^22 rows, b = 30, alone: 3717 us of substitution on the
+  // float64 pipe, 1059 us); narrow ones substitute (2^22 x 61, b = 5, with the Gram: 674 us
+  // against 897 by the inverse)
+  bool want_inv = rp.Tri && rp.Inv && !hc && b > 8;
+  // Gram items of a chunk: for every 8 columns of Y' (16 in wide kernels), the 16-column
+  // groups of Z down to the block's diagonal
+  const bool y_only = hc && !rp.Tri && ax == 0 && rp.acc_y && b > 8;
+  int nblk = 0, q = 0, blk_start[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  auto count_items = [&]() {
+    const int w = want_inv || y_only ? 16 : 8;
+    nblk = (b + w - 1) / w;
+    for (int k = 0; k < nblk; ++k) {
+      const int need = zr == 0 ? 0 : ax + (rp.acc_y ? std::min(b, w * k + w) : 0);
+      blk_start[k + 1] = blk_start[k] + (need + 15) / 16;
+    }
+    q = blk_start[nblk];
+  };
+  count_items();
   // Tile height and chunk.  Four items a tile keep the four warps busy in one turn, and long
   // chunks spare scans, conversions and joins of the sums (2^22 x 61, chunks of 32 -> 64 rows
   // at q = 3: 484 -> 470 us; more turns of shorter chunks, q = 1 in 64-row tiles: 494 us); a
@@ -139,6 +150,9 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   } else if (q == 0) {
     const int blk = tc_blk_bytes(a, rp.C ? 16 : 8) + tc_blk_bytes(b, 8);
     while (T < 256 && blk * (2 * T / 16) <= 20 * 1024) T *= 2;
+  } else if (want_inv || y_only) {
+    T = q == 1 ? 128 : 64;
+    kc = q <= 2 ? 32 : 64;
   } else if (narrow_gram && rp.Tri) {
     T = q == 1 ? 256 : 128;
     kc = q <= 2 ? 64 : 128;
@@ -154,27 +168,22 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     T /= 2;
     kc = std::max(16, kc / 2);
   }
-  const bool hc = rp.C != nullptr;
   auto kernel_of = [&](int tri) {
+    if (y_only) return tc_kernel_g3();
     return q == 0 ? tc_kernel_g0(hc, tri, d > 0) : (ax == 0 && b <= 8 ? tc_kernel_g2(hc, tri) : tc_kernel_g1(hc, tri));
   };
-  bool want_inv = rp.Tri && rp.Inv && !rp.C && b > 8;
   TcKernel kern = kernel_of(want_inv ? 2 : (rp.Tri ? 1 : 0));
   if (!kern) return RBO_ERR_ARG;
   const int limit = tc_smem_limit((const void*)kern);
   const size_t epi_bytes = ((size_t)L + 2) * 8 + epilogue_doubles(rp) * 8;
   TcLayout l;
   size_t smem = 0;
-  // Panels of more than 8 columns multiply by the inverse on the tensor cores where the
-  // caller vouches for the factor (2^22 rows, b = 30, alone: 3717 us of substitution on the
-  // float64 pipe, 1059 us); narrow ones substitute (2^22 x 61, b = 5, with the Gram: 674 us
-  // against 897 by the inverse)
-  const bool gen = q > 0 && !(ax == 0 && b <= 8);  // general Gram
+  const bool gen = q > 0 && !(ax == 0 && b <= 8) && !y_only;  // general Gram
   const bool xs = rp.C ? !gen : (rp.Tri && gen);   // as the kernels' XS
   bool digits = rp.C != nullptr || want_inv;
   for (;;) {
     kc = (ax == 0 && b <= 8) ? std::max(16, T / 4) : std::min(kc, T);  // sym8: the warps' own rows
-    l = tc_layout(a, b, T, q * (T / kc), rp.C != nullptr, digits, rp.Tri != nullptr, want_inv && digits, d,
+    l = tc_layout(a, b, T, q * (T / kc) * (want_inv || y_only ? 2 : 1), rp.C != nullptr, digits, rp.Tri != nullptr, want_inv && digits, d,
                   d > 0 ? rp.sk.rec_bytes : 0, xs);
     smem = std::max(l.bytes, epi_bytes) + 1024;  // + alignment slack of the base
     if ((long long)smem <= limit) break;
@@ -183,6 +192,7 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
       digits = false;
       if (want_inv) {
         want_inv = false;
+        count_items();
         kern = kernel_of(1);
       }
     } else return RBO_ERR_ARG;

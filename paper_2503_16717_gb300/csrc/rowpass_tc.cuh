@@ -48,16 +48,23 @@ struct TcDev {
   PassDev P;
 };
 
+// Panels of more than 8 columns after the inverse or an update alone (wide): two column tiles
+// at a time, which share the digits of the left operand (2^22 rows, a = 31, b = 30: inverse +
+// Gram 2374 -> 1990 us, update + Gram 2675 -> 2150 us, inverse alone 1034 -> 958 us).
+__host__ __device__ constexpr bool tc_wide(int tri, int g) { return tri == 2 || g == 3; }
 // CTAs per SM the registers are bounded for: the substitution alone waits for the float64 pipe
 // and wants warps (2^22 rows, b = 5: 153 us at 4, 138 at 8 with spills, 135 at 6); with the
-// Gram of 8 columns 5 (251 -> 246 us); everything else needs its 128 registers.
+// Gram of 8 columns 5 (251 -> 246 us); with a general Gram 3, free of spills, since the shared
+// memory allows few more (solve + Gram 572 -> 549 us, update + solve + Gram 822 -> 781 us);
+// the wide ones need 168 registers; everything else 128.
 constexpr int tc_min_ctas(bool hc, int tri, int g) {
+  if (tc_wide(tri, g) || (tri == 1 && g == 1)) return 3;
   return tri == 1 && !hc ? (g == 0 ? 6 : (g == 2 ? 5 : 4)) : 4;
 }
 
 // HC: projection (C digits); TRI: triangular factor, 0 none, 1 substitution, 2 product with its
 // inverse (digits); G: Gram, 0 none, 1 general, 2 of at most
-// 8 columns of Y' alone; SK: sparse sketch (no triangle, no Gram).  Each kind of pass is its
+// 8 columns of Y' alone, 3 of more columns of Y' alone after an update; SK: sparse sketch (no triangle, no Gram).  Each kind of pass is its
 // own kernel: fewer live registers and less code than one kernel with all phases.
 template <bool HC, int TRI, int G, bool SK>
 __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_kernel(const __grid_constant__ TcDev D) {
@@ -70,6 +77,8 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   // rows: two warps idle, 2^22 x 61: 742 -> 674 us; b = 30 with the inverse 2683 -> 2393 us).
   constexpr bool HT = TRI != 0, inv = TRI == 2;
   constexpr bool XL = HT && !HC && G == 1, XS = (HC && G != 1) || XL;
+  // panels of more than 8 columns: two column tiles at a time
+  constexpr int NT = tc_wide(TRI, G) ? 2 : 1;
   __shared__ __align__(8) uint64_t bars[NST], barx;
   __shared__ int s_flag;
   __shared__ int s_last;
@@ -147,7 +156,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
     for (int t = tid; t < b; t += TC_NT) dinv[t] = 1.0 / rp.Tri[t + (size_t)t * ldt];
   }
   if constexpr (G != 0)
-    for (int t = tid; t < P.items * 128; t += TC_NT) accs[t] = 0.0;
+    for (int t = tid; t < P.items * 128 * NT; t += TC_NT) accs[t] = 0.0;
   if constexpr (SK) {
     for (int t = tid; t < d * b; t += TC_NT) ska[t] = 0;  // (all-zero bits also as float32 pairs)
     if (tid < 64) s_scale[tid] = s_shift[tid] = s_nan[tid] = 0;
@@ -263,10 +272,11 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
     if (HT && rp.tri_first) tri_solve();
     if constexpr (HC) {
       for (int k = rw >> 4; k < re >> 4; ++k)
-        tc_update_rows(xs + k * xblk, ys + k * yblk, a, b, cf, ec, bad_c, rp.C, ldc);
+        tc_update_rows<NT>(xs + k * xblk, ys + k * yblk, a, b, cf, ec, bad_c, rp.C, ldc);
       synced = false;
       if (XS && !SK) {
         __syncthreads();  // every warp is done with X (sketch passes: at their own barrier)
+        synced = true;
         if (tid == 0 && P.use_bulk && tile + (int)gridDim.x < P.ntiles) {
           fence_proxy_async();
           issue_x(tile + gridDim.x);
@@ -382,7 +392,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
           return;
         }
         phx ^= 1u;
-      } else if (G == 1 && (HC || HT) && !synced) {
+      } else if ((G == 1 || G == 3) && (HC || HT) && !synced) {
         __syncthreads();
       }
       const TcTile xt{xs, xblk}, yt{ys, yblk};
@@ -393,8 +403,8 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
           const int chunk = item / q, task = item - chunk * q;
           int nt = 0;
           while (nt + 1 < P.nblk && task >= P.blk_start[nt + 1]) ++nt;
-          tc_gram_item(xt, yt, ax, P.zr, b, task - P.blk_start[nt], nt, (chunk * P.kc) >> 4, P.kc >> 4,
-                       accs + item * 128);
+          tc_gram_item<NT>(xt, yt, ax, P.zr, b, task - P.blk_start[nt], nt * NT, (chunk * P.kc) >> 4, P.kc >> 4,
+                           accs + item * 128 * NT);
         }
       }
     }
@@ -414,11 +424,11 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       zi = ax + c;
       zc = i - ax;
     }
-    const int task = P.blk_start[zc >> 3] + (zi >> 4);
+    const int task = P.blk_start[(zc >> 3) / NT] + (zi >> 4);
     const int ri = zi & 15, ci = zc & 7;
-    const double* p = accs + (size_t)task * 128 + (2 * (ri >> 3) + (ci & 1)) * 32 + 4 * (ri & 7) + (ci >> 1);
+    const double* p = accs + (size_t)(task * NT + (zc >> 3) % NT) * 128 + (2 * (ri >> 3) + (ci & 1)) * 32 + 4 * (ri & 7) + (ci >> 1);
     double sum = 0.0;
-    for (int item = 0; item < P.items; item += q) sum += p[(size_t)item * 128];
+    for (int item = 0; item < P.items; item += q) sum += p[(size_t)item * 128 * NT];
     mypart[o] = sum;
   }
   tree_reduce_epilogue(P, smem, &s_flag, &s_last);
@@ -428,6 +438,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
 typedef void (*TcKernel)(TcDev);
 TcKernel tc_kernel_g0(bool hc, int tri, bool sk);  // no Gram   (rowpass_tc_g0.cu)
 TcKernel tc_kernel_g1(bool hc, int tri);            // general   (rowpass_tc_g1.cu)
+TcKernel tc_kernel_g3();                            // wide Y'^T Y' after an update (rowpass_tc_g1.cu)
 TcKernel tc_kernel_g2(bool hc, int tri);            // Y'^T Y', at most 8 columns (rowpass_tc_g2.cu)
 
 }  // namespace rbo

@@ -7,4 +7,5 @@ TcKernel tc_kernel_g1(bool hc, int tri) {
   if (tri) return tri == 2 ? rowpass_tc_kernel<false, 2, 1, false> : rowpass_tc_kernel<false, 1, 1, false>;
   return rowpass_tc_kernel<false, 0, 1, false>;
 }
+TcKernel tc_kernel_g3() { return rowpass_tc_kernel<true, 0, 3, false>; }
 }  // namespace rbo

@@ -181,33 +181,36 @@ __device__ __forceinline__ void fx_mma_first(float (&d)[4], uint32_t a0, uint32_
 // All pairs I + J <= 6 of one K step: A = four pairs of values, p[row half][K half] (rows
 // g / g + 8), B = digits bd[J][K half]
 // FIRST: the first step of a sum, which starts from `init` instead of the accumulators.
-template <int I, bool FIRST>
-__device__ __forceinline__ void fx_level(float (&acc)[7][4], const FxPair& p00, const FxPair& p10,
-                                         const FxPair& p01, const FxPair& p11, const uint32_t (&bd)[7][2],
+// NT column tiles of B share the digits of A, which are two thirds of a step's instructions.
+template <int I, bool FIRST, int NT>
+__device__ __forceinline__ void fx_level(float (&acc)[NT][7][4], const FxPair& p00, const FxPair& p10,
+                                         const FxPair& p01, const FxPair& p11, const uint32_t (&bd)[NT][7][2],
                                          const FxMask& k, const float (&init)[4]) {
   const uint32_t a0 = fx_digit<I>(p00, k), a1 = fx_digit<I>(p10, k), a2 = fx_digit<I>(p01, k),
                  a3 = fx_digit<I>(p11, k);
 #pragma unroll
-  for (int J = 0; J + I <= 6; ++J) {
-    if (FIRST && I == 0) fx_mma_first(acc[J], a0, a1, a2, a3, bd[J][0], bd[J][1], init);
-    else fx_mma(acc[I + J], a0, a1, a2, a3, bd[J][0], bd[J][1]);
-  }
+  for (int h = 0; h < NT; ++h)
+#pragma unroll
+    for (int J = 0; J + I <= 6; ++J) {
+      if (FIRST && I == 0) fx_mma_first(acc[h][J], a0, a1, a2, a3, bd[h][J][0], bd[h][J][1], init);
+      else fx_mma(acc[h][I + J], a0, a1, a2, a3, bd[h][J][0], bd[h][J][1]);
+    }
 }
-template <bool FIRST>
-__device__ __forceinline__ void fx_step(float (&acc)[7][4], FxPair& p00, FxPair& p10, FxPair& p01,
-                                        FxPair& p11, const uint32_t (&bd)[7][2], const FxMask& k,
+template <bool FIRST, int NT>
+__device__ __forceinline__ void fx_step(float (&acc)[NT][7][4], FxPair& p00, FxPair& p10, FxPair& p01,
+                                        FxPair& p11, const uint32_t (&bd)[NT][7][2], const FxMask& k,
                                         const float (&init)[4]) {
-  fx_level<0, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<1, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<2, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<3, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<0, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<1, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<2, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<3, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
   fx_mask_low(p00, k);
   fx_mask_low(p10, k);
   fx_mask_low(p01, k);
   fx_mask_low(p11, k);
-  fx_level<4, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<5, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<6, FIRST>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<4, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<5, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<6, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
 }
 // digits of a B fragment (K pairs q0: 2t, 2t+1 and q1: 2t+8, 2t+9 of column g)
 __device__ __forceinline__ void fx_bdigits(FxPair& q0, FxPair& q1, uint32_t (&bd)[7][2], const FxMask& k) {

@@ -47,83 +47,113 @@ __device__ __forceinline__ void tc_gram_flush(float (&acc)[7][4], bool small, in
   }
 }
 
-// acc_out (4 x 32 doubles, this warp's own) += Z(:, 16 mt ..)^T Y(:, 8 nt ..) over the nks
-// blocks of 16 rows from block b0; Z = [X (ax columns, tile xt), Y (tile yt)], zr columns
-// (the last one stands in for columns past the end, whose sums are not read).
+// acc_out (NT times 4 x 32 doubles, this warp's own) += Z(:, 16 mt ..)^T Y(:, 8 nt ..) over the
+// nks blocks of 16 rows from block b0, for the NT column tiles from nt; Z = [X (ax columns, tile
+// xt), Y (tile yt)], zr columns (the last one stands in for columns past the end, whose sums are
+// not read).
 // Lane (g, t) = (lane / 4, lane % 4) owns rows 4t..4t+3 of every block for the columns g,
 // g + 8 of Z and g of Y: the order of the rows inside a step is the same for both
 // operands, which is all a contraction needs, and makes every load 16 bytes.
 // acc_out[o * 32 + lane] belongs to Z column 16 mt + g + 8 (o / 2), Y column 8 nt + 2t + o % 2.
+template <int NT>
 static __device__ __forceinline__ void tc_gram_item(const TcTile xt, const TcTile yt, int ax, int zr, int b,
                                                     int mt, int nt, int b0, int nks, double* acc_out) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int i0 = 16 * mt;
-  const int za = min(i0 + g, zr - 1), zc = min(i0 + 8 + g, zr - 1), yc = min(8 * nt + g, b - 1);
+  const int za = min(i0 + g, zr - 1), zc = min(i0 + 8 + g, zr - 1);
   const int blk0 = za < ax ? xt.blk : yt.blk, blk1 = zc < ax ? xt.blk : yt.blk;
   const int ca = za < ax ? za : za - ax, cc = zc < ax ? zc : zc - ax;
   const unsigned char* z0 = (za < ax ? xt.base : yt.base) + b0 * blk0 + ca * 128;
   const unsigned char* z1 = (zc < ax ? xt.base : yt.base) + b0 * blk1 + cc * 128;
-  const unsigned char* y0 = yt.base + b0 * yt.blk + yc * 128;
-  const int oa = ((2 * t) ^ (ca & 7)) << 4, ob = ((2 * t) ^ (cc & 7)) << 4, oy = ((2 * t) ^ (yc & 7)) << 4;
-  FxMax m0, m1, mb;
+  const int oa = ((2 * t) ^ (ca & 7)) << 4, ob = ((2 * t) ^ (cc & 7)) << 4;
+  const unsigned char* y0[NT];
+  int oy[NT];
+#pragma unroll
+  for (int h = 0; h < NT; ++h) {
+    const int yc = min(8 * (nt + h) + g, b - 1);
+    y0[h] = yt.base + b0 * yt.blk + yc * 128;
+    oy[h] = ((2 * t) ^ (yc & 7)) << 4;
+  }
+  FxMax m0, m1, mb[NT];
   for (int ks = 0; ks < nks; ++ks) {
-    const unsigned char *pa = z0 + ks * blk0, *pc = z1 + ks * blk1, *py = y0 + ks * yt.blk;
+    const unsigned char *pa = z0 + ks * blk0, *pc = z1 + ks * blk1;
     const double2 u0 = tc_ld2(pa + oa), u1 = tc_ld2(pa + (oa ^ 16));
     const double2 w0 = tc_ld2(pc + ob), w1 = tc_ld2(pc + (ob ^ 16));
-    const double2 v0 = tc_ld2(py + oy), v1 = tc_ld2(py + (oy ^ 16));
+#pragma unroll
+    for (int h = 0; h < NT; ++h) {
+      const unsigned char* py = y0[h] + ks * yt.blk;
+      const double2 v0 = tc_ld2(py + oy[h]), v1 = tc_ld2(py + (oy[h] ^ 16));
+      mb[h].add(v0.x, v0.y);
+      mb[h].add(v1.x, v1.y);
+    }
     m0.add(u0.x, u0.y);
     m0.add(u1.x, u1.y);
     m1.add(w0.x, w0.y);
     m1.add(w1.x, w1.y);
-    mb.add(v0.x, v0.y);
-    mb.add(v1.x, v1.y);
   }
   m0.reduce4();
   m1.reduce4();
-  mb.reduce4();
-  const int E0 = m0.scale(), E1 = m1.scale(), Eb = mb.scale();
-  if (__any_sync(0xffffffffu, E0 == 0 || E1 == 0 || Eb == 0)) {
-    const int ya = min(8 * nt + 2 * t, b - 1), yb = min(8 * nt + 2 * t + 1, b - 1);
-    const unsigned char* yp = yt.base + b0 * yt.blk;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    for (int r = 0; r < 16 * nks; ++r) {
-      const double x0 = tc_ld(z0 - ca * 128 + TcTile::off(blk0, r, ca));
-      const double x1 = tc_ld(z1 - cc * 128 + TcTile::off(blk1, r, cc));
-      const double u = tc_ld(yp + TcTile::off(yt.blk, r, ya)), v = tc_ld(yp + TcTile::off(yt.blk, r, yb));
-      s0 = fma(x0, u, s0);
-      s1 = fma(x0, v, s1);
-      s2 = fma(x1, u, s2);
-      s3 = fma(x1, v, s3);
+  const int E0 = m0.scale(), E1 = m1.scale();
+  int Eb[NT];
+  bool out = E0 == 0 || E1 == 0;
+#pragma unroll
+  for (int h = 0; h < NT; ++h) {
+    mb[h].reduce4();
+    Eb[h] = mb[h].scale();
+    out = out || Eb[h] == 0;
+  }
+  if (__any_sync(0xffffffffu, out)) {
+#pragma unroll 1
+    for (int h = 0; h < NT; ++h) {
+      const int ya = min(8 * (nt + h) + 2 * t, b - 1), yb = min(8 * (nt + h) + 2 * t + 1, b - 1);
+      const unsigned char* yp = yt.base + b0 * yt.blk;
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+      for (int r = 0; r < 16 * nks; ++r) {
+        const double x0 = tc_ld(z0 - ca * 128 + TcTile::off(blk0, r, ca));
+        const double x1 = tc_ld(z1 - cc * 128 + TcTile::off(blk1, r, cc));
+        const double u = tc_ld(yp + TcTile::off(yt.blk, r, ya)), v = tc_ld(yp + TcTile::off(yt.blk, r, yb));
+        s0 = fma(x0, u, s0);
+        s1 = fma(x0, v, s1);
+        s2 = fma(x1, u, s2);
+        s3 = fma(x1, v, s3);
+      }
+      double* ao = acc_out + h * 128;
+      ao[lane] += s0;
+      ao[32 + lane] += s1;
+      ao[64 + lane] += s2;
+      ao[96 + lane] += s3;
     }
-    acc_out[lane] += s0;
-    acc_out[32 + lane] += s1;
-    acc_out[64 + lane] += s2;
-    acc_out[96 + lane] += s3;
     return;
   }
-  const FxScale k0 = fx_scale(E0), k1 = fx_scale(E1), kb = fx_scale(Eb);
+  const FxScale k0 = fx_scale(E0), k1 = fx_scale(E1);
+  FxScale kb[NT];
+#pragma unroll
+  for (int h = 0; h < NT; ++h) kb[h] = fx_scale(Eb[h]);
   const FxMask km = fx_masks();
   const bool small = nks <= 2;
-  float acc[7][4], init[4];
+  float acc[NT][7][4], init[4];
   fx_init(init, small);
   auto step = [&](int ks, auto first) {
-    const unsigned char *pa = z0 + ks * blk0, *pc = z1 + ks * blk1, *py = y0 + ks * yt.blk;
-    const double2 v0 = tc_ld2(py + oy), v1 = tc_ld2(py + (oy ^ 16));
+    const unsigned char *pa = z0 + ks * blk0, *pc = z1 + ks * blk1;
     const double2 u0 = tc_ld2(pa + oa), u1 = tc_ld2(pa + (oa ^ 16));
     const double2 w0 = tc_ld2(pc + ob), w1 = tc_ld2(pc + (ob ^ 16));
-    uint32_t bd[7][2];
-    {
-      FxPair q0 = fx_pair(v0.x, v0.y, kb, km), q1 = fx_pair(v1.x, v1.y, kb, km);
-      fx_bdigits(q0, q1, bd, km);
+    uint32_t bd[NT][7][2];
+#pragma unroll
+    for (int h = 0; h < NT; ++h) {
+      const unsigned char* py = y0[h] + ks * yt.blk;
+      const double2 v0 = tc_ld2(py + oy[h]), v1 = tc_ld2(py + (oy[h] ^ 16));
+      FxPair q0 = fx_pair(v0.x, v0.y, kb[h], km), q1 = fx_pair(v1.x, v1.y, kb[h], km);
+      fx_bdigits(q0, q1, bd[h], km);
     }
     FxPair p00 = fx_pair(u0.x, u0.y, k0, km), p01 = fx_pair(u1.x, u1.y, k0, km);
     FxPair p10 = fx_pair(w0.x, w0.y, k1, km), p11 = fx_pair(w1.x, w1.y, k1, km);
-    fx_step<decltype(first)::value>(acc, p00, p10, p01, p11, bd, km, init);
+    fx_step<decltype(first)::value, NT>(acc, p00, p10, p01, p11, bd, km, init);
   };
   step(0, FxTrue());
 #pragma unroll 1
   for (int ks = 1; ks < nks; ++ks) step(ks, FxFalse());
-  tc_gram_flush(acc, small, E0, E1, Eb, zr - i0 > 8, acc_out);
+#pragma unroll
+  for (int h = 0; h < NT; ++h) tc_gram_flush(acc[h], small, E0, E1, Eb[h], zr - i0 > 8, acc_out + h * 128);
 }
 
 // The same for Y^T Y of at most 8 columns: the A digits are the B digits, and rows 8..15 of
@@ -236,9 +266,27 @@ static __device__ void tc_build_c(const double* C, int ldc, int a, int b, uint2*
   __syncthreads();
 }
 
+// digits of the NT column tiles from n0 at K step ks (the last tile stands in for one past it)
+template <int NT>
+static __device__ __forceinline__ void tc_load_b(const uint2* cf, int n0, int NB, int KS, int ks, int lane,
+                                                 uint32_t (&bd)[NT][7][2]) {
+#pragma unroll
+  for (int h = 0; h < NT; ++h) {
+    const uint2* q = cf + ((size_t)(min(n0 + h, NB - 1) * KS + ks) * 7) * 32 + lane;
+#pragma unroll
+    for (int J = 0; J < 7; ++J) {
+      const uint2 u = q[J * 32];
+      bd[h][J][0] = u.x;
+      bd[h][J][1] = u.y;
+    }
+  }
+}
+
 // y -= x C for the 16 tile rows of one block (xb: a columns padded with zeros to a multiple
 // of 16, yb: b columns, both block bases).  A row's scale is the largest exponent of its a entries.  Lane (g, t) owns rows
 // g and g + 8, columns 2t, 2t+1, 2t+8, 2t+9 of every 16-column step.
+// NT column tiles at a time share the digits of x.
+template <int NT>
 static __device__ __forceinline__ void tc_update_rows(const unsigned char* xb, unsigned char* yb, int a, int b,
                                                    const uint2* cf, const int* ec, int bad, const double* C,
                                                    int ldc) {
@@ -269,8 +317,8 @@ static __device__ __forceinline__ void tc_update_rows(const unsigned char* xb, u
   const FxScale k0 = fx_scale(E0), k1 = fx_scale(E1);
   const FxMask km = fx_masks();
   const bool small = KS <= 2;
-  for (int nt = 0; nt < NB; ++nt) {
-    float acc[7][4], init[4];
+  for (int n0 = 0; n0 < NB; n0 += NT) {
+    float acc[NT][7][4], init[4];
     fx_init(init, small);
     auto step = [&](int ks, auto first) {
       const unsigned char* p = xb + ks * 2048;
@@ -278,35 +326,35 @@ static __device__ __forceinline__ void tc_update_rows(const unsigned char* xb, u
       FxPair p10 = fx_pair(tc_ld(p + (o0 ^ 64)), tc_ld(p + (o1 ^ 64)), k1, km);
       FxPair p01 = fx_pair(tc_ld(p + 1024 + o0), tc_ld(p + 1024 + o1), k0, km);
       FxPair p11 = fx_pair(tc_ld(p + 1024 + (o0 ^ 64)), tc_ld(p + 1024 + (o1 ^ 64)), k1, km);
-      uint32_t bd[7][2];
-#pragma unroll
-      for (int J = 0; J < 7; ++J) {
-        const uint2 u = cf[((size_t)(nt * KS + ks) * 7 + J) * 32 + lane];
-        bd[J][0] = u.x;
-        bd[J][1] = u.y;
-      }
-      fx_step<decltype(first)::value>(acc, p00, p10, p01, p11, bd, km, init);
+      uint32_t bd[NT][7][2];
+      tc_load_b<NT>(cf, n0, NB, KS, ks, lane, bd);
+      fx_step<decltype(first)::value, NT>(acc, p00, p10, p01, p11, bd, km, init);
     };
     step(0, FxTrue());
 #pragma unroll 1
     for (int ks = 1; ks < KS; ++ks) step(ks, FxFalse());
-    fx_ints(acc, small);
-    unsigned char* yt = yb + nt * 1024;
 #pragma unroll
-    for (int o = 0; o < 4; ++o) {
-      const int c = 8 * nt + 2 * t + (o & 1);
-      const double v = fx_join(acc, o);
-      if (c < b) {
-        double* yp = reinterpret_cast<double*>(yt + (((o & 1) ? o1 : o0) ^ ((o >> 1) * 64)));
-        *yp = fma(-v, fx_weight(o >> 1 ? E1 : E0, ec[c]), *yp);
+    for (int h = 0; h < NT; ++h) {
+      const int nt = n0 + h;
+      if (nt >= NB) break;
+      fx_ints(acc[h], small);
+      unsigned char* yt = yb + nt * 1024;
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        const int c = 8 * nt + 2 * t + (o & 1);
+        const double v = fx_join(acc[h], o);
+        if (c < b) {
+          double* yp = reinterpret_cast<double*>(yt + (((o & 1) ? o1 : o0) ^ ((o >> 1) * 64)));
+          *yp = fma(-v, fx_weight(o >> 1 ? E1 : E0, ec[c]), *yp);
+        }
       }
     }
   }
 }
 
 // y = y Inv for the 16 tile rows of one block (yb: b columns padded with zeros to a multiple
-// of 16), Inv upper triangular as B fragments (tc_build_c).  Column tiles are finished from
-// the right: tile nt reads columns up to 8 nt + 7 only.
+// of 16), Inv upper triangular as B fragments (tc_build_c).  Pairs of column tiles are finished
+// from the right: tiles nt, nt + 1 (nt even) read columns up to 8 nt + 15 only.
 static __device__ __forceinline__ void tc_trmul_rows(unsigned char* yb, int b, const uint2* cf, const int* ec, int bad,
                                                      const double* Inv) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -333,10 +381,10 @@ static __device__ __forceinline__ void tc_trmul_rows(unsigned char* yb, int b, c
   }
   const FxScale k0 = fx_scale(E0), k1 = fx_scale(E1);
   const FxMask km = fx_masks();
-  for (int nt = NB - 1; nt >= 0; --nt) {
-    const int ks_end = min(KS, (nt >> 1) + 1);
+  for (int n0 = (NB - 1) & ~1; n0 >= 0; n0 -= 2) {
+    const int ks_end = (n0 >> 1) + 1;
     const bool small = ks_end <= 2;
-    float acc[7][4], init[4];
+    float acc[2][7][4], init[4];
     fx_init(init, small);
     auto step = [&](int ks, auto first) {
       const unsigned char* p = yb + ks * 2048;
@@ -344,28 +392,28 @@ static __device__ __forceinline__ void tc_trmul_rows(unsigned char* yb, int b, c
       FxPair p10 = fx_pair(tc_ld(p + (o0 ^ 64)), tc_ld(p + (o1 ^ 64)), k1, km);
       FxPair p01 = fx_pair(tc_ld(p + 1024 + o0), tc_ld(p + 1024 + o1), k0, km);
       FxPair p11 = fx_pair(tc_ld(p + 1024 + (o0 ^ 64)), tc_ld(p + 1024 + (o1 ^ 64)), k1, km);
-      uint32_t bd[7][2];
-#pragma unroll
-      for (int J = 0; J < 7; ++J) {
-        const uint2 u = cf[((size_t)(nt * KS + ks) * 7 + J) * 32 + lane];
-        bd[J][0] = u.x;
-        bd[J][1] = u.y;
-      }
-      fx_step<decltype(first)::value>(acc, p00, p10, p01, p11, bd, km, init);
+      uint32_t bd[2][7][2];
+      tc_load_b<2>(cf, n0, NB, KS, ks, lane, bd);
+      fx_step<decltype(first)::value, 2>(acc, p00, p10, p01, p11, bd, km, init);
     };
     step(0, FxTrue());
 #pragma unroll 1
     for (int ks = 1; ks < ks_end; ++ks) step(ks, FxFalse());
-    fx_ints(acc, small);
-    __syncwarp();  // every lane has read this tile's columns
-    unsigned char* yt = yb + nt * 1024;
+    __syncwarp();  // every lane has read these tiles' columns
 #pragma unroll
-    for (int o = 0; o < 4; ++o) {
-      const int c = 8 * nt + 2 * t + (o & 1);
-      const double v = fx_join(acc, o);
-      if (c < b)
-        *reinterpret_cast<double*>(yt + (((o & 1) ? o1 : o0) ^ ((o >> 1) * 64))) =
-            v * fx_weight(o >> 1 ? E1 : E0, ec[c]);
+    for (int h = 0; h < 2; ++h) {
+      const int nt = n0 + h;
+      if (nt >= NB) break;
+      fx_ints(acc[h], small);
+      unsigned char* yt = yb + nt * 1024;
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        const int c = 8 * nt + 2 * t + (o & 1);
+        const double v = fx_join(acc[h], o);
+        if (c < b)
+          *reinterpret_cast<double*>(yt + (((o & 1) ? o1 : o0) ^ ((o >> 1) * 64))) =
+              v * fx_weight(o >> 1 ? E1 : E0, ec[c]);
+      }
     }
   }
 }
