@@ -157,8 +157,10 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     T = q == 1 ? 256 : 128;
     kc = q <= 2 ? 64 : 128;
   } else if (q == 1) {
-    const bool narrow = a + b <= 16, upd = rp.C && ax == 0;  // (update + sym8: more CTAs)
-    T = upd ? 64 : (narrow ? 256 : 128);
+    // update + sym8: an X stage of at most 32 KB (2^22 x 61: 539 us against 566 with 64 rows for
+    // every a and 581 with 128)
+    const bool narrow = a + b <= 16, upd = rp.C && ax == 0;
+    T = upd ? (a <= 16 ? 256 : (a <= 32 ? 128 : 64)) : (narrow ? 256 : 128);
     kc = narrow ? 64 : 32;
   } else if (q <= (narrow_gram ? 2 : 3)) {
     kc = 32;
