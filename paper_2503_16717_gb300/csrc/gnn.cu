@@ -230,21 +230,26 @@ __global__ void decode_back_edges_kernel(int64_t nnz, const int32_t* __restrict_
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const float w0 = bf(w, OFF_WO + lane);
   float acc[4] = {0.f, 0.f, 0.f, 0.f};  // g_wo[lane], g_wo[32+lane], g_wo[64+lane], g_bo (lane 0)
-  // edges warp0, warp0 + nwarps, ... in order, the loads of 4 of them issued together
-  for (int64_t q0 = warp0; q0 < nnz; q0 += 4 * nwarps) {
-    float d[4], ev[4], hi[4], hj[4];
+  // edges warp0, warp0 + nwarps, ... in order, the loads of U of them issued together
+  constexpr int U = 8;
+  for (int64_t q0 = warp0; q0 < nnz; q0 += U * nwarps) {
+    float d[U], ev[U], hi[U], hj[U];
+    int iu[U], ju[U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t q = q0 + u * nwarps;
-      const bool v = q < nnz;
-      const int i = v ? erow[q] : 0, j = v ? col[q] : 0;
-      d[u] = v ? dout[q] : 0.f;
-      ev[u] = v ? e[q * W + lane] : 0.f;
-      hi[u] = v ? h[(int64_t)i * W + lane] : 0.f;
-      hj[u] = v ? h[(int64_t)j * W + lane] : 0.f;
+    for (int u = 0; u < U; ++u) {
+      const int64_t q = std::min<int64_t>(q0 + u * nwarps, nnz - 1);
+      iu[u] = erow[q];
+      ju[u] = col[q];
+      d[u] = dout[q];
+      ev[u] = e[q * W + lane];
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < U; ++u) {
+      hi[u] = h[(int64_t)iu[u] * W + lane];
+      hj[u] = h[(int64_t)ju[u] * W + lane];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
       const int64_t q = q0 + u * nwarps;
       if (q < nnz) {
         acc[0] = fmaf(d[u], ev[u], acc[0]);
@@ -284,7 +289,18 @@ __global__ void gather_cols_kernel(int64_t n, const int32_t* __restrict__ rowptr
   const int64_t i = t / W;
   const int c = (int)(t % W);
   float s = dhl[t];
-  for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) s += dhj[(int64_t)tpos[e] * W + c];
+  const int re = rowptr[i + 1];
+  for (int e = rowptr[i]; e < re; e += 8) {  // 8 loads in flight, added in order
+    float v[8];
+    int p[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) p[u] = tpos[min(e + u, re - 1)];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = dhj[(int64_t)p[u] * W + c];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (e + u < re) s += v[u];
+  }
   dhl[t] = s;
 }
 
