@@ -348,7 +348,7 @@ static int loss_grad(rbo_gnn_s* g, const rbo_csr* A, const double* R, int nr, in
   decode_back_edges_kernel<<<NBLK_RED, BLK, sm_dec, st>>>(nnz, w.erow, A->col, w.e[NL], w.h[NL],
                                                           w.dout, g->wbf, w.de, w.part);
   reduce_group(g->dec, w.part, g->grad, st);
-  decode_back_nodes_kernel<<<grid1(n * W), 256, 0, st>>>(n, A->rowptr, w.tpos, w.dout, g->wbf, w.dh);
+  decode_back_nodes_kernel<<<grid1(n * (W / 4)), 256, 0, st>>>(n, A->rowptr, w.tpos, w.dout, g->wbf, w.dh);
   *launches += 3;
   float *dh = w.dh, *dhn = w.dh2, *de = w.de, *den = w.de2;
   for (int l = NL - 1; l >= 0; --l) {
@@ -363,7 +363,7 @@ static int loss_grad(rbo_gnn_s* g, const rbo_csr* A, const double* R, int nr, in
                                   &nb)))
       return e;
     reduce_group(g->layer_msg[l], w.part, g->grad, st, nb);
-    gather_cols_kernel<<<grid1(n * W), 256, 0, st>>>(n, A->rowptr, w.tpos, w.dhj, dhn);
+    gather_cols_kernel<<<grid1(n * (W / 4)), 256, 0, st>>>(n, A->rowptr, w.tpos, w.dhj, dhn);
     *launches += 5;
     std::swap(dh, dhn);
     std::swap(de, den);

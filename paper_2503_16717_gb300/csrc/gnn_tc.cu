@@ -650,7 +650,8 @@ __global__ void __launch_bounds__(TNT, 2) layer_back_tc_kernel(const __grid_cons
     const int64_t q0 = tile * TT + warp * 32;
     // An item past the last one, or of an index out of range, reads another's rows and takes
     // zeros instead: the loads have no branches, and a half's 80 of them are in flight together
-    // (512^2, 1.3 million edges: 790 us with a branch an edge, whose loads wait one by one)
+    // (512^2, 1.3 million edges: 277 us; 790 us with a branch an edge, whose loads wait one by
+    // one)
     int ri = 0, cj = 0;
     bool valid = q0 + lane < P.cnt;
     if (MSG && valid) {
