@@ -58,13 +58,15 @@ extern "C" {
 #define RBO_PREC_FP64   0  /* float64 data and results (the reference path).  The
                               projections y - x C and the Gram sums are formed on the
                               fp16 tensor cores from exact integer products: the values
-                              of a column over at most 64 rows (of a row over the columns,
+                              of a column over at most 128 rows (of a row over the columns,
                               for a projection) share a power-of-two scale and enter as
                               55-bit integers, off by at most a quarter of an ulp of the
                               largest of them; a group with a non-finite value or outside
-                              2^+-463 takes float64 FMAs.  The sketch sums 53-bit integers
+                              2^+-463 takes float64 FMAs.  The sketch sums 54-bit integers
                               on the scale of the column's largest value so far.
-                              Triangular solves and the small factors are IEEE float64    */
+                              Triangular solves are float64 substitutions, or for the last
+                              factors of big panels (near the identity) the same products
+                              with the float64 inverse; the small factors are IEEE float64 */
 #define RBO_PREC_MIXED  1  /* sketch apply and first-pass projection coefficients in
                               float32 with float32 accumulation; Gram matrices feeding
                               the final Cholesky, the small factors, every update of V

@@ -3,7 +3,7 @@
 //
 // The Gram matrices of BCGS and CholQR (Sections 4-5, the reductions Q^T W and W^T W)
 // are the float64 contractions of the method.  On this GPU the float64 pipe (2 FMA per
-// SM per clock) caps a float64 Gram pass near 1.1 TFLOP/s, far below the HBM rate, while
+// SM per clock) caps a Gram pass on it near 1.1 TFLOP/s, far below the HBM rate, while
 // the fp16 tensor cores are three orders of magnitude faster.  Splitting every float64
 // value into digits that fp16 represents exactly turns the Gram into exact integer
 // products (the idea of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012):
@@ -722,8 +722,11 @@ bool ozaki_gram_supported(const RowPass& rp) {
   return a + rp.b <= OZ_MAXA;
 }
 
-// Measured on GB300 (n = 1e6, b = 5): this kernel takes 0.30-0.34 ms whatever the width,
-// the float64 pass 0.11 ms at a = 5, 0.33 ms at a = 30 and 0.56 ms at a = 56.
+// Measured on GB300 (n = 1e6, b = 5): this kernel takes 0.27-0.34 ms whatever the width.  The
+// float64-pipe pass it was weighed against took 0.11 ms at a = 5, 0.33 ms at a = 30 and 0.56 ms
+// at a = 56; the float64 pass of today (digits too, rowpass_tc.cuh) takes 0.06, 0.11 and 0.19 ms.
+// The line stays where it was for callers who ask for this kernel's arithmetic by its precision
+// mode: float64 is the faster mode at every width.
 bool ozaki_gram_pays(const RowPass& rp) {
   const int a = rp.acc_x ? rp.a : 0;
   return a + rp.b >= 36;

@@ -22,10 +22,12 @@
 //      to the warps; an item always goes to the same warp, which keeps its float64 sums
 //      in its own shared-memory slots.
 // Measured on GB300, n = 2^22, b = 5, mean over a = 1, 6, .. 56 (float64-pipe kernels it
-// replaces -> here): Gram 1116 -> 500 us, update + Gram 1337 -> 844 us, solve + Gram
-// 1345 -> 658 us, update + sketch (d = 244, 8 entries a row) 1521 -> 1081 us; one-stage
-// orthogonalization of 61 columns 72.5 -> 44.3 ms.  The integer conversion bounds it (IPC
-// 2.0 of 4, ALU pipe 45 %, tensor pipe 20 %, DRAM 30 % of the copy rate).
+// replaces -> here): Gram 1116 -> 468 us, update + Gram 1337 -> 539 us, solve + Gram
+// 1345 -> 549 us, update + sketch (d = 244, 8 entries a row) 1521 -> 747 us; orthogonalization
+// of 61 columns in one stage 72.5 -> 33.6 ms, in two 76.3 -> 32.7 ms.  The integer conversion
+// bounds it (IPC 2.2 of 4, ALU pipe 45-50 %, tensor pipe 30 %, DRAM 35 % of the copy rate; a
+// pass of one to 16 columns X costs the same), in the sketch passes the bank conflicts of the
+// gathered sums too (870 shared-memory cycles a 64-row tile, 313 without conflicts).
 // The last CTAs reduce the partials in a fixed order and run the small dense epilogue
 // (rowpass_common.cuh).
 #pragma once
