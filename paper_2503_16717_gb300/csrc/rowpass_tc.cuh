@@ -204,7 +204,10 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       bool ok = mbar_wait_bounded(&bars[s], (uint32_t)(it >> 1) & 1u);
       if (XS && !XL) ok = mbar_wait_bounded(&barx, phx) && ok;
       if (__syncthreads_or(!ok)) {
-        if (tid == 0) set_error(P.status, RBO_ERR_TIMEOUT, 1);
+        if (tid == 0) {
+          set_error(P.status, RBO_ERR_TIMEOUT, 1);
+          if (XL && it == 0) mbar_wait_bounded(&barx, phx);  // the other copy in flight
+        }
         return;
       }
       if (!XL) phx ^= 1u;
@@ -390,7 +393,10 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       // the chunks of sym8 items are the warps' own rows; general items read other warps'
       if (XL && P.use_bulk) {
         if (__syncthreads_or(!mbar_wait_bounded(&barx, phx))) {
-          if (tid == 0) set_error(P.status, RBO_ERR_TIMEOUT, 1);
+          if (tid == 0) {
+            set_error(P.status, RBO_ERR_TIMEOUT, 1);
+            if (tile + (int)gridDim.x < P.ntiles) mbar_wait_bounded(&bars[s ^ 1], (uint32_t)((it + 1) >> 1) & 1u);
+          }
           return;
         }
         phx ^= 1u;
