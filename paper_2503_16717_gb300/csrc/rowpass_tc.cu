@@ -187,7 +187,7 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
     kc = (ax == 0 && b <= 8) ? std::max(16, T / 4) : std::min(kc, T);  // sym8: the warps' own rows
     l = tc_layout(a, b, T, q * (T / kc) * (want_inv || y_only ? 2 : 1), rp.C != nullptr, digits, rp.Tri != nullptr, want_inv && digits, d,
                   d > 0 ? rp.sk.rec_bytes : 0, xs);
-    smem = std::max(l.bytes, epi_bytes) + 1024;  // + alignment slack of the base
+    smem = std::max(l.bytes + 1024, epi_bytes);  // the tiles start at the next multiple of 1024
     if ((long long)smem <= limit) break;
     if (T > 16 && d == 0) T /= 2;
     else if (digits) {  // C stays float64, a factor is substituted

@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
     for (int item = 0; item < P.items; item += q) sum += p[(size_t)item * 128 * NT];
     mypart[o] = sum;
   }
-  tree_reduce_epilogue(P, smem, &s_flag, &s_last);
+  tree_reduce_epilogue(P, smem_raw, &s_flag, &s_last);
 }
 
 // The kernel of a kind of pass; null for a combination no pass uses
