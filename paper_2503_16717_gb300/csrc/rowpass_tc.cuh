@@ -355,7 +355,9 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
             ex = __reduce_max_sync(0xffffffffu, ex);
             if (lane == 0) {
               if (ex == 0x7FF) s_nan[c] = 1;
-              const int old = s_scale[c], now = (ex > old && ex != 0x7FF) ? ex + 1 : old;  // room to grow
+              // (room to grow, but never up to the exponent field of Inf and NaN, which must stay past
+              // every scale)
+              const int old = s_scale[c], now = (ex > old && ex != 0x7FF) ? min(ex + 1, 0x7FE) : old;
               s_shift[c] = min(now - old, 63);
               s_scale[c] = now;
             }
