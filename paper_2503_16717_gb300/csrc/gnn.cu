@@ -38,21 +38,32 @@ __device__ __forceinline__ float bf(const __nv_bfloat16* w, int i) { return __bf
 __device__ __forceinline__ float relu(float x) { return x > 0.f ? x : 0.f; }
 
 // ---- graph construction ---------------------------------------------------------------
-// per row: row id of every edge, diagonal value, position of (j, i) for every (i, j)
-__global__ void graph_edges_kernel(int64_t n, const int32_t* __restrict__ rowptr,
+// per row: row id of every edge, diagonal value, position of (j, i) for every (i, j).  Row
+// pointers that do not cover the nnz edges and columns outside the matrix are reported; the
+// kernels that use the rows or columns of the edges as indices return at once after an error,
+// so that no edge is left without its row.
+__global__ void graph_edges_kernel(int64_t n, int64_t nnz, const int32_t* __restrict__ rowptr,
                                    const int32_t* __restrict__ col, const double* __restrict__ val,
                                    int32_t* __restrict__ erow, int32_t* __restrict__ tpos,
                                    double* __restrict__ dinv, DevStatus* status) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int beg = rowptr[i], end = rowptr[i + 1];
+  if (beg < 0 || end < beg || (int64_t)end > nnz || (i == 0 && beg != 0) || (i == n - 1 && (int64_t)end != nnz)) {
+    set_error(status, RBO_ERR_ARG, 22);
+    return;
+  }
   double dia = 0.0;
   for (int e = beg; e < end; ++e) {
     erow[e] = (int32_t)i;
     const int j = col[e];
+    if (j < 0 || (int64_t)j >= n) {
+      set_error(status, RBO_ERR_ARG, 23);
+      return;
+    }
     if (j == (int)i) dia = val[e];
     // binary search for column i in row j (columns sorted)
-    int lo = rowptr[j], hi = rowptr[j + 1] - 1, pos = -1;
+    int lo = max(rowptr[j], 0), hi = (int)std::min<int64_t>(rowptr[j + 1], nnz) - 1, pos = -1;
     while (lo <= hi) {
       const int mid = (lo + hi) >> 1;
       const int cm = col[mid];
@@ -69,9 +80,9 @@ __global__ void graph_edges_kernel(int64_t n, const int32_t* __restrict__ rowptr
 __global__ void graph_features_kernel(int64_t n, const int32_t* __restrict__ rowptr,
                                       const int32_t* __restrict__ col, const double* __restrict__ val,
                                       const int32_t* __restrict__ tpos, const double* __restrict__ dinv,
-                                      float* __restrict__ x, float* __restrict__ f) {
+                                      float* __restrict__ x, float* __restrict__ f, const DevStatus* status) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || status->code != 0) return;
   double rs = 0.0, cs = 0.0;
   for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
     const int j = col[e];
@@ -110,9 +121,9 @@ __global__ void decode_terms_kernel(int64_t nnz, const int32_t* __restrict__ ero
                                     const int32_t* __restrict__ col, const float* __restrict__ pe,
                                     const float* __restrict__ sdec, const float* __restrict__ tdec,
                                     const __nv_bfloat16* __restrict__ w, const double* __restrict__ dinv,
-                                    double* __restrict__ Mval) {
+                                    double* __restrict__ Mval, const DevStatus* status) {
   const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (q >= nnz) return;
+  if (q >= nnz || status->code != 0) return;
   const int i = erow[q], j = col[q];
   const float out = pe[q] + sdec[i] + tdec[j] + bf(w, OFF_BO) + (i == j ? 1.f : 0.f);
   Mval[q] = (double)out * dinv[i];
@@ -123,9 +134,9 @@ __global__ void decode_terms_kernel(int64_t nnz, const int32_t* __restrict__ ero
 __global__ void spmm_kernel(int64_t n, int nr, const int32_t* __restrict__ rowptr,
                             const int32_t* __restrict__ col, const double* __restrict__ v,
                             const double* __restrict__ R, int64_t ldr, double* __restrict__ Z,
-                            int64_t ldz) {
+                            int64_t ldz, const DevStatus* status) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= n * nr) return;
+  if (t >= n * nr || status->code != 0) return;
   const int64_t i = t % n;
   const int k = (int)(t / n);
   double s = 0.0;

@@ -16,10 +16,10 @@ namespace rbo {
 namespace gnn {
 
 // kernels (gnn.cu)
-__global__ void graph_edges_kernel(int64_t, const int32_t*, const int32_t*, const double*, int32_t*,
+__global__ void graph_edges_kernel(int64_t, int64_t, const int32_t*, const int32_t*, const double*, int32_t*,
                                    int32_t*, double*, DevStatus*);
 __global__ void graph_features_kernel(int64_t, const int32_t*, const int32_t*, const double*,
-                                      const int32_t*, const double*, float*, float*);
+                                      const int32_t*, const double*, float*, float*, const DevStatus*);
 __global__ void encode_kernel(int64_t, int, const float*, const __nv_bfloat16*, int, int, float*);
 // tensor-core message and node-update layers (gnn_tc.cu)
 int message_tc_launch(bool train, int64_t nnz, int64_t n, const int32_t* rowptr, const int32_t* erow,
@@ -30,9 +30,10 @@ int node_update_tc_launch(int64_t n, const int32_t* rowptr, float* agg, const fl
                           const float* hin, const float* f, const __nv_bfloat16* w, int l, float* rh, float* hout, float* sdec,
                           float* tdec, DevStatus* status, cudaStream_t st);
 __global__ void decode_terms_kernel(int64_t, const int32_t*, const int32_t*, const float*, const float*,
-                                    const float*, const __nv_bfloat16*, const double*, double*);
+                                    const float*, const __nv_bfloat16*, const double*, double*,
+                                    const DevStatus*);
 __global__ void spmm_kernel(int64_t, int, const int32_t*, const int32_t*, const double*,
-                            const double*, int64_t, double*, int64_t);
+                            const double*, int64_t, double*, int64_t, const DevStatus*);
 __global__ void spmm_t_kernel(int64_t, int, const int32_t*, const int32_t*, const int32_t*,
                               const double*, const double*, int64_t, double*, int64_t);
 __global__ void residual_norms_kernel(int64_t, int, const double*, int64_t, double*, int64_t,
@@ -263,10 +264,10 @@ static unsigned grid1(int64_t threads, int bs = 256) {
 static int forward(rbo_gnn_s* g, const rbo_csr* A, Work& w, Arena* ar, cudaStream_t st, bool train,
                    int* launches) {
   const int64_t n = A->n, nnz = A->nnz;
-  graph_edges_kernel<<<grid1(n), 256, 0, st>>>(n, A->rowptr, A->col, A->val, w.erow, w.tpos, w.dinv,
+  graph_edges_kernel<<<grid1(n), 256, 0, st>>>(n, nnz, A->rowptr, A->col, A->val, w.erow, w.tpos, w.dinv,
                                                ar->status);
   graph_features_kernel<<<grid1(n), 256, 0, st>>>(n, A->rowptr, A->col, A->val, w.tpos, w.dinv, w.x,
-                                                  w.f);
+                                                  w.f, ar->status);
   // (inference computes h_0 from the features inside the first layer)
   if (train) encode_kernel<<<grid1(n * W), 256, 0, st>>>(n, 2, w.f, g->wbf, OFF_WN, OFF_BN, w.h[0]);
   *launches += train ? 3 : 2;
@@ -289,7 +290,7 @@ static int forward(rbo_gnn_s* g, const rbo_csr* A, Work& w, Arena* ar, cudaStrea
     *launches += 2;
   }
   decode_terms_kernel<<<grid1(nnz), 256, 0, st>>>(nnz, w.erow, A->col, w.pe, w.sdec, w.tdec, g->wbf,
-                                                  w.dinv, w.Mval);
+                                                  w.dinv, w.Mval, ar->status);
   *launches += 1;
   return note_cuda(cudaGetLastError());
 }
@@ -312,8 +313,8 @@ static int loss_grad(rbo_gnn_s* g, const rbo_csr* A, const double* R, int nr, in
   if ((e = work_take(ar, w, n, nnz, nr, true))) return e;
   if ((e = forward(g, A, w, ar, st, true, launches))) return e;
   // Z = M R ; Y = A Z ; E = R - Y (in Y) with per-block norms
-  spmm_kernel<<<grid1(n * nr), 256, 0, st>>>(n, nr, A->rowptr, A->col, w.Mval, R, ldr, w.Z, n);
-  spmm_kernel<<<grid1(n * nr), 256, 0, st>>>(n, nr, A->rowptr, A->col, A->val, w.Z, n, w.Y, n);
+  spmm_kernel<<<grid1(n * nr), 256, 0, st>>>(n, nr, A->rowptr, A->col, w.Mval, R, ldr, w.Z, n, ar->status);
+  spmm_kernel<<<grid1(n * nr), 256, 0, st>>>(n, nr, A->rowptr, A->col, A->val, w.Z, n, w.Y, n, ar->status);
   const int nb = 256;
   residual_norms_kernel<<<dim3(nb, nr), 256, 0, st>>>(n, nr, R, ldr, w.Y, n, w.npart);
   *launches += 3;
