@@ -179,7 +179,7 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   };
   TcKernel kern = kernel_of(want_inv ? 2 : (rp.Tri ? 1 : 0));
   if (!kern) return RBO_ERR_ARG;
-  const int limit = tc_smem_limit((const void*)kern);
+  int limit = tc_smem_limit((const void*)kern);
   const size_t epi_bytes = ((size_t)L + 2) * 8 + epilogue_doubles(rp) * 8;
   TcLayout l;
   size_t smem = 0;
@@ -199,6 +199,8 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
         want_inv = false;
         count_items();
         kern = kernel_of(1);
+        if (!kern) return RBO_ERR_ARG;
+        limit = tc_smem_limit((const void*)kern);
       }
     } else return RBO_ERR_ARG;
   }
