@@ -1,10 +1,10 @@
 // CSR sparse kernels of the matrix-powers kernel (Section 4) and the small vector
 // kernels of the GMRES driver.
 //
-// SpMV: rows of up to ~12 entries on average (stencils) go to a persistent kernel in
-// which each warp stages the entries of 32 consecutive rows in shared memory and
-// every lane runs its own row; denser rows use a group of LPR = 8 or 32 lanes per
-// row that read consecutive entries and combine with shuffles in a fixed order.
+// SpMV: rows of up to ~12 entries on average (stencils) go to a kernel in which each
+// block stages the entries of 256 consecutive rows in shared memory and every thread
+// runs its own row; denser rows use a group of LPR = 8 or 32 lanes per row that read
+// consecutive entries and combine with shuffles in a fixed order.
 // Every sum has a fixed order, so the result is deterministic.  The optional
 // diagonal scaling D of the right Jacobi preconditioner (A D x) is applied to the
 // gathered x entries; the optional shift terms of the Newton and Chebyshev bases
@@ -68,93 +68,221 @@ __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, int64_t nnz,
 // (no load instructions and no registers for the bytes in flight, which bound an earlier
 // form that staged 32 rows per warp with plain loads), then every thread walks its own row,
 // the x gathers of 8 entries in flight.  Two interleaved chains per row (even and odd
-// entries) added at the end, a fixed order; no cross-lane float64 reduction.  Blocks with
-// more entries than the staging holds (`cap`), malformed row pointers or unaligned arrays
-// read them from global memory instead.  SCALE is a template argument because the float64
-// pipe (2 operations per SM and cycle) bounds the kernel: a multiplication by a scale that
-// is not there would be half of its work.  7-point 100^3: 40 -> 27 us, 5-point 2048^2: 111 ->
-// 79 us (63 % of the copy rate); one row per thread straight from global memory 45 and 139 us.
-constexpr int SPR = 256;  // rows (threads) per block
+// entries) added at the end, a fixed order; no cross-lane float64 reduction.  Arrays that are
+// not 16-byte aligned are staged with plain loads.  SCALE is a template argument because the
+// float64 pipe (2 operations per SM and cycle) bounds the kernel: a multiplication by a scale
+// that is not there would be half of its work.  32 rows a warp staged with plain loads -> here:
+// 7-point 100^3 39 -> 24 us, 5-point 2048^2 111 -> 64 us (78 % of the copy rate); one row per
+// thread straight from global memory 45 and 139 us.  8 blocks per SM (32 registers): the solve of
+// 60 iterations at 2048^2 takes 41.2 ms, with 6 blocks 42.4.
+// Blocks with more entries than the staging holds (`cap`) stage them piece by piece.  There a
+// row of more than SPL_WARP entries is summed by its warp and one of more than SPL_BLOCK by
+// the block, so that no thread walks a long row alone while the others wait (10^6 rows, one of
+// 100000 entries: 5.0 ms staged per warp, 10 ms walked by its thread, 0.2 ms here; rows of 20 and
+// of 2 entries, half each: 165 us walked from global memory, 100 us in pieces).
+constexpr int SPR = 256;         // rows (threads) per block
+constexpr int SPL_WARP = 128;    // about where a thread's chain of gathers takes as long as the
+                                 // warp's turn and its reduction
+constexpr int SPL_BLOCK = 4096;  // 16 turns of a warp; 2 of the block, whose reduction has barriers
+struct SpmvArgs {
+  int64_t n, nnz;
+  const int32_t* rowptr;
+  const int32_t* col;
+  const double* val;
+  const double* dscale;
+  const double* x;
+  const double* bvec;
+  double* y;
+  DevStatus* status;
+  SpmvShift sh;
+  uint32_t ncol;  // columns that a 32-bit index can name: min(n, 2^31)
+  int cap, bulk;  // entries that the staging holds; arrays are aligned for bulk copies
+};
+// entries cp[0..len), vp[0..len) added to the two chains; bad: a column outside the matrix.
+// Whole warp: the lanes leave the products of a turn together, after the warp's longest row,
+// since a float64 operation takes its pipe for 16 cycles for one lane as for 32, and when its
+// predicate is off in all of them (5 entries a row at 2048^2: 83 -> 64 us).
+template <bool SCALE, int U>
+__device__ __forceinline__ void spmv_walk(const SpmvArgs& A, const int32_t* cp, const double* vp, int len, double& s0,
+                                          double& s1, bool& bad) {
+  const int longest = __reduce_max_sync(0xffffffffu, len);
+  for (int e = 0; e < longest; e += U) {
+    const int k = len - e, kw = longest - e;  // entries left
+    int c[U];
+    double xv[U], dv[SCALE ? U : 1];
+#pragma unroll
+    for (int j = 0; j < U; ++j) c[j] = j < k ? cp[e + j] : -1;
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const bool ok = (uint32_t)c[j] < A.ncol;
+      bad = bad || (j < k && !ok);
+      xv[j] = 0.0;
+      if (SCALE) dv[j] = 0.0;
+      if (ok) {
+        xv[j] = __ldg(A.x + c[j]);
+        if (SCALE) dv[j] = __ldg(A.dscale + c[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      if (j >= kw) break;
+      const double t = SCALE ? dv[j] * xv[j] : xv[j], v = j < k ? vp[e + j] : 0.0;
+      if (j & 1) s1 = fma(v, t, s1);
+      else s0 = fma(v, t, s0);
+    }
+  }
+}
+
+// row pointers of row r, whose block's entries are e0 .. e1 - 1 (range: a part of the arrays); a
+// row that is not part of them is reported and left empty
+__device__ __forceinline__ void spmv_row(const SpmvArgs& A, int64_t r, int e0, int e1, bool range, int& beg, int& end) {
+  beg = end = 0;
+  if (r >= A.n) return;
+  beg = __ldg(A.rowptr + r);
+  end = __ldg(A.rowptr + r + 1);
+  if (range ? (beg < e0 || end < beg || end > e1) : (beg < 0 || end < beg || (int64_t)end > A.nnz)) {
+    if (A.status) set_error(A.status, RBO_ERR_ARG, 11);
+    end = beg;
+  }
+}
+__device__ __forceinline__ void spmv_store(const SpmvArgs& A, int64_t r, double s, bool bad) {
+  if (bad && A.status) set_error(A.status, RBO_ERR_ARG, 12);
+  if (r < A.n) A.y[r] = A.bvec ? (A.bvec[r] - s) : shifted(s, A.sh, r);
+}
+
+// Sum of this thread's row where it is a long one, else 0: rows of more than SPL_WARP entries by
+// their warp, of more than SPL_BLOCK by the block.  Whole block.
 template <bool SCALE>
-__global__ void __launch_bounds__(SPR, 6) spmv_block_kernel(int64_t n, int64_t nnz, int cap,
-                                                         const int32_t* __restrict__ rowptr,
-                                                         const int32_t* __restrict__ col,
-                                                         const double* __restrict__ val,
-                                                         const double* __restrict__ dscale,
-                                                         const double* __restrict__ x,
-                                                         const double* __restrict__ bvec,
-                                                         double* __restrict__ y, DevStatus* status,
-                                                         SpmvShift sh) {
+__device__ __noinline__ double spmv_long_rows(const SpmvArgs& A, int64_t r0, int beg, int len) {
+  __shared__ double s_red[32];
+  __shared__ unsigned s_long[SPR / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double s0 = 0.0;
+  bool bad = false;
+  // part of a long row: entries id, id + step, ..
+  auto part = [&](int from, int cnt, int id, int step) {
+    double t = 0.0;
+    for (int64_t e = id; e < cnt; e += 4 * (int64_t)step) {
+      double p[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t q = e + u * (int64_t)step;
+        p[u] = 0.0;
+        if (q < cnt) {
+          const int cj = __ldg(A.col + from + q);
+          const bool ok = (uint32_t)cj < A.ncol;
+          bad = bad || !ok;
+          if (ok) p[u] = __ldg(A.val + from + q) * (SCALE ? __ldg(A.dscale + cj) * __ldg(A.x + cj) : __ldg(A.x + cj));
+        }
+      }
+      t += (p[0] + p[1]) + (p[2] + p[3]);
+    }
+    return t;
+  };
+  for (unsigned m = __ballot_sync(0xffffffffu, len > SPL_WARP && len <= SPL_BLOCK); m; m &= m - 1u) {
+    const int l = __ffs((int)m) - 1;
+    const double t = warp_sum(part(__shfl_sync(0xffffffffu, beg, l), __shfl_sync(0xffffffffu, len, l), lane, 32));
+    if (lane == l) s0 = t;
+  }
+  const unsigned lb = __ballot_sync(0xffffffffu, len > SPL_BLOCK);
+  if (lane == 0) s_long[warp] = lb;
+  __syncthreads();
+  for (int w = 0; w < SPR / 32; ++w)
+    for (unsigned m = s_long[w]; m; m &= m - 1u) {
+      const int t = 32 * w + __ffs((int)m) - 1, from = __ldg(A.rowptr + r0 + t);
+      const double v = block_sum(part(from, __ldg(A.rowptr + r0 + t + 1) - from, tid, SPR), s_red);
+      if (tid == t) s0 = v;
+    }
+  if (bad && A.status) set_error(A.status, RBO_ERR_ARG, 12);
+  return s0;
+}
+
+// A block whose entries do not fit the staging at once, or whose row pointers are out of order.
+// Apart from the kernel, whose registers it would take.
+template <bool SCALE>
+__device__ __noinline__ void spmv_pieces(const SpmvArgs& A, double* sval, int32_t* scol) {
+  const int tid = threadIdx.x, cap = A.cap;
+  const int64_t r0 = blockIdx.x * (int64_t)SPR, r = r0 + tid;
+  const int e0 = __ldg(A.rowptr + r0), e1 = __ldg(A.rowptr + (r0 + SPR < A.n ? r0 + SPR : A.n));
+  const bool range = e0 >= 0 && e1 >= e0 && (int64_t)e1 <= A.nnz;
+  int beg, end;
+  spmv_row(A, r, e0, e1, range, beg, end);
+  const int len = end - beg;
+  const bool lng = len > SPL_WARP;
+  double s0 = 0.0, s1 = 0.0;
+  bool bad = false;
+  if (!range) {  // the rows that lie in the arrays
+    spmv_walk<SCALE, SCALE ? 2 : 4>(A, A.col + beg, A.val + beg, len, s0, s1, bad);
+    spmv_store(A, r, s0 + s1, bad);
+    return;
+  }
+  for (int64_t k0 = e0; k0 < e1; k0 += cap) {
+    const int k1 = (int)(k0 + cap < e1 ? k0 + cap : e1), lo = beg > k0 ? beg : (int)k0, hi = end < k1 ? end : k1;
+    const bool mine = !lng && lo < hi;
+    if (!__syncthreads_or(mine)) continue;  // (the readers of the last piece are done)
+    const int cnt = k1 - (int)k0;
+    for (int e = tid; e < cnt; e += 4 * SPR) {  // 8 loads in flight
+      double v[4];
+      int c[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (e + u * SPR < cnt) {
+          v[u] = __ldg(A.val + k0 + e + u * SPR);
+          c[u] = __ldg(A.col + k0 + e + u * SPR);
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (e + u * SPR < cnt) {
+          sval[e + u * SPR] = v[u];
+          scol[e + u * SPR] = c[u];
+        }
+    }
+    __syncthreads();
+    spmv_walk<SCALE, SCALE ? 2 : 4>(A, scol + (lo - (int)k0), sval + (lo - (int)k0), mine ? hi - lo : 0, s0, s1, bad);
+  }
+  s0 += spmv_long_rows<SCALE>(A, r0, beg, len);
+  spmv_store(A, r, s0 + s1, bad);
+}
+
+template <bool SCALE>
+__global__ void __launch_bounds__(SPR, SCALE ? 6 : 8) spmv_block_kernel(const __grid_constant__ SpmvArgs A) {
   extern __shared__ __align__(16) unsigned char sm_sp[];
   __shared__ __align__(8) uint64_t bar;
-  double* sval = reinterpret_cast<double*>(sm_sp);                 // cap + 2 values
-  int32_t* scol = reinterpret_cast<int32_t*>(sval + cap + 2);       // cap + 4 indices
+  double* sval = reinterpret_cast<double*>(sm_sp);                   // cap + 2 values
+  int32_t* scol = reinterpret_cast<int32_t*>(sval + A.cap + 2);       // cap + 4 indices
   const int tid = threadIdx.x;
   const int64_t r0 = blockIdx.x * (int64_t)SPR, r = r0 + tid;
-  const int64_t rl = r0 + SPR < n ? r0 + SPR : n;
-  const int e0 = __ldg(rowptr + r0), e1 = __ldg(rowptr + rl);
-  const bool staged = cap > 0 && e0 >= 0 && e1 >= e0 && (int64_t)e1 <= nnz && e1 - e0 <= cap;
+  const int e0 = __ldg(A.rowptr + r0), e1 = __ldg(A.rowptr + (r0 + SPR < A.n ? r0 + SPR : A.n));
+  if (e0 < 0 || e1 < e0 || (int64_t)e1 > A.nnz || e1 - e0 > A.cap) {
+    spmv_pieces<SCALE>(A, sval, scol);
+    return;
+  }
   // 16-byte aligned starts at or before e0, whole 16-byte pieces before e1
-  const int v0 = e0 & ~1, c0 = e0 & ~3;
-  if (staged) {
-    const uint32_t bv = (uint32_t)(e1 - v0) * 8u & ~15u, bc = (uint32_t)(e1 - c0) * 4u & ~15u;
-    if (tid == 0) {
+  const int v0 = A.bulk ? e0 & ~1 : e0, c0 = A.bulk ? e0 & ~3 : e0;
+  {
+    const uint32_t bv = A.bulk ? (uint32_t)(e1 - v0) * 8u & ~15u : 0u, bc = A.bulk ? (uint32_t)(e1 - c0) * 4u & ~15u : 0u;
+    if (tid == 0 && A.bulk) {
       mbar_init(&bar, 1);
       fence_mbar_init();
       mbar_arrive_expect_tx(&bar, bv + bc);
-      if (bv) bulk_copy_g2s(sval, val + v0, bv, &bar);
-      if (bc) bulk_copy_g2s(scol, col + c0, bc, &bar);
+      if (bv) bulk_copy_g2s(sval, A.val + v0, bv, &bar);
+      if (bc) bulk_copy_g2s(scol, A.col + c0, bc, &bar);
     }
     // what is left after the whole pieces
-    for (int e = v0 + (int)(bv / 8) + tid; e < e1; e += SPR) sval[e - v0] = __ldg(val + e);
-    for (int e = c0 + (int)(bc / 4) + tid; e < e1; e += SPR) scol[e - c0] = __ldg(col + e);
+    for (int e = (int)(bv / 8) + tid; e < e1 - v0; e += SPR) sval[e] = __ldg(A.val + v0 + e);
+    for (int e = (int)(bc / 4) + tid; e < e1 - c0; e += SPR) scol[e] = __ldg(A.col + c0 + e);
   }
-  int beg = 0, end = 0;
-  if (r < n) {
-    beg = __ldg(rowptr + r);
-    end = __ldg(rowptr + r + 1);
-    const bool bad = staged ? (beg < e0 || end < beg || end > e1) : (beg < 0 || end < beg || (int64_t)end > nnz);
-    if (bad) {
-      if (status) set_error(status, RBO_ERR_ARG, 11);
-      end = beg;
-    }
-  }
+  int beg, end;
+  spmv_row(A, r, e0, e1, true, beg, end);
   __syncthreads();
-  if (staged && !mbar_wait_bounded(&bar, 0u)) {
-    if (status) set_error(status, RBO_ERR_TIMEOUT, 13);
+  if (A.bulk && !mbar_wait_bounded(&bar, 0u)) {
+    if (A.status) set_error(A.status, RBO_ERR_TIMEOUT, 13);
     return;
   }
-  if (r >= n) return;
   double s0 = 0.0, s1 = 0.0;
   bool bad = false;
-  auto walk = [&](const int32_t* cp, const double* vp, int len) {
-    for (int e = 0; e < len; e += 8) {
-      const int k = len - e;  // entries left
-      int c[8];
-      double v[8], xv[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) c[j] = j < k ? cp[e + j] : 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const bool ok = (uint64_t)(int64_t)c[j] < (uint64_t)n;
-        bad = bad || !ok;
-        const int cj = ok ? c[j] : 0;
-        xv[j] = __ldg(x + cj);
-        if (SCALE) xv[j] *= __ldg(dscale + cj);
-        v[j] = ok && j < k ? vp[e + j] : 0.0;
-      }
-#pragma unroll
-      for (int j = 0; j < 8; j += 2) {
-        if (j < k) s0 = fma(v[j], xv[j], s0);
-        if (j + 1 < k) s1 = fma(v[j + 1], xv[j + 1], s1);
-      }
-    }
-  };
-  if (staged) walk(scol + (beg - c0), sval + (beg - v0), end - beg);
-  else walk(col + beg, val + beg, end - beg);
-  if (bad && status) set_error(status, RBO_ERR_ARG, 12);
-  const double s = s0 + s1;
-  y[r] = bvec ? (bvec[r] - s) : shifted(s, sh, r);
+  spmv_walk<SCALE, SCALE ? 4 : 8>(A, scol + (beg - c0), sval + (beg - v0), end - beg, s0, s1, bad);
+  spmv_store(A, r, s0 + s1, bad);
 }
 
 static int spmv_dispatch_inner(const CsrDev& A, const double* dscale, const double* x,
@@ -196,16 +324,16 @@ static int spmv_dispatch_inner(const CsrDev& A, const double* dscale, const doub
   if (avg <= 12.0) {
     const int64_t blocks = (A.n + SPR - 1) / SPR;
     if (blocks > 0x7FFFFFFFLL) return RBO_ERR_ARG;
-    // staging for a quarter more entries than the average block has (at most 3840: 46 KB)
-    const bool aligned = ((uintptr_t)A.col & 15) == 0 && ((uintptr_t)A.val & 15) == 0;
-    const int cap = aligned ? ((int)(avg * SPR * 1.25) + 67) & ~3 : 0;
+    // staging for a quarter more entries than the average block has (at most 3904: 46 KB)
+    const int bulk = ((uintptr_t)A.col & 15) == 0 && ((uintptr_t)A.val & 15) == 0 ? 1 : 0;
+    const int cap = ((int)(avg * SPR * 1.25) + 67) & ~3;
     const size_t smem = (size_t)(cap + 2) * 8 + (size_t)(cap + 4) * 4;
+    SpmvArgs P{A.n, A.nnz, A.rowptr, A.col, A.val, dscale, x, b, y, status, sh,
+               (uint32_t)std::min<int64_t>(A.n, (int64_t)1 << 31), cap, bulk};
     if (dscale)
-      spmv_block_kernel<true><<<(unsigned)blocks, SPR, smem, st>>>(A.n, A.nnz, cap, A.rowptr, A.col, A.val, dscale,
-                                                                   x, b, y, status, sh);
+      spmv_block_kernel<true><<<(unsigned)blocks, SPR, smem, st>>>(P);
     else
-      spmv_block_kernel<false><<<(unsigned)blocks, SPR, smem, st>>>(A.n, A.nnz, cap, A.rowptr, A.col, A.val, dscale,
-                                                                    x, b, y, status, sh);
+      spmv_block_kernel<false><<<(unsigned)blocks, SPR, smem, st>>>(P);
   } else if (avg <= 24.0)
     spmv_go<8>(A, dscale, x, b, y, status, st, sh);
   else
