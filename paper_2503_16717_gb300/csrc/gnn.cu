@@ -309,7 +309,7 @@ __global__ void decode_back_edges_kernel(int64_t nnz, const int32_t* __restrict_
 }
 
 // dh_i = wo[32:64] * sum_{e in row i} dout_e + wo[64:96] * sum_{e in row i} dout_{tpos e}
-__global__ void decode_back_nodes_kernel(int64_t n, const int32_t* __restrict__ rowptr,
+__global__ void __launch_bounds__(256, 5) decode_back_nodes_kernel(int64_t n, const int32_t* __restrict__ rowptr,
                                          const int32_t* __restrict__ tpos,
                                          const float* __restrict__ dout,
                                          const __nv_bfloat16* __restrict__ w, float* __restrict__ dh) {
@@ -318,17 +318,23 @@ __global__ void decode_back_nodes_kernel(int64_t n, const int32_t* __restrict__ 
   const int64_t i = t / (W / 4);
   const int c = 4 * (int)(t % (W / 4));
   float s1 = 0.f, s2 = 0.f;
-  const int re = rowptr[i + 1];
-  for (int e = rowptr[i]; e < re; e += 8) {  // 8 loads in flight, added in order
+  // 8 loads in flight, added in order; the indices of the next 8 come in with them (as in
+  // gather_cols_kernel: a row of 10^5 edges waits for one load after another otherwise; loss and
+  // gradient with such a row 181 -> 146 ms)
+  const int rb = rowptr[i], re = rowptr[i + 1];
+  int p[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) p[u] = rb < re ? tpos[min(rb + u, re - 1)] : 0;
+  for (int e = rb; e < re; e += 8) {
     float a[8], b[8];
-    int p[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      p[u] = tpos[min(e + u, re - 1)];
+      b[u] = dout[p[u]];
       a[u] = dout[min(e + u, re - 1)];
     }
+    if (e + 8 < re)
 #pragma unroll
-    for (int u = 0; u < 8; ++u) b[u] = dout[p[u]];
+      for (int u = 0; u < 8; ++u) p[u] = tpos[min(e + 8 + u, re - 1)];
 #pragma unroll
     for (int u = 0; u < 8; ++u)
       if (e + u < re) {
@@ -345,7 +351,7 @@ __global__ void decode_back_nodes_kernel(int64_t n, const int32_t* __restrict__ 
 // dh_l[i] += sum over row i of dhj[tpos e]  (the column scatter, gathered per node); 8 lanes
 // a node, 8 edges in flight, added in order (1.3 million edges: 35 us; 70 us with a row of 128 bytes a
 // load, one edge after the other)
-__global__ void gather_cols_kernel(int64_t n, const int32_t* __restrict__ rowptr,
+__global__ void __launch_bounds__(256, 5) gather_cols_kernel(int64_t n, const int32_t* __restrict__ rowptr,
                                    const int32_t* __restrict__ tpos, const float* __restrict__ dhj,
                                    float* __restrict__ dhl) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -354,14 +360,17 @@ __global__ void gather_cols_kernel(int64_t n, const int32_t* __restrict__ rowptr
   const int c4 = (int)(t % (W / 4));
   float4* out = reinterpret_cast<float4*>(dhl + i * W) + c4;
   float4 s = *out;
-  const int re = rowptr[i + 1];
-  for (int e = rowptr[i]; e < re; e += 8) {
-    float4 v[8];
-    int p[8];
+  const int rb = rowptr[i], re = rowptr[i + 1];
+  int p[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) p[u] = tpos[min(e + u, re - 1)];
+  for (int u = 0; u < 8; ++u) p[u] = rb < re ? tpos[min(rb + u, re - 1)] : 0;
+  for (int e = rb; e < re; e += 8) {
+    float4 v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = *row4(dhj, p[u], c4);
+    if (e + 8 < re)  // (the indices of the next 8 come in with these rows)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) p[u] = tpos[min(e + 8 + u, re - 1)];
 #pragma unroll
     for (int u = 0; u < 8; ++u)
       if (e + u < re) {

@@ -491,8 +491,11 @@ __global__ void __launch_bounds__(TNT, TCTAS)
         buf[j * TLD + 32 + lane] = av[j];
       }
     }
-    // the messages behind the cuts, in order, 16 loads in flight: the k-th belongs to the node
-    // whose count range holds k
+    // The messages behind the cuts, in order: the k-th belongs to the node whose count range
+    // holds k.  A node's sum stays in a register until the next node's first message; 32
+    // messages of one node are consecutive rows of m, added without a look at their nodes
+    // (inference with 20 rows of 10^4 edges: 16.3 ms with all messages read here, 40 with a sum
+    // in shared memory and 16 messages in flight, 14.6 here; 100 edges a row: 1.63, 2.23, 1.63).
     if (cut) {
       int upto = tn;  // counts up to and including this lane's node
 #pragma unroll
@@ -501,12 +504,33 @@ __global__ void __launch_bounds__(TNT, TCTAS)
         if (lane >= o) upto += u;
       }
       const int total = __shfl_sync(0xffffffffu, upto, 31);
-      for (int k0 = 0; k0 < total; k0 += 16) {
+      float* sum = buf + 32 + lane;
+      int cur = -1;
+      float run = 0.f;
+      auto open = [&](int j) {  // j is the node of the messages that follow
+        if (j == cur) return;
+        if (cur >= 0) sum[cur * TLD] = run;
+        run = sum[j * TLD];
+        cur = j;
+      };
+      for (int k0 = 0; k0 < total;) {
         int node = 0;  // lane k: node of message k0 + k
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
           if (__shfl_sync(0xffffffffu, upto, node + o - 1) <= k0 + lane) node += o;
         const int edge = __shfl_sync(0xffffffffu, te - (upto - tn), node) + k0 + lane;
+        const int first = __shfl_sync(0xffffffffu, node, 0);
+        if (k0 + 32 <= total && __all_sync(0xffffffffu, node == first)) {
+          const float* mq = m + (int64_t)__shfl_sync(0xffffffffu, edge, 0) * W + lane;
+          float v[32];
+#pragma unroll
+          for (int u = 0; u < 32; ++u) v[u] = mq[u * W];
+          open(first);
+#pragma unroll
+          for (int u = 0; u < 32; ++u) run += v[u];
+          k0 += 32;
+          continue;
+        }
         float v[16];
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
@@ -516,9 +540,14 @@ __global__ void __launch_bounds__(TNT, TCTAS)
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
           const int j = __shfl_sync(0xffffffffu, node, u);
-          if (k0 + u < total) buf[j * TLD + 32 + lane] += v[u];
+          if (k0 + u < total) {
+            open(j);
+            run += v[u];
+          }
         }
+        k0 += 16;
       }
+      if (cur >= 0) sum[cur * TLD] = run;
     }
     if (keep_agg) {  // cut rows, and nodes without edges
 #pragma unroll 8
