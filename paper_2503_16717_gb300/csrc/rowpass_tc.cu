@@ -110,8 +110,8 @@ int rowpass_sketch_T(int a_max, int b_max, int d, int zeta) {
 int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* launches, int num_sms) {
   RowPass rp = rpin;
   const int d = rp.sk_d > 0 ? rp.sk_d : 0;
-  // A tensor copy's coordinates are 32 bits wide.  Longer arrays are staged with plain loads in
-  // the sketch passes, which no other kernel serves; the others go to rowpass_kernel.
+  // A tensor copy's coordinates are 32 bits wide.  Longer arrays come in without it in the sketch
+  // passes, which no other kernel serves; the others go to rowpass_kernel.
   const bool long_rows = rp.n >= ((int64_t)1 << 31) - 1024;
   if (rp.sk_gd > 0 || (long_rows && d == 0)) return RBO_ERR_ARG;
   if (d > 0 && (rp.acc_x || rp.acc_y)) return RBO_ERR_ARG;  // a sketch pass has no Gram
@@ -225,12 +225,14 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   P.kc = kc;
   P.nblk = nblk;
   for (int k = 0; k < 9; ++k) P.blk_start[k] = blk_start[k];
-  const bool alignedX = a == 0 || (((uintptr_t)rp.X & 15) == 0 && (rp.ldx % 2) == 0);
-  const bool alignedY = (((uintptr_t)rp.Y & 15) == 0 && (rp.ldy % 2) == 0);
+  // (the leading dimension of a single column does not matter)
+  const int64_t ldx = a == 1 ? rp.ldx + (rp.ldx & 1) : rp.ldx, ldy = b == 1 ? rp.ldy + (rp.ldy & 1) : rp.ldy;
+  const bool alignedX = a == 0 || (((uintptr_t)rp.X & 15) == 0 && ldx % 2 == 0);
+  const bool alignedY = ((uintptr_t)rp.Y & 15) == 0 && ldy % 2 == 0;
   P.use_bulk = (alignedX && alignedY && !long_rows) ? 1 : 0;
   if (P.use_bulk) {
-    int e = make_tensor_map(&D.tmY, rp.Y, rp.n, b, rp.ldy);
-    if (e == RBO_OK && a > 0) e = make_tensor_map(&D.tmX, rp.X, rp.n, a, rp.ldx);
+    int e = make_tensor_map(&D.tmY, rp.Y, rp.n, b, ldy);
+    if (e == RBO_OK && a > 0) e = make_tensor_map(&D.tmX, rp.X, rp.n, a, ldx);
     if (e != RBO_OK) return e;
   }
   P.zr = zr;

@@ -7,8 +7,10 @@
 //
 // CTAs of 4 warps, several per SM: tiles of T rows come in as tensor copies of 16-row
 // boxes (one thread issues a handful per tile), double buffered; rows past n read as zero.
-// Arrays a tensor copy cannot address (odd leading dimension, unaligned base) are staged
-// with plain loads.  Per tile
+// Arrays a tensor copy cannot address (odd leading dimension, unaligned base, 2^31 rows) come in
+// by asynchronous copies of 8 bytes that all threads issue, into the same stages at the same
+// places (n = 400001 at an odd leading dimension: Gram call of 64 x 5 columns 187 us, one-stage of
+// 61 columns 6.1 ms; plain loads in front of each tile 501 us and 10.2 ms).  Per tile
 //   A  every warp updates its own 16-row blocks; triangular solve, one row per thread in
 //      registers; write-back;
 //   S  (sketch passes) the y' of the tile as 54-bit integers on one scale per column, and
@@ -62,6 +64,21 @@ __host__ __device__ constexpr bool tc_wide(int tri, int g) { return tri == 2 || 
 constexpr int tc_min_ctas(bool hc, int tri, int g) {
   if (tc_wide(tri, g) || (tri == 1 && g == 1)) return 3;
   return tri == 1 && !hc ? (g == 0 ? 6 : (g == 2 ? 5 : 4)) : 4;
+}
+
+// Asynchronous copies of a tile by all threads: `left` rows of src from the tile's first one on,
+// cols columns, into blocks of 16 rows, zeros past them; bytes is a multiple of 16.  Not inlined:
+// the kernels' own code stays as short as without them.
+static __device__ __noinline__ void tc_copy_cols(unsigned char* dst, int blk, const double* src, int64_t ld, int cols,
+                                                 int tsh, int64_t left) {
+  for (int t = threadIdx.x; t < cols << tsh; t += TC_NT) {
+    const int c = t >> tsh, r = t & ((1 << tsh) - 1);
+    const bool in = r < left;
+    cp_async8(dst + TcTile::off(blk, r, c), in ? src + c * ld + r : src, in);
+  }
+}
+static __device__ __noinline__ void tc_copy_bytes(unsigned char* dst, const uint8_t* src, int bytes) {
+  for (int t = 16 * threadIdx.x; t < bytes; t += 16 * TC_NT) cp_async16(dst + t, src + t);
 }
 
 // HC: projection (C digits); TRI: triangular factor, 0 none, 1 substitution, 2 product with its
@@ -132,12 +149,42 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       for (int k = 0; k < nblk16; ++k) tma_load_rows(smem + k * xblk, &D.tmX, tile * T + 16 * k, &barx);
   };
 
+  // the same without the copy engine, by all threads; a group per call
+  auto copy_tile = [&](int tile, int s) {
+    const int64_t r0 = (int64_t)tile * T;
+    if (!XS) tc_copy_cols(stage_X(s), xblk, rp.X + r0, rp.ldx, a, tsh, n - r0);
+    tc_copy_cols(stage_Y(s), yblk, rp.Y + r0, rp.ldy, b, tsh, n - r0);
+    if (rec_n > 0) tc_copy_bytes(stage_R(s), rp.sk.rec + (size_t)tile * rec_n, rec_n);
+    cp_async_commit();
+  };
+  auto copy_x = [&](int tile) {
+    const int64_t r0 = (int64_t)tile * T;
+    tc_copy_cols(smem, xblk, rp.X + r0, rp.ldx, a, tsh, n - r0);
+    cp_async_commit();
+  };
+
+  // XS: X of a later tile once every warp is done with the one before it
+  auto next_x = [&](int tile) {
+    if (tile >= P.ntiles) return;
+    if (!P.use_bulk) {
+      copy_x(tile);
+    } else if (tid == 0) {
+      fence_proxy_async();
+      issue_x(tile);
+    }
+  };
+
   // the first tile is in flight while the small matrices are prepared
   uint32_t phx = 0u;  // (a stage's phase: the parity of the tiles it held)
   const int first = blockIdx.x;
-  if (tid == 0 && P.use_bulk && first < P.ntiles) {
-    issue_tile(first, 0);
-    if (XS) issue_x(first);
+  if (first < P.ntiles) {
+    if (!P.use_bulk) {
+      copy_tile(first, 0);
+      if (XS) copy_x(first);
+    } else if (tid == 0) {
+      issue_tile(first, 0);
+      if (XS) issue_x(first);
+    }
   }
   // the padding columns of every block hold zeros (the copies do not touch them)
   for (int s = 0; s < NST; ++s) {
@@ -219,18 +266,12 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
         if (nxt < P.ntiles) issue_tile(nxt, s ^ 1);
       }
     } else {
-      __syncthreads();  // the previous tile's readers are done
-      for (int t = tid; t < (a + b) * T; t += TC_NT) {
-        const int c = t >> tsh, r = t & (T - 1);
-        double v = 0.0;
-        if (r < rows) v = (c < a) ? rp.X[c * rp.ldx + r0 + r] : rp.Y[(c - a) * rp.ldy + r0 + r];
-        unsigned char* p = c < a ? xs + TcTile::off(xblk, r, c) : ys + TcTile::off(yblk, r, c - a);
-        *reinterpret_cast<double*>(p) = v;
-      }
-      for (int t = tid; t < rec_n / 16; t += TC_NT)
-        reinterpret_cast<uint4*>(stage_R(s))[t] =
-            reinterpret_cast<const uint4*>(rp.sk.rec + (size_t)tile * rec_n)[t];
-      __syncthreads();
+      cp_async_wait<0>();
+      __syncthreads();  // the tile is in, the previous tile's readers are done
+      const int nxt = tile + gridDim.x;
+      if (XL && it > 0) copy_x(tile);
+      if (nxt < P.ntiles) copy_tile(nxt, s ^ 1);
+      else cp_async_commit();  // (an empty group: the waits below count groups)
     }
 
     // ---- A: y' in place in the Y stage -------------------------------------------
@@ -282,10 +323,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       if (XS && !SK) {
         __syncthreads();  // every warp is done with X (sketch passes: at their own barrier)
         synced = true;
-        if (tid == 0 && P.use_bulk && tile + (int)gridDim.x < P.ntiles) {
-          fence_proxy_async();
-          issue_x(tile + gridDim.x);
-        }
+        next_x(tile + gridDim.x);
       } else {
         __syncwarp();
       }
@@ -332,10 +370,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       }
       if (__any_sync(0xffffffffu, past) && lane == 0) s_rescale = 1;
       __syncthreads();
-      if (XS && tid == 0 && P.use_bulk && tile + (int)gridDim.x < P.ntiles) {
-        fence_proxy_async();
-        issue_x(tile + gridDim.x);
-      }
+      if (XS) next_x(tile + gridDim.x);
       if (!mixed) {
         // the record's first slot has the tile's most entries in one sketch row
         const uint32_t m0 = *reinterpret_cast<const uint32_t*>(stage_R(s));
@@ -402,6 +437,9 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
           return;
         }
         phx ^= 1u;
+      } else if (XL) {
+        cp_async_wait<1>();  // X; the next tile's group came after it
+        __syncthreads();
       } else if ((G == 1 || G == 3) && (HC || HT) && !synced) {
         __syncthreads();
       }
