@@ -485,6 +485,27 @@ static int occupancy(int smem) {
   return nb;
 }
 
+// Whether the float64 pipe does a pass (without a sketch) sooner than the tensor cores.  Its time
+// goes by the FMAs of a row, that of the digits by the tiles of 16 x 8 products, however few of
+// their columns are used; in FMAs a tile of a general Gram costs 24, the Gram of at most 8
+// columns of Y' 14, the update of up to 16 columns X 28 and of each 16 more 14 (triangular solves
+// are the same in both).  4 million rows, float64 pipe / digits: Gram 1 x 5 78 / 198 us, 5 x 4 175 /
+// 200, 10 x 3 250 / 248, 6 x 5 237 / 199; solve + Gram of 3 columns 160 / 165 us, of 4 223 / 197;
+// update + Gram p = 1, b = 5 303 / 387 us, p = 10, b = 3 360 / 374, p = 9, b = 4 430 / 376; a solve
+// alone, b = 1 35 / 45 us, b = 2 53 / 50.  Beyond 72 columns a tile of rows leaves the float64 kernel
+// fewer than three CTAs per SM (128 x 1: 285 / 231 us at 400000 rows), and fewer rows than one of
+// its tiles of 512 per SM are served sooner in short tiles (one-stage of 7 single columns, 20000
+// rows 783 / 723 us, 40000 788 / 786, 80000 823 / 904, 10^6 1815 / 2730).
+static bool narrow_pass(const RowPass& rp, int num_sms) {
+  const int a = rp.C || rp.acc_x ? rp.a : 0, b = rp.b, ax = rp.acc_x ? a : 0;
+  if (b > 8 || a + b > 72 || rp.n < 512 * (int64_t)num_sms) return false;
+  const int zr = ax + (rp.acc_y ? b : 0), xt = (a + 15) / 16;
+  if (!rp.C && zr == 0) return b == 1;
+  const int fmas = (rp.C ? a * b : 0) + zr * b;
+  const int gram = zr == 0 ? 0 : (ax == 0 ? 14 : 24 * ((zr + 15) / 16));
+  return fmas <= (rp.C ? 28 + 14 * (xt - 1) : 0) + gram;
+}
+
 int rowpass_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* launches) {
   RowPass rp = rpin;
   if (rp.n <= 0 || rp.b <= 0 || rp.b > 64 || rp.a < 0 || rp.a > 128) return RBO_ERR_ARG;
@@ -532,9 +553,9 @@ int rowpass_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* launche
       return RBO_ERR_ARG;
     return rowpass_tc_launch(rp, ar, st, launches, sm_count());
   }
-  // float64 passes: contractions on the tensor cores (a Gaussian sketch adds generated Z
-  // rows, which only the kernel here has)
-  if (arith == 0 && rp.sk_gd == 0) {
+  // float64 passes: contractions on the tensor cores, unless they are too narrow for that (a
+  // Gaussian sketch adds generated Z rows, which only the kernel here has)
+  if (arith == 0 && rp.sk_gd == 0 && !narrow_pass(rp, sm_count())) {
     const int e = rowpass_tc_launch(rp, ar, st, launches, sm_count());
     if (e != RBO_ERR_ARG) return e;
   }
