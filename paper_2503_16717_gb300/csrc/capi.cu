@@ -272,9 +272,13 @@ int rbo_sketch_apply(rbo_sketch sk, int64_t n, int32_t k, const double* W, int64
   r.n = n; r.Y = const_cast<double*>(W); r.ldy = ldw; r.b = k;
   set_sketch(r, c);
   r.mixed = precision == RBO_PREC_MIXED ? 1 : 0;
-  r.epi.op = EPI_SKETCH_OUT; r.epi.out_sk = dout;
+  const bool cg = sk->type == RBO_SKETCH_COUNT_GAUSS;
+  r.epi.op = cg ? EPI_GROUPS : EPI_SKETCH_OUT; r.epi.out_sk = dout;
   int launches = 0;
   if ((e = rowpass_launch(r, ar, st, &launches))) return e;
+  if (cg && (e = count_gauss_launch(ar->gpart, ar->ngroups, c.d_inner, c.d, k, c.seed, c.cg_in, dout, ar->status, st,
+                                    &launches)))
+    return e;
   if (cudaMemcpyAsync(out, dout, (size_t)sk->d * k * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return RBO_ERR_CUDA;
   return finish_status(ar, st, nullptr);

@@ -33,7 +33,8 @@ size_t orth_ctx_bytes(int pmax, int kmax, int ks, int d, int64_t n, int zeta, in
   sched_shape(type, d, d_inner, zeta, &ds, &zs);
   const size_t tab =
       (d > 0 && ds > 0) ? sketch_sched_bytes(n, rowpass_sketch_T(pmax, ks, ds, zs), ds, zs) + 256 : 0;
-  return (2 * pk + 8 * kk + dd + pk + kk) * 8 + 18 * 256 + tab;
+  const size_t cg = type == RBO_SKETCH_COUNT_GAUSS && d > 0 ? (size_t)(d + d_inner) * kmax : 0;
+  return (2 * pk + 8 * kk + dd + pk + kk + cg) * 8 + 20 * 256 + tab;
 }
 
 void set_sketch(RowPass& r, const OrthCtx& c) {
@@ -41,7 +42,7 @@ void set_sketch(RowPass& r, const OrthCtx& c) {
   if (c.sk_type == RBO_SKETCH_GAUSSIAN) {
     r.sk_gd = c.d;
   } else if (c.sk_type == RBO_SKETCH_COUNT_GAUSS) {
-    r.sk_d = c.d_inner; r.sk_zeta = 1; r.sk = c.sk; r.sk_cg = c.d;
+    r.sk_d = c.d_inner; r.sk_zeta = 1; r.sk = c.sk;
   } else {
     r.sk_d = c.d; r.sk_zeta = c.zeta; r.sk = c.sk;
   }
@@ -71,6 +72,11 @@ int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int ks, int64_t n) {
   c.tmp = (double*)c.ar->take((pk + kk) * 8);
   if (!c.C1 || !c.C2 || !c.Rh || !c.Rp || !c.R2 || !c.T || !c.GB || !c.RpInv || !c.R2Inv || !c.qs || !c.tmp)
     return RBO_ERR_NOMEM;
+  if (c.d > 0 && c.sk_type == RBO_SKETCH_COUNT_GAUSS) {
+    c.cg_in = (double*)c.ar->take((size_t)c.d_inner * kmax * 8);
+    c.cg_out = (double*)c.ar->take((size_t)c.d * kmax * 8);
+    if (!c.cg_in || !c.cg_out) return RBO_ERR_NOMEM;
+  }
   c.sk = SketchSched();
   int ds = 0, zs = 0;
   sched_shape(c.sk_type, c.d, c.d_inner, c.zeta, &ds, &zs);
@@ -95,6 +101,32 @@ int orth_ctx_alloc(OrthCtx& c, int pmax, int kmax, int ks, int64_t n) {
     int _e = (x);              \
     if (_e != RBO_OK) return _e; \
   } while (0)
+
+// A pass r with the call's sketch, then the step `epi` (EPI_HH or EPI_SKB2) on the sketch: for
+// sparse-sign and Count-Gauss in kernels of their own where the cluster kernel serves the shape,
+// for Count-Gauss after the product with G; else in the last CTA of the pass.
+static int sketched_pass(OrthCtx& c, RowPass& r, const Epilogue& epi) {
+  const int k = r.b, poff = epi.op == EPI_SKB2 ? epi.poff : 0;
+  const bool cg = c.sk_type == RBO_SKETCH_COUNT_GAUSS;
+  const bool cluster = c.sk_type != RBO_SKETCH_GAUSSIAN && skb2_supported(c.d, k, poff);
+  set_sketch(r, c);
+  r.mixed = c.mixed;
+  r.epi = epi;
+  if (cluster || cg) r.epi.op = EPI_GROUPS;
+  RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
+  const double* v = c.ar->gpart;
+  int nparts = c.ar->ngroups;
+  if (cg) {
+    RBO_TRY(count_gauss_launch(v, nparts, c.d_inner, c.d, k, c.seed, c.cg_in, c.cg_out, c.ar->status, c.st, &c.launches));
+    v = c.cg_out;
+    nparts = 1;
+    if (!cluster) return sketch_epilogue_launch(epi, v, c.d, k, c.ar->status, c.st, &c.launches);
+  }
+  if (!cluster) return RBO_OK;
+  const bool hh = epi.op == EPI_HH;
+  return skb2_launch(v, nparts, (int64_t)c.d * k, hh ? nullptr : epi.qs, hh ? epi.out_r : epi.T, c.d, k,
+                     hh ? k : epi.K, poff, epi.stage, epi.block, c.ar->status, c.st, &c.launches);
+}
 
 int normalise_column(OrthCtx& c, int64_t n, double* v, double* Rdev, int ldR, int col0) {
   const int64_t ldeven = (n + 1) & ~int64_t(1);  // only column 0 is used
@@ -145,27 +177,21 @@ int one_stage_block(OrthCtx& c, int64_t n, const double* Q, int64_t ldq, int p, 
     RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
   }
   // P2: W = W - Q C1, then sketch -> R_hat (or Gram -> chol for CholQR2)
-  bool cluster = false;  // the Householder factor in its own cluster kernel
   {
     RowPass r;
     r.df64 = c.df64; r.ozaki = c.ozaki; r.tag = 2;
     r.n = n; r.X = Q; r.ldx = ldq; r.a = p; r.Y = W; r.ldy = ldw; r.b = k;
     if (p > 0) { r.C = c.C1; r.write_y = 1; }
+    Epilogue e;
+    e.op = rand ? EPI_HH : EPI_CHOL; e.out_r = c.Rh; e.stage = RBO_STAGE_INTRA; e.block = blk;
     if (rand) {
-      set_sketch(r, c);
-      r.mixed = c.mixed;
-      cluster = c.sk_type == RBO_SKETCH_SPARSE_SIGN && skb2_supported(c.d, k, 0);
-      r.epi.op = cluster ? EPI_GROUPS : EPI_HH;
-      r.epi.out_r = c.Rh; r.epi.stage = RBO_STAGE_INTRA; r.epi.block = blk;
+      RBO_TRY(sketched_pass(c, r, e));
     } else {
       r.acc_y = 1;
-      r.epi.op = EPI_CHOL; r.epi.out_r = c.Rh; r.epi.stage = RBO_STAGE_INTRA; r.epi.block = blk;
+      r.epi = e;
+      RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
     }
-    RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
   }
-  if (cluster)
-    RBO_TRY(skb2_launch(c.ar->gpart, c.ar->ngroups, (int64_t)c.d * k, nullptr, c.Rh, c.d, k, k, 0, RBO_STAGE_INTRA,
-                        blk, c.ar->status, c.st, &c.launches));
   // P3: W = W R_hat^{-1}; R' = chol(W^T W)
   {
     RowPass r;
@@ -265,19 +291,9 @@ int bigpanel_add(OrthCtx& c, BigPanel& bp, int k) {
     r.df64 = c.df64; r.ozaki = c.ozaki; r.tag = 8;
     r.n = bp.n; r.X = bp.Q; r.ldx = bp.ldq; r.a = P; r.Y = W; r.ldy = bp.ldv; r.b = k;
     if (P > 0) { r.C = c.C1 + (size_t)cols * P; r.ldc = P; r.write_y = 1; }
-    set_sketch(r, c);
-    r.mixed = c.mixed;
-    const bool cluster = c.sk_type == RBO_SKETCH_SPARSE_SIGN && skb2_supported(c.d, k, cols);
-    if (cluster) {
-      r.epi.op = EPI_GROUPS;
-    } else {
-      r.epi.op = EPI_SKB2; r.epi.qs = c.qs; r.epi.T = c.T; r.epi.K = K; r.epi.poff = cols;
-    }
-    r.epi.stage = RBO_STAGE_BIGPANEL; r.epi.block = bp.blk;
-    RBO_TRY(rowpass_launch(r, c.ar, c.st, &c.launches));
-    if (cluster)
-      RBO_TRY(skb2_launch(c.ar->gpart, c.ar->ngroups, (int64_t)c.d * k, c.qs, c.T, c.d, k, K, cols,
-                          RBO_STAGE_BIGPANEL, bp.blk, c.ar->status, c.st, &c.launches));
+    Epilogue e;
+    e.op = EPI_SKB2; e.qs = c.qs; e.T = c.T; e.K = K; e.poff = cols; e.stage = RBO_STAGE_BIGPANEL; e.block = bp.blk;
+    RBO_TRY(sketched_pass(c, r, e));
   }
   {
     RowPass r;

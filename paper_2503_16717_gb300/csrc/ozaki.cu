@@ -709,7 +709,7 @@ int g_oz_smem_set[64] = {};
 }  // namespace
 
 bool ozaki_gram_supported(const RowPass& rp) {
-  if (!rp.ozaki || rp.C || rp.Tri || rp.write_y || rp.sk_d > 0 || rp.sk_gd > 0 || rp.sk_cg > 0 ||
+  if (!rp.ozaki || rp.C || rp.Tri || rp.write_y || rp.sk_d > 0 || rp.sk_gd > 0 ||
       rp.mixed || rp.df64)
     return false;
   if (!rp.acc_x && !rp.acc_y) return false;

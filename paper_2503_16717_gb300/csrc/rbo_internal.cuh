@@ -158,8 +158,6 @@ struct RowPass {
   int sk_d = 0, sk_zeta = 0; uint64_t sk_seed = 0;  // accumulate S Y' (d x b), sparse-sign
   SketchSched sk;                // sketch schedule of the n rows (required with sk_d > 0)
   int sk_gd = 0;                 // Gaussian sketch rows (entries generated per tile; Z rows)
-  int sk_cg = 0;                 // Count-Gauss: final rows (Gaussian stage in the epilogue;
-                                 // sk_d is then the Count stage, zeta 1)
   int mixed = 0;                 // float32 accumulation of X^T Y' and S Y'
   int df64 = 0;                  // float32-pair arithmetic for the Gram (and small projections)
   int ozaki = 0;                 // Gram on the tensor cores (exact digit products, ozaki.cu):
@@ -193,6 +191,14 @@ int rowpass_tc_launch(const RowPass& rp, Arena* ar, cudaStream_t st, int* launch
 bool skb2_supported(int d, int k, int poff);
 int skb2_launch(const double* v, int nparts, int64_t stride, double* qs, double* T, int d, int k, int K, int poff,
                 int stage, int block, DevStatus* status, cudaStream_t st, int* launches);
+// out (d x k) = G times the sum of the nparts partials of a Count stage (di x k each); S: di x k
+// scratch (count_gauss.cu)
+int count_gauss_launch(const double* part, int nparts, int di, int d, int k, uint64_t seed, double* S, double* out,
+                       DevStatus* status, cudaStream_t st, int* launches);
+// Epilogue (EPI_HH or EPI_SKB2) on a finished sketch v (d x k); RBO_ERR_ARG when it does not fit
+// a CTA's shared memory
+int sketch_epilogue_launch(const Epilogue& epi, const double* v, int d, int k, DevStatus* status, cudaStream_t st,
+                           int* launches);
 
 // Sketch schedule: S restricted to each tile of T basis rows, transposed once per
 // call so that the row pass needs neither hashing nor a scatter with conflicts.
@@ -288,6 +294,7 @@ struct OrthCtx {
   double *T = nullptr, *qs = nullptr, *GB = nullptr;
   double *RpInv = nullptr, *R2Inv = nullptr;  // inverses of Rp and R2 (two-stage)
   double* tmp = nullptr;  // pmax*kmax + kmax*kmax doubles for small staging
+  double *cg_in = nullptr, *cg_out = nullptr;  // Count-Gauss: Count stage and product of a panel
 };
 // Take the small buffers from the arena for blocks with up to pmax previous columns
 // and kmax columns per block (K for two-stage).  Returns RBO_OK or RBO_ERR_NOMEM.

@@ -517,7 +517,7 @@ int rowpass_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* launche
   if (rp.ozaki && ozaki_gram_supported(rp) && (rp.ozaki == 2 || ozaki_gram_pays(rp)))
     return ozaki_gram_launch(rp, ar, st, launches, sm_count());
   if (rp.sk_d > DMAX || rp.sk_zeta > ZMAX) return RBO_ERR_ARG;
-  if (rp.sk_gd < 0 || rp.sk_gd > 256 || rp.sk_cg < 0 || rp.sk_cg > DMAX) return RBO_ERR_ARG;
+  if (rp.sk_gd < 0 || rp.sk_gd > 256) return RBO_ERR_ARG;
   if (rp.sk_gd > 0 && rp.sk_d > 0) return RBO_ERR_ARG;
   const int zr = rp.sk_gd + (rp.acc_x ? rp.a : 0) + (rp.acc_y ? rp.b : 0);
   const int no = zr * rp.b;

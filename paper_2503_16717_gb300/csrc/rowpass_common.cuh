@@ -124,28 +124,16 @@ static __device__ void assemble(const Epilogue& e, const double* R2, int k, doub
   __syncthreads();
 }
 
-// Rows of the sketch S Y' a pass produces (after the Count-Gauss Gaussian stage).
-__host__ __device__ inline int sketch_rows(const RowPass& rp) {
-  return rp.sk_gd > 0 ? rp.sk_gd : (rp.sk_cg > 0 ? rp.sk_cg : rp.sk_d);
-}
+// Rows of the sketch S Y' a pass produces.
+__host__ __device__ inline int sketch_rows(const RowPass& rp) { return rp.sk_gd > 0 ? rp.sk_gd : rp.sk_d; }
 
 // The reduced sketch S Y' (sketch_rows x b, column-major) into A: sparse-sign from
-// the scattered part of the partial; Gaussian from its Z rows; Count-Gauss as G times
-// the scattered Count stage, G generated here (float32 Box-Muller, as in the tiles).
+// the scattered part of the partial; Gaussian from its Z rows.
 static __device__ void load_sketch(const PassDev& P, const double* red, double* A) {
   const RowPass& rp = P.p;
   const int b = rp.b, d = sketch_rows(rp);
   if (rp.sk_gd > 0) {
     for (int t = threadIdx.x; t < d * b; t += blockDim.x) A[t] = red[(t % d) * b + t / d];
-  } else if (rp.sk_cg > 0) {
-    const int di = rp.sk_d;
-    for (int t = threadIdx.x; t < d * b; t += blockDim.x) {
-      const int k = t % d, c = t / d;
-      double s = 0.0;
-      for (int j = 0; j < di; ++j)
-        s = fma((double)gauss_entry(rp.sk_seed, (uint64_t)j, k, d), red[P.no + j + (size_t)c * di], s);
-      A[t] = s;
-    }
   } else {
     for (int t = threadIdx.x; t < d * b; t += blockDim.x) A[t] = red[P.no + t];
   }
