@@ -16,10 +16,13 @@
 //   S  (sketch passes) the y' of the tile as 54-bit integers on one scale per column, and
 //      their signed sums per sketch row from the tile's schedule record: the thread that
 //      owns a slot of the record sums the slot's entries and adds them to the row's 64-bit
-//      integer accumulators.  A column's scale only grows (the accumulators are shifted
-//      when a tile raises it) and the accumulators enter the CTA's float64 partial before a
-//      sketch row can have summed 384 entries (a few thousand rows, by the tiles' largest
-//      counts), so that a tile costs no float64 operation per sketch row;
+//      integer accumulators.  A column's scale follows its tiles: up when a value is past it,
+//      down when a tile's values are all 2^SK_FAR below it.  The accumulators enter the CTA's
+//      float64 partial when a scale falls or rises by more than SK_RISE, and before a sketch row
+//      can have summed 384 entries (a few thousand rows, by the tiles' largest counts), so that
+//      most tiles cost no float64 operation per sketch row, and so that a value is off by at most
+//      2^(SK_FAR - 1 + SK_RISE - 54) of the largest of its own tile, 2^-53 where the tiles of a
+//      column are alike;
 //   B  the Gram items, (16 Z columns) x (8 Y' columns) x (a chunk of kc rows), are dealt
 //      to the warps; an item always goes to the same warp, which keeps its float64 sums
 //      in its own shared-memory slots.
@@ -46,6 +49,8 @@ namespace rbo {
 
 constexpr int TC_NT = 128;
 constexpr int TC_NW = TC_NT / 32;
+constexpr int SK_FAR = 6;   // sketch scales: 16 rows of like values nearly never lie all below 2^-6
+constexpr int SK_RISE = 3;  // of the largest seen; a scale with room of one bit rises by 2 at least
 
 struct TcDev {
   CUtensorMap tmX, tmY;
@@ -81,6 +86,94 @@ static __device__ __noinline__ void tc_copy_bytes(unsigned char* dst, const uint
   for (int t = 16 * threadIdx.x; t < bytes; t += 16 * TC_NT) cp_async16(dst + t, src + t);
 }
 
+// Sketch sums into the CTA's partial (= for the first time, then +=), each thread its own entries;
+// the sums start again from zero.  (This and the next function are not inlined: they run every
+// few dozen tiles, and a pass with them in its loop takes 5 % longer.)
+static __device__ __noinline__ void sk_flush(long long* ska, int d, int b, const int* scale, const bool* nan,
+                                             double* part, bool first, bool mixed) {
+  for (int t = threadIdx.x; t < d * b; t += TC_NT) {
+    const int c = t / d;
+    if (mixed) {
+      part[t] = (double)reinterpret_cast<const float*>(ska)[t];
+      continue;
+    }
+    const int sc = scale[c];
+    double v = (double)ska[t];
+    v = sc >= 60 ? v * __hiloint2double((sc - 53) << 20, 0) : scalbn(v, sc - 1076);
+    if (nan[c]) v = __longlong_as_double(0x7FF8000000000000LL);
+    part[t] = first ? v : part[t] + v;
+    ska[t] = 0;
+  }
+}
+struct SkTile {
+  const unsigned char* ys;
+  int yblk, T, tsh, d, b;
+  long long *ska, *skf;
+  double* part;
+  int* scale;     // per column: exponent field of the scale,
+  short* base;    // of the scale at the last flush,
+  short* now;     // of the next scale
+  bool* nan;      // the column has a value that is not finite
+  int* rescale;   // set when a warp found a value past its scale or 16 far below it
+  bool first;
+};
+// Scales for this tile and its values on them; true when the sums went into the partial.  Whole
+// block, all threads past the conversion of the tile; ends with a barrier.
+static __device__ __noinline__ bool sk_rescale(const SkTile& S, bool full) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = S.b, d = S.d;
+  const bool rescale = *S.rescale != 0;
+  bool change = false, flush = full;
+  if (rescale) {
+    for (int c = warp; c < b; c += TC_NW) {
+      int ex = 0;
+      for (int r = lane; r < S.T; r += 32)
+        ex = max(ex, (__double2hiint(tc_ld(S.ys + TcTile::off(S.yblk, r, c))) >> 20) & 0x7FF);
+      ex = __reduce_max_sync(0xffffffffu, ex);
+      if (lane == 0) {
+        // (room to grow, but never up to the exponent field of Inf and NaN, which must stay past
+        // every scale)
+        const int old = S.scale[c];
+        if (ex == 0x7FF) S.nan[c] = true;
+        S.now[c] = (short)(ex != 0x7FF && ex > 0 && (ex > old || ex + SK_FAR <= old) ? min(ex + 1, 0x7FE) : old);
+      }
+    }
+    __syncthreads();
+    for (int c = lane; c < b; c += 32) {
+      const int old = S.scale[c], now = S.now[c];
+      change = change || now != old;
+      flush = flush || now < old || (old > 0 && now > S.base[c] + SK_RISE);
+    }
+    change = __any_sync(0xffffffffu, change);  // (the same in every warp)
+    flush = __any_sync(0xffffffffu, flush);
+  }
+  if (flush) {  // sums on the scales they were formed with
+    sk_flush(S.ska, d, b, S.scale, S.nan, S.part, S.first, false);
+  } else if (change) {  // small rises: the sums move along
+    for (int t = tid; t < d * b; t += TC_NT) {
+      const int k = S.now[t / d] - S.scale[t / d];
+      if (k > 0 && S.ska[t] != 0) S.ska[t] = (S.ska[t] + (1LL << (k - 1))) >> k;
+    }
+  }
+  __syncthreads();  // scales read above
+  if (tid < b) {
+    if (change) S.scale[tid] = S.now[tid];
+    if (flush || S.base[tid] == 0) S.base[tid] = (short)S.scale[tid];
+  }
+  if (tid == 0) *S.rescale = 0;
+  if (change) {
+    __syncthreads();
+    for (int t = tid; t < S.T * b; t += TC_NT) {
+      const int c = t >> S.tsh, r = t & (S.T - 1);
+      const double v = tc_ld(S.ys + TcTile::off(S.yblk, r, c));
+      const long long f = S.nan[c] ? 0 : fx_round54(v, S.scale[c]);
+      S.skf[2 * r * b + c] = f;
+      S.skf[(2 * r + 1) * b + c] = -f;
+    }
+  }
+  __syncthreads();
+  return flush;
+}
+
 // HC: projection (C digits); TRI: triangular factor, 0 none, 1 substitution, 2 product with its
 // inverse (digits); G: Gram, 0 none, 1 general, 2 of at most
 // 8 columns of Y' alone, 3 of more columns of Y' alone after an update; SK: sparse sketch (no triangle, no Gram).  Each kind of pass is its
@@ -102,7 +195,9 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   __shared__ int s_flag;
   __shared__ int s_last;
   __shared__ int s_bad;
-  __shared__ int s_scale[64], s_shift[64], s_nan[64], s_rescale;  // sketch: per column
+  __shared__ int s_scale[64], s_rescale;  // sketch: per column
+  __shared__ short s_base[64], s_new[64];
+  __shared__ bool s_nan[64];
   const PassDev& P = D.P;
   const RowPass& rp = P.p;
   if (read_code(P.status) != 0) return;
@@ -208,7 +303,10 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
     for (int t = tid; t < P.items * 128 * NT; t += TC_NT) accs[t] = 0.0;
   if constexpr (SK) {
     for (int t = tid; t < d * b; t += TC_NT) ska[t] = 0;  // (all-zero bits also as float32 pairs)
-    if (tid < 64) s_scale[tid] = s_shift[tid] = s_nan[tid] = 0;
+    if (tid < 64) {
+      s_scale[tid] = s_base[tid] = 0;
+      s_nan[tid] = false;
+    }
     if (tid == 0) s_rescale = 0;
   }
   if (HC && P.c_digits) tc_build_c(rp.C, ldc, a, b, cf, ec, &s_bad);
@@ -219,24 +317,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   const int rsh = max(4, tsh - 2), rpw = 1 << rsh, rw = warp * rpw, re = min(rw + rpw, T);
   double* mypart = P.L > 0 ? P.partials + (size_t)blockIdx.x * P.L : nullptr;
   const bool mixed = SK && rp.mixed;  // float32 values and sums of the sketch
-  // sketch sums into the partial: mypart = / += (each thread its own entries)
-  bool sk_first = true;
-  auto sk_flush = [&]() {
-    for (int t = tid; t < d * b; t += TC_NT) {
-      const int c = t / d;
-      if (mixed) {
-        mypart[t] = (double)reinterpret_cast<const float*>(ska)[t];
-        continue;
-      }
-      const int sc = s_scale[c];
-      double v = (double)ska[t];
-      v = sc >= 60 ? v * __hiloint2double((sc - 53) << 20, 0) : scalbn(v, sc - 1076);
-      if (s_nan[c]) v = __longlong_as_double(0x7FF8000000000000LL);
-      mypart[t] = sk_first ? v : mypart[t] + v;
-      ska[t] = 0;
-    }
-    sk_first = false;
-  };
+  bool sk_first = true;  // nothing in the partial yet
   int sk_cnt = 0;  // entries a sketch row can have summed since the last flush
   const int q = P.blk_start[P.nblk];  // Gram items per chunk
 
@@ -350,68 +431,51 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
 
     // ---- S: sketch sums ---------------------------------------------------------------
     if constexpr (SK) {
-      // every warp converts its rows with the columns' current scales; only a tile with a
-      // value past a scale (or not finite) takes the block-wide path below
-      bool past = false;
-      for (int t = lane; t < (re - rw) * b; t += 32) {
-        const int r = rw + (t & (rpw - 1)), c = t >> rsh;
-        const double v = tc_ld(ys + TcTile::off(yblk, r, c));
+      // Every warp converts its 16 rows with the columns' current scales, two columns at a time;
+      // only a tile with a value past a scale (or not finite), or with 16 rows of a column all
+      // far below it, takes the block-wide path below.
+      bool past = false, low = false;
+      for (int t0 = 0; t0 < (re - rw) * b; t0 += 32) {
+        const int t = t0 + lane, r = rw + (t & 15), c = t >> 4;
+        const bool in = c < b;
+        const double v = in ? tc_ld(ys + TcTile::off(yblk, r, c)) : 0.0;
         if (mixed) {
-          const float f = f64_to_f32_int(v);
-          reinterpret_cast<float*>(skf)[2 * r * b + c] = f;
-          reinterpret_cast<float*>(skf)[(2 * r + 1) * b + c] = -f;
+          if (in) {
+            const float f = f64_to_f32_int(v);
+            reinterpret_cast<float*>(skf)[2 * r * b + c] = f;
+            reinterpret_cast<float*>(skf)[(2 * r + 1) * b + c] = -f;
+          }
         } else {
-          const int sc = s_scale[c];
-          past = past || ((__double2hiint(v) >> 20) & 0x7FF) > sc;
-          const long long f = fx_round54(v, sc);
-          skf[2 * r * b + c] = f;
-          skf[(2 * r + 1) * b + c] = -f;
+          const int sc = in ? s_scale[c] : 0, ex = (__double2hiint(v) >> 20) & 0x7FF;
+          past = past || ex > sc;
+          const unsigned near = __ballot_sync(0xffffffffu, ex + SK_FAR > sc);
+          if (near < 0x10000u || (near & 0xFFFFu) == 0u) {
+            const unsigned some = __ballot_sync(0xffffffffu, ex > 0);
+            low = low || (near < 0x10000u && some >= 0x10000u) || ((near & 0xFFFFu) == 0u && (some & 0xFFFFu) != 0u);
+          }
+          if (in) {
+            const long long f = fx_round54(v, sc);
+            skf[2 * r * b + c] = f;
+            skf[(2 * r + 1) * b + c] = -f;
+          }
         }
       }
-      if (__any_sync(0xffffffffu, past) && lane == 0) s_rescale = 1;
+      if ((__any_sync(0xffffffffu, past) || low) && lane == 0) s_rescale = 1;
       __syncthreads();
       if (XS) next_x(tile + gridDim.x);
       if (!mixed) {
         // the record's first slot has the tile's most entries in one sketch row
         const uint32_t m0 = *reinterpret_cast<const uint32_t*>(stage_R(s));
         const int most = m0 == 0xFFFFFFFFu ? 0 : (int)(m0 >> 23);
-        const bool rescale = s_rescale != 0, full = sk_cnt + most > 384;  // 2^54 * 384 < 2^63
-        if (full) {
-          sk_flush();
-          sk_cnt = 0;
+        const bool full = sk_cnt + most > 384;  // 2^54 * 384 < 2^63
+        if (full || s_rescale != 0) {
+          const SkTile st{ys, yblk, T, tsh, d, b, ska, skf, mypart, s_scale, s_base, s_new, s_nan, &s_rescale, sk_first};
+          if (sk_rescale(st, full)) {
+            sk_first = false;
+            sk_cnt = 0;
+          }
         }
         sk_cnt += most;
-        if (rescale) {
-          __syncthreads();  // scales read by the flush and the conversion
-          for (int c = warp; c < b; c += TC_NW) {
-            int ex = 0;
-            for (int r = lane; r < T; r += 32)
-              ex = max(ex, (__double2hiint(tc_ld(ys + TcTile::off(yblk, r, c))) >> 20) & 0x7FF);
-            ex = __reduce_max_sync(0xffffffffu, ex);
-            if (lane == 0) {
-              if (ex == 0x7FF) s_nan[c] = 1;
-              // (room to grow, but never up to the exponent field of Inf and NaN, which must stay past
-              // every scale)
-              const int old = s_scale[c], now = (ex > old && ex != 0x7FF) ? min(ex + 1, 0x7FE) : old;
-              s_shift[c] = min(now - old, 63);
-              s_scale[c] = now;
-            }
-          }
-          __syncthreads();
-          for (int t = tid; t < d * b; t += TC_NT) {
-            const int k = s_shift[t / d];
-            if (k > 0) ska[t] = k >= 63 ? 0 : (ska[t] + (1LL << (k - 1))) >> k;
-          }
-          for (int t = tid; t < T * b; t += TC_NT) {
-            const int c = t >> tsh, r = t & (T - 1);
-            const double v = tc_ld(ys + TcTile::off(yblk, r, c));
-            const long long f = s_nan[c] ? 0 : fx_round54(v, s_scale[c]);
-            skf[2 * r * b + c] = f;
-            skf[(2 * r + 1) * b + c] = -f;
-          }
-          if (tid == 0) s_rescale = 0;
-        }
-        if (rescale || full) __syncthreads();
       }
       const uint32_t* meta = reinterpret_cast<const uint32_t*>(stage_R(s));
       for (int c0 = 0; c0 < b; c0 += CB) {
@@ -461,7 +525,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   // ---------------- partials + fixed-order two-level tree -------------------------
   if (P.L == 0) return;
   __syncthreads();
-  if constexpr (SK) sk_flush();
+  if constexpr (SK) sk_flush(ska, d, b, s_scale, s_nan, mypart, sk_first, mixed);
   if constexpr (G != 0)
   for (int o = tid; o < P.no; o += TC_NT) {
     const int i = o / b, c = o % b;
