@@ -87,10 +87,9 @@ static __device__ __noinline__ void tc_copy_bytes(unsigned char* dst, const uint
 }
 
 // Sketch sums into the CTA's partial (= for the first time, then +=), each thread its own entries;
-// the sums start again from zero.  (This and the next function are not inlined: they run every
-// few dozen tiles, and a pass with them in its loop takes 5 % longer.)
-static __device__ __noinline__ void sk_flush(long long* ska, int d, int b, const int* scale, const bool* nan,
-                                             double* part, bool first, bool mixed) {
+// the sums start again from zero
+static __device__ __forceinline__ void sk_flush(long long* ska, int d, int b, const int* scale, const bool* nan,
+                                                double* part, bool first, bool mixed) {
   for (int t = threadIdx.x; t < d * b; t += TC_NT) {
     const int c = t / d;
     if (mixed) {
@@ -105,29 +104,28 @@ static __device__ __noinline__ void sk_flush(long long* ska, int d, int b, const
     ska[t] = 0;
   }
 }
-struct SkTile {
-  const unsigned char* ys;
-  int yblk, T, tsh, d, b;
-  long long *ska, *skf;
-  double* part;
-  int* scale;     // per column: exponent field of the scale,
-  short* base;    // of the scale at the last flush,
-  short* now;     // of the next scale
-  bool* nan;      // the column has a value that is not finite
-  int* rescale;   // set when a warp found a value past its scale or 16 far below it
-  bool first;
+struct SkScales {   // per column:
+  int scale[64];    // exponent field of the scale,
+  short base[64];   // of the scale at the last flush,
+  short now[64];    // of the next scale
+  bool nan[64];     // the column has a value that is not finite
+  int rescale;      // set when a warp found a value past its scale, or 16 far below it
 };
-// Scales for this tile and its values on them; true when the sums went into the partial.  Whole
-// block, all threads past the conversion of the tile; ends with a barrier.
-static __device__ __noinline__ bool sk_rescale(const SkTile& S, bool full) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = S.b, d = S.d;
-  const bool rescale = *S.rescale != 0;
+// Scales for this tile (y' at ys, bytes from the start of the dynamic shared memory, as ska and
+// skf) and its values on them; true when the sums (cnt: entries a row can hold) went into the
+// partial.  Whole block, all threads past the conversion of the tile; ends with a barrier.  Not
+// inlined: it runs every few dozen tiles, and a pass with it in its loop takes 5 % longer.
+static __device__ __noinline__ bool sk_rescale(SkScales& S, int ys, int yblk, int tsh, int d, int b, int ska_off,
+                                               int skf_off, double* part, bool first, bool full, int cnt) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  long long *ska = reinterpret_cast<long long*>(smem_raw + ska_off), *skf = reinterpret_cast<long long*>(smem_raw + skf_off);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = 1 << tsh;
   bool change = false, flush = full;
-  if (rescale) {
+  if (S.rescale != 0) {
     for (int c = warp; c < b; c += TC_NW) {
       int ex = 0;
-      for (int r = lane; r < S.T; r += 32)
-        ex = max(ex, (__double2hiint(tc_ld(S.ys + TcTile::off(S.yblk, r, c))) >> 20) & 0x7FF);
+      for (int r = lane; r < T; r += 32)
+        ex = max(ex, (__double2hiint(tc_ld(smem_raw + ys + TcTile::off(yblk, r, c))) >> 20) & 0x7FF);
       ex = __reduce_max_sync(0xffffffffu, ex);
       if (lane == 0) {
         // (room to grow, but never up to the exponent field of Inf and NaN, which must stay past
@@ -144,30 +142,30 @@ static __device__ __noinline__ bool sk_rescale(const SkTile& S, bool full) {
       flush = flush || now < old || (old > 0 && now > S.base[c] + SK_RISE);
     }
     change = __any_sync(0xffffffffu, change);  // (the same in every warp)
-    flush = __any_sync(0xffffffffu, flush);
+    flush = __any_sync(0xffffffffu, flush) && cnt > 0;
   }
   if (flush) {  // sums on the scales they were formed with
-    sk_flush(S.ska, d, b, S.scale, S.nan, S.part, S.first, false);
-  } else if (change) {  // small rises: the sums move along
+    sk_flush(ska, d, b, S.scale, S.nan, part, first, false);
+  } else if (change && cnt > 0) {  // small rises: the sums move along
     for (int t = tid; t < d * b; t += TC_NT) {
       const int k = S.now[t / d] - S.scale[t / d];
-      if (k > 0 && S.ska[t] != 0) S.ska[t] = (S.ska[t] + (1LL << (k - 1))) >> k;
+      if (k > 0 && ska[t] != 0) ska[t] = (ska[t] + (1LL << (k - 1))) >> k;
     }
   }
   __syncthreads();  // scales read above
   if (tid < b) {
     if (change) S.scale[tid] = S.now[tid];
-    if (flush || S.base[tid] == 0) S.base[tid] = (short)S.scale[tid];
+    if (flush || cnt == 0 || S.base[tid] == 0) S.base[tid] = (short)S.scale[tid];
   }
-  if (tid == 0) *S.rescale = 0;
+  if (tid == 0) S.rescale = 0;
   if (change) {
     __syncthreads();
-    for (int t = tid; t < S.T * b; t += TC_NT) {
-      const int c = t >> S.tsh, r = t & (S.T - 1);
-      const double v = tc_ld(S.ys + TcTile::off(S.yblk, r, c));
+    for (int t = tid; t < T * b; t += TC_NT) {
+      const int c = t >> tsh, r = t & (T - 1);
+      const double v = tc_ld(smem_raw + ys + TcTile::off(yblk, r, c));
       const long long f = S.nan[c] ? 0 : fx_round54(v, S.scale[c]);
-      S.skf[2 * r * b + c] = f;
-      S.skf[(2 * r + 1) * b + c] = -f;
+      skf[2 * r * b + c] = f;
+      skf[(2 * r + 1) * b + c] = -f;
     }
   }
   __syncthreads();
@@ -195,9 +193,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   __shared__ int s_flag;
   __shared__ int s_last;
   __shared__ int s_bad;
-  __shared__ int s_scale[64], s_rescale;  // sketch: per column
-  __shared__ short s_base[64], s_new[64];
-  __shared__ bool s_nan[64];
+  __shared__ SkScales s_sk;  // sketch
   const PassDev& P = D.P;
   const RowPass& rp = P.p;
   if (read_code(P.status) != 0) return;
@@ -304,10 +300,10 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   if constexpr (SK) {
     for (int t = tid; t < d * b; t += TC_NT) ska[t] = 0;  // (all-zero bits also as float32 pairs)
     if (tid < 64) {
-      s_scale[tid] = s_base[tid] = 0;
-      s_nan[tid] = false;
+      s_sk.scale[tid] = s_sk.base[tid] = 0;
+      s_sk.nan[tid] = false;
     }
-    if (tid == 0) s_rescale = 0;
+    if (tid == 0) s_sk.rescale = 0;
   }
   if (HC && P.c_digits) tc_build_c(rp.C, ldc, a, b, cf, ec, &s_bad);
   if (inv) tc_build_c(rp.Inv, b, b, b, cf, ec, &s_bad);
@@ -446,7 +442,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
             reinterpret_cast<float*>(skf)[(2 * r + 1) * b + c] = -f;
           }
         } else {
-          const int sc = in ? s_scale[c] : 0, ex = (__double2hiint(v) >> 20) & 0x7FF;
+          const int sc = in ? s_sk.scale[c] : 0, ex = (__double2hiint(v) >> 20) & 0x7FF;
           past = past || ex > sc;
           const unsigned near = __ballot_sync(0xffffffffu, ex + SK_FAR > sc);
           if (near < 0x10000u || (near & 0xFFFFu) == 0u) {
@@ -460,7 +456,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
           }
         }
       }
-      if ((__any_sync(0xffffffffu, past) || low) && lane == 0) s_rescale = 1;
+      if ((__any_sync(0xffffffffu, past) || low) && lane == 0) s_sk.rescale = 1;
       __syncthreads();
       if (XS) next_x(tile + gridDim.x);
       if (!mixed) {
@@ -468,9 +464,10 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
         const uint32_t m0 = *reinterpret_cast<const uint32_t*>(stage_R(s));
         const int most = m0 == 0xFFFFFFFFu ? 0 : (int)(m0 >> 23);
         const bool full = sk_cnt + most > 384;  // 2^54 * 384 < 2^63
-        if (full || s_rescale != 0) {
-          const SkTile st{ys, yblk, T, tsh, d, b, ska, skf, mypart, s_scale, s_base, s_new, s_nan, &s_rescale, sk_first};
-          if (sk_rescale(st, full)) {
+        if (full || s_sk.rescale != 0) {
+          const int base = (int)(smem - smem_raw);
+          if (sk_rescale(s_sk, (int)(ys - smem_raw), yblk, tsh, d, b, base + P.off_sk, base + P.off_skf, mypart, sk_first,
+                         full, sk_cnt)) {
             sk_first = false;
             sk_cnt = 0;
           }
@@ -525,7 +522,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
   // ---------------- partials + fixed-order two-level tree -------------------------
   if (P.L == 0) return;
   __syncthreads();
-  if constexpr (SK) sk_flush(ska, d, b, s_scale, s_nan, mypart, sk_first, mixed);
+  if constexpr (SK) sk_flush(ska, d, b, s_sk.scale, s_sk.nan, mypart, sk_first, mixed);
   if constexpr (G != 0)
   for (int o = tid; o < P.no; o += TC_NT) {
     const int i = o / b, c = o % b;
