@@ -99,6 +99,7 @@ extern "C" int rbo_gram_noalloc(int64_t n, int32_t a, const double* X, int64_t l
   r.ldy = ldy;
   r.b = b;
   r.acc_x = 1;
+  r.elementwise = 1;
   r.max_ctas = max_ctas;
   r.epi.op = EPI_STORE;
   r.epi.out = C;

@@ -175,6 +175,7 @@ int rowpass_tc_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* laun
   }
   auto kernel_of = [&](int tri) {
     if (y_only) return tc_kernel_g3();
+    if (rp.elementwise && ax > 0 && !hc && !rp.Tri) return tc_kernel_g4();
     return q == 0 ? tc_kernel_g0(hc, tri, d > 0) : (ax == 0 && b <= 8 ? tc_kernel_g2(hc, tri) : tc_kernel_g1(hc, tri));
   };
   TcKernel kern = kernel_of(want_inv ? 2 : (rp.Tri ? 1 : 0));

@@ -174,7 +174,8 @@ static __device__ __noinline__ bool sk_rescale(SkScales& S, int ys, int yblk, in
 
 // HC: projection (C digits); TRI: triangular factor, 0 none, 1 substitution, 2 product with its
 // inverse (digits); G: Gram, 0 none, 1 general, 2 of at most
-// 8 columns of Y' alone, 3 of more columns of Y' alone after an update; SK: sparse sketch (no triangle, no Gram).  Each kind of pass is its
+// 8 columns of Y' alone, 3 of more columns of Y' alone after an update, 4 general with a bound for
+// every entry; SK: sparse sketch (no triangle, no Gram).  Each kind of pass is its
 // own kernel: fewer live registers and less code than one kernel with all phases.
 template <bool HC, int TRI, int G, bool SK>
 __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_kernel(const __grid_constant__ TcDev D) {
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
           const int chunk = item / q, task = item - chunk * q;
           int nt = 0;
           while (nt + 1 < P.nblk && task >= P.blk_start[nt + 1]) ++nt;
-          tc_gram_item<NT>(xt, yt, ax, P.zr, b, task - P.blk_start[nt], nt * NT, (chunk * P.kc) >> 4, P.kc >> 4,
+          tc_gram_item<NT, G == 4>(xt, yt, ax, P.zr, b, task - P.blk_start[nt], nt * NT, (chunk * P.kc) >> 4, P.kc >> 4,
                            accs + item * 128 * NT);
         }
       }
@@ -548,6 +549,7 @@ typedef void (*TcKernel)(TcDev);
 TcKernel tc_kernel_g0(bool hc, int tri, bool sk);  // no Gram   (rowpass_tc_g0.cu)
 TcKernel tc_kernel_g1(bool hc, int tri);            // general   (rowpass_tc_g1.cu)
 TcKernel tc_kernel_g3();                            // wide Y'^T Y' after an update (rowpass_tc_g1.cu)
+TcKernel tc_kernel_g4();                            // general with a bound for every entry (rowpass_tc_g1.cu)
 TcKernel tc_kernel_g2(bool hc, int tri);            // Y'^T Y', at most 8 columns (rowpass_tc_g2.cu)
 
 }  // namespace rbo

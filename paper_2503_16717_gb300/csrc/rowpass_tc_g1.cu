@@ -8,4 +8,5 @@ TcKernel tc_kernel_g1(bool hc, int tri) {
   return rowpass_tc_kernel<false, 0, 1, false>;
 }
 TcKernel tc_kernel_g3() { return rowpass_tc_kernel<true, 0, 3, false>; }
+TcKernel tc_kernel_g4() { return rowpass_tc_kernel<false, 0, 4, false>; }
 }  // namespace rbo

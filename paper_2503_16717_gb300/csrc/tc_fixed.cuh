@@ -18,11 +18,13 @@
 //     level stay below 2^24, so every sum is exact in any order;
 //   - the levels 0..6 (28 digit pairs) are joined in 64-bit integers and enter the
 //     float64 result with one conversion and one FMA.  The pairs left out (I + J >= 7)
-//     weigh at most 6 * 2^54 / 2^110 < 2^-53.4 of the largest product of the group per
-//     term, 2^-56 root mean square over the digits' signs; joining rounds at 2^-55 of it
-//     once per chunk.
+//     weigh at most 6 * 2^54 / 2^108 < 2^-51.4 of the largest product of the group per
+//     term (whose factors are at least 2^54 each), about 2^-55 root mean square over the
+//     digits' signs; joining rounds at 2^-55 of it once per chunk.
 // A group with a non-finite value, or with its largest value outside 2^+-463, is
-// computed by float64 FMAs instead.
+// computed by float64 FMAs instead.  So is, where the Gram itself is asked for, an entry's chunk
+// in which the large values of the two columns do not meet (tc_tile.cuh): there the error, which
+// goes by the largest values, could exceed that of float64 sums, which goes by the products.
 //
 // Why the digits go from registers into mma.sync: every thread forms the digits of the
 // fragment elements it owns, so no operand passes through shared or tensor memory
@@ -38,7 +40,8 @@
 namespace rbo {
 
 constexpr int FX_EMIN = 560;    // smallest and largest exponent field of a group in
-constexpr int FX_EMAX = 1486;   // fixed point (2^-463 .. 2^463); zero groups use FX_EMIN
+constexpr int FX_EMAX = 1486;   // fixed point (2^-463 .. 2^463)
+constexpr int FX_EZERO = 559;   // scale of a group of zeros
 constexpr uint32_t FX_MAGIC = 0x4B400000u;  // 1.5 * 2^23: float bits minus this = integer
 
 // twice the largest |x| high word and the OR of low words of the scanned values
@@ -60,7 +63,7 @@ struct FxMax {
   // group with nonzero bits counts as below FX_EMIN)
   __device__ __forceinline__ int scale() const {
     const int e = (int)(m >> 21);
-    if ((m | nz) == 0u) return FX_EMIN;
+    if ((m | nz) == 0u) return FX_EZERO;
     return (e >= FX_EMIN && e <= FX_EMAX) ? e : 0;
   }
 };
@@ -182,10 +185,11 @@ __device__ __forceinline__ void fx_mma_first(float (&d)[4], uint32_t a0, uint32_
 // g / g + 8), B = digits bd[J][K half]
 // FIRST: the first step of a sum, which starts from `init` instead of the accumulators.
 // NT column tiles of B share the digits of A, which are two thirds of a step's instructions.
+// sizes: unless null, the same sums of the sizes of the top digits alone.
 template <int I, bool FIRST, int NT>
 __device__ __forceinline__ void fx_level(float (&acc)[NT][7][4], const FxPair& p00, const FxPair& p10,
                                          const FxPair& p01, const FxPair& p11, const uint32_t (&bd)[NT][7][2],
-                                         const FxMask& k, const float (&init)[4]) {
+                                         const FxMask& k, const float (&init)[4], float (*sizes)[4]) {
   const uint32_t a0 = fx_digit<I>(p00, k), a1 = fx_digit<I>(p10, k), a2 = fx_digit<I>(p01, k),
                  a3 = fx_digit<I>(p11, k);
 #pragma unroll
@@ -195,22 +199,31 @@ __device__ __forceinline__ void fx_level(float (&acc)[NT][7][4], const FxPair& p
       if (FIRST && I == 0) fx_mma_first(acc[h][J], a0, a1, a2, a3, bd[h][J][0], bd[h][J][1], init);
       else fx_mma(acc[h][I + J], a0, a1, a2, a3, bd[h][J][0], bd[h][J][1]);
     }
+  if (I == 0 && sizes != nullptr) {
+    const float zero[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int h = 0; h < NT; ++h) {
+      const uint32_t b0 = bd[h][0][0] & ~k.sign, b1 = bd[h][0][1] & ~k.sign;
+      if (FIRST) fx_mma_first(sizes[h], a0 & ~k.sign, a1 & ~k.sign, a2 & ~k.sign, a3 & ~k.sign, b0, b1, zero);
+      else fx_mma(sizes[h], a0 & ~k.sign, a1 & ~k.sign, a2 & ~k.sign, a3 & ~k.sign, b0, b1);
+    }
+  }
 }
 template <bool FIRST, int NT>
 __device__ __forceinline__ void fx_step(float (&acc)[NT][7][4], FxPair& p00, FxPair& p10, FxPair& p01,
                                         FxPair& p11, const uint32_t (&bd)[NT][7][2], const FxMask& k,
-                                        const float (&init)[4]) {
-  fx_level<0, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<1, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<2, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<3, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
+                                        const float (&init)[4], float (*sizes)[4] = nullptr) {
+  fx_level<0, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init, sizes);
+  fx_level<1, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init, nullptr);
+  fx_level<2, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init, nullptr);
+  fx_level<3, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init, nullptr);
   fx_mask_low(p00, k);
   fx_mask_low(p10, k);
   fx_mask_low(p01, k);
   fx_mask_low(p11, k);
-  fx_level<4, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<5, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
-  fx_level<6, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init);
+  fx_level<4, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init, nullptr);
+  fx_level<5, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init, nullptr);
+  fx_level<6, FIRST, NT>(acc, p00, p10, p01, p11, bd, k, init, nullptr);
 }
 // digits of a B fragment (K pairs q0: 2t, 2t+1 and q1: 2t+8, 2t+9 of column g)
 __device__ __forceinline__ void fx_bdigits(FxPair& q0, FxPair& q1, uint32_t (&bd)[7][2], const FxMask& k) {

@@ -47,6 +47,64 @@ __device__ __forceinline__ void tc_gram_flush(float (&acc)[7][4], bool small, in
   }
 }
 
+// Chunks whose error the digits do not bound well enough.  With the unit of a product of two top
+// digits, a chunk of k rows is off by at most k 2^-38.6 (the pairs left out, the truncated bits),
+// whatever its terms; the sum of |d_x d_y| over the top digits is the sum of the terms' sizes to
+// within the smallest of them (whole warp).  At 16 k and more (the largest value of a column has a top digit of
+// 64 .. 128: a quarter of that, met in both columns, in every row, or fewer and larger) the chunk is
+// off by at most 2^-41 of the sum of the terms' sizes, less than 4096 roundings of a float64 sum;
+// chunks of Gaussian columns lie ten times above.  Below, the chunk is summed by FMAs.  It costs 5 %
+// (Gram of 60 x 5 columns at 4 million rows 757 -> 790 us, with an outlier in every chunk 1500), so it
+// is for Grams that are results themselves: in the orthogonalization, whose errors are measured
+// against the norms of the columns, the plain ones serve.
+__device__ __forceinline__ bool tc_gram_small(const float (&sizes)[4], int nks, int E0, int E1, int Eb) {
+  const int t = threadIdx.x & 3;
+  const int Ea = __shfl_sync(0xffffffffu, Eb, 8 * t), Ec = __shfl_sync(0xffffffffu, Eb, 8 * t + 4);
+  const float lim = (float)(256 * nks);
+  const bool z0 = E0 != FX_EZERO, z1 = E1 != FX_EZERO, ya = Ea != FX_EZERO, yc = Ec != FX_EZERO;
+  return (sizes[0] < lim && z0 && ya) || (sizes[1] < lim && z0 && yc) || (sizes[2] < lim && z1 && ya) ||
+         (sizes[3] < lim && z1 && yc);
+}
+
+// The same item by float64 FMAs, for the guarded Gram, where it may run often: the outputs dealt to
+// the lanes, up to four each (an outlier in every chunk of 59 x 5 columns: 355 us at 400001 rows;
+// two rows and two columns of 16 x 8 a lane, 440).  Not inlined: the digit products keep their
+// registers.  Whole warp.
+static __device__ __noinline__ void tc_gram_fma(const TcTile xt, const TcTile yt, int ax, int zr, int b, int mt, int nt,
+                                                int ntiles, int b0, int nks, double* acc_out) {
+  const int lane = threadIdx.x & 31, zw = min(16, zr - 16 * mt);
+  __syncwarp();
+  for (int h = 0; h < ntiles; ++h) {
+    const int c0 = 8 * (nt + h), cnt = zw * min(8, b - c0);
+    const unsigned char *px[4], *py[4];
+    int zc[4], yc[4], xb[4];
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int o = min(lane + 32 * u, max(cnt, 1) - 1), z = 16 * mt + o % zw;
+      yc[u] = min(c0 + o / zw, b - 1);
+      zc[u] = z < ax ? z : z - ax;
+      xb[u] = z < ax ? xt.blk : yt.blk;
+      px[u] = (z < ax ? xt.base : yt.base) + b0 * xb[u];
+      py[u] = yt.base + b0 * yt.blk;
+    }
+    for (int r = 0; r < 16 * nks; ++r)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (32 * u < cnt)
+          s[u] = fma(tc_ld(px[u] + TcTile::off(xb[u], r, zc[u])), tc_ld(py[u] + TcTile::off(yt.blk, r, yc[u])), s[u]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int o = lane + 32 * u;
+      if (o < cnt) {
+        const int zi = o % zw, c = o / zw;
+        acc_out[h * 128 + (2 * (zi >> 3) + (c & 1)) * 32 + 4 * (zi & 7) + (c >> 1)] += s[u];
+      }
+    }
+  }
+  __syncwarp();
+}
+
 // acc_out (NT times 4 x 32 doubles, this warp's own) += Z(:, 16 mt ..)^T Y(:, 8 nt ..) over the
 // nks blocks of 16 rows from block b0, for the NT column tiles from nt; Z = [X (ax columns, tile
 // xt), Y (tile yt)], zr columns (the last one stands in for columns past the end, whose sums are
@@ -55,7 +113,8 @@ __device__ __forceinline__ void tc_gram_flush(float (&acc)[7][4], bool small, in
 // g + 8 of Z and g of Y: the order of the rows inside a step is the same for both
 // operands, which is all a contraction needs, and makes every load 16 bytes.
 // acc_out[o * 32 + lane] belongs to Z column 16 mt + g + 8 (o / 2), Y column 8 nt + 2t + o % 2.
-template <int NT>
+// GUARD: chunks whose large values do not meet are summed by FMAs (tc_gram_small).
+template <int NT, bool GUARD>
 static __device__ __forceinline__ void tc_gram_item(const TcTile xt, const TcTile yt, int ax, int zr, int b,
                                                     int mt, int nt, int b0, int nks, double* acc_out) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -103,6 +162,10 @@ static __device__ __forceinline__ void tc_gram_item(const TcTile xt, const TcTil
     out = out || Eb[h] == 0;
   }
   if (__any_sync(0xffffffffu, out)) {
+    if constexpr (GUARD) {
+      tc_gram_fma(xt, yt, ax, zr, b, mt, nt, NT, b0, nks, acc_out);
+      return;
+    }
 #pragma unroll 1
     for (int h = 0; h < NT; ++h) {
       const int ya = min(8 * (nt + h) + 2 * t, b - 1), yb = min(8 * (nt + h) + 2 * t + 1, b - 1);
@@ -131,7 +194,7 @@ static __device__ __forceinline__ void tc_gram_item(const TcTile xt, const TcTil
   for (int h = 0; h < NT; ++h) kb[h] = fx_scale(Eb[h]);
   const FxMask km = fx_masks();
   const bool small = nks <= 2;
-  float acc[NT][7][4], init[4];
+  float acc[NT][7][4], sizes[NT][4], init[4];
   fx_init(init, small);
   auto step = [&](int ks, auto first) {
     const unsigned char *pa = z0 + ks * blk0, *pc = z1 + ks * blk1;
@@ -147,11 +210,23 @@ static __device__ __forceinline__ void tc_gram_item(const TcTile xt, const TcTil
     }
     FxPair p00 = fx_pair(u0.x, u0.y, k0, km), p01 = fx_pair(u1.x, u1.y, k0, km);
     FxPair p10 = fx_pair(w0.x, w0.y, k1, km), p11 = fx_pair(w1.x, w1.y, k1, km);
-    fx_step<decltype(first)::value, NT>(acc, p00, p10, p01, p11, bd, km, init);
+    fx_step<decltype(first)::value, NT>(acc, p00, p10, p01, p11, bd, km, init, GUARD ? sizes : nullptr);
   };
   step(0, FxTrue());
 #pragma unroll 1
   for (int ks = 1; ks < nks; ++ks) step(ks, FxFalse());
+  if constexpr (GUARD) {
+    bool few = false;
+#pragma unroll
+    for (int h = 0; h < NT; ++h) {
+      const bool f = tc_gram_small(sizes[h], nks, E0, E1, Eb[h]);  // (whole warp: shuffles)
+      few = few || f;
+    }
+    if (__any_sync(0xffffffffu, few)) {
+      tc_gram_fma(xt, yt, ax, zr, b, mt, nt, NT, b0, nks, acc_out);
+      return;
+    }
+  }
 #pragma unroll
   for (int h = 0; h < NT; ++h) tc_gram_flush(acc[h], small, E0, E1, Eb[h], zr - i0 > 8, acc_out + h * 128);
 }
