@@ -9,7 +9,10 @@ two-stage scheme (s_hat = 20).  `value` is the mean time to solution per solve.
 The working set (CSR 88 MB + basis 490 MB + vectors) exceeds the 129 MB L2, so no
 L2 flush is needed between steps.
 
-Also reported (the block orthogonalization alone, V = 2^24 x 61 glued blocks,
+The printed line holds the headline; everything below is written to --sections
+(default bench_sections.json beside this file).
+
+Also measured (the block orthogonalization alone, V = 2^24 x 61 glued blocks,
 two-stage s_hat = 30 and one-stage, FP64 and mixed precision): orthogonalized
 columns/s, algorithmic HBM GB/s and ||I - Q^T Q||_2, under "orth".
 
@@ -25,6 +28,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -302,9 +306,48 @@ def run_ours(args):
             "s_sweep": sweep_res,
             "cpu_baseline": cpu,
         }
-        print(json.dumps(line), flush=True)
+        emit(line, args.sections)
     if dist:
         dist.destroy_process_group()
+
+
+# what the printed line holds; everything else goes to the sections file
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "solves", "roofline", "e2e", "gpu_launches", "clocks",
+            "cpu_baseline")
+
+
+def _plain(v):
+    """`v` with values that JSON has no form for (NaN, infinities) as null."""
+    if isinstance(v, dict):
+        return {k: _plain(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_plain(x) for x in v]
+    if isinstance(v, float) and not math.isfinite(v):
+        return None
+    return v
+
+
+def headline(line):
+    """The printed line: the headline keys, of the roofline its plain values."""
+    out = {k: line[k] for k in HEADLINE if k in line}
+    if isinstance(out.get("roofline"), dict):
+        out["roofline"] = {k: v for k, v in out["roofline"].items() if not isinstance(v, (dict, list))}
+    return _plain(out)
+
+
+def emit(line, path):
+    """Writes all sections to `path` and prints the headline as one line, which stays short
+    enough for readers that keep the end of a run's output only."""
+    out = headline(line)
+    if path:
+        try:
+            with open(path, "w") as f:
+                json.dump(_plain(line), f, indent=1, allow_nan=False)
+            out["sections"] = os.path.basename(path)
+        except OSError as e:
+            print(f"sections not written: {e}", file=sys.stderr)
+    print(json.dumps(out, allow_nan=False), flush=True)
 
 
 def measured_traffic(passes, n, launches):
@@ -1032,6 +1075,9 @@ def main():
                          "gradient (512^2), print them as one JSON object and exit")
     ap.add_argument("--gnn-grid", type=int, default=2048,
                     help="grid points per side of the --gnn-only inference instance")
+    ap.add_argument("--sections", default=os.path.join(ROOT, "bench_sections.json"),
+                    help="file for everything beside the headline (orthogonalization, precision modes, "
+                         "kernels, learned preconditioner, stress solves); empty for none")
     args = ap.parse_args()
     if args.gnn_only:
         import torch
