@@ -147,11 +147,10 @@ struct RowPass {
   double* Y = nullptr; int64_t ldy = 0; int b = 0;
   const double* C = nullptr;     // a x b (ld ldc): projection coefficients, null = none
   int ldc = 0;                   // 0 means a
-  const double* Tri = nullptr;   // b x b (ld ldtri) upper triangular, null = none
+  const double* Tri = nullptr;   // b x b (ld ldtri) upper triangular, null = none: y' = (y - x C) Tri^-1
   int ldtri = 0;                 // 0 means b
   const double* Inv = nullptr;   // inverse of Tri (b x b), set where Tri is the factor of a
                                  // nearly orthonormal Gram: y Tri^-1 may be formed as y Inv
-  int tri_first = 0;             // 1: y' = y Tri^-1 - x C;  0: y' = (y - x C) Tri^-1
   int write_y = 0;
   int acc_x = 0;                 // accumulate X^T Y'
   int acc_y = 0;                 // accumulate Y'^T Y'

@@ -290,15 +290,11 @@ __global__ void __launch_bounds__(NT, (ARITH == 0 ? 3 : 2)) rowpass_kernel(const
         ys[c * TP + r] = v0 + v1;
       }
     };
-    if (rp.Tri && rp.tri_first) {
-      tri_solve();
-      __syncthreads();
-    }
     if (rp.C) {
       project();
       __syncthreads();
     }
-    if (rp.Tri && !rp.tri_first) {
+    if (rp.Tri) {
       tri_solve();
       __syncthreads();
     }
@@ -512,8 +508,8 @@ int rowpass_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* launche
   if (rp.a > 0 && rp.X == nullptr) return RBO_ERR_ARG;
   if (rp.a == 0) { rp.C = nullptr; rp.acc_x = 0; }
   // Gram passes of the tensor-core mode go to the digit-product kernel when their shape
-  // allows it and (unless the caller asked for it outright, ozaki == 2) when it beats
-  // the float64 pass (ozaki.cu); every other pass runs here in float64
+  // allows it and (unless the caller asked for it outright, ozaki == 2) when it is wide
+  // enough (ozaki.cu); every other pass runs as in float64
   if (rp.ozaki && ozaki_gram_supported(rp) && (rp.ozaki == 2 || ozaki_gram_pays(rp)))
     return ozaki_gram_launch(rp, ar, st, launches, sm_count());
   if (rp.sk_d > DMAX || rp.sk_zeta > ZMAX) return RBO_ERR_ARG;
@@ -629,9 +625,6 @@ int rowpass_launch(const RowPass& rpin, Arena* ar, cudaStream_t st, int* launche
   P.off_dinv = (int)off_dinv;
   P.off_sk = 0;
   P.off_gth = (int)off_gth;
-  P.rec_off = 0;
-  P.off_ys = 0;
-  P.ystage_bytes = 0;
   P.off_red = (int)off_red;
   P.partials = nullptr;
   P.gpart = nullptr;

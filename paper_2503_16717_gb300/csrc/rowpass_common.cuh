@@ -37,11 +37,9 @@ struct PassDev {
   // shared memory layout (byte offsets from the dynamic base)
   int off_stage, stage_bytes, off_c, off_tri, off_dinv, off_sk, off_red;
   int off_gth;            // Gaussian sketch entries of the tile (sk_gd x TP)
-  int rec_off;            // sketch schedule record of the tile, offset inside a stage
   int kc, off_acc, off_ec;   // tensor-core pass: Gram chunk rows, item sums, C column scales
   int xblk, yblk;            // bytes of a 16-row block of X and of Y
   int off_skf, c_digits;  // sketch tile values; whether C is held as digits
-  int off_ys, ystage_bytes;  // sketch kernel: ring of Y stages (Y columns + record)
 };
 
 // ------------------------------------------------------------------------------------
@@ -415,7 +413,7 @@ static inline size_t epilogue_doubles(const RowPass& rp) {
 }
 
 // ------------------------------------------------------------------------------------
-// sketch entry sums of one tile (both row-pass kernels)
+// sketch entry sums of one tile
 // ------------------------------------------------------------------------------------
 // Sketch sums of a tile: meta is its schedule record (mcap slot words, then the entry
 // bytes).  The thread that owns a slot adds the rows of its entries to the sketch row's

@@ -393,7 +393,6 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
       else __syncthreads();
       synced = !own;
     };
-    if (HT && rp.tri_first) tri_solve();
     if constexpr (HC) {
       for (int k = rw >> 4; k < re >> 4; ++k)
         tc_update_rows<NT>(xs + k * xblk, ys + k * yblk, a, b, cf, ec, bad_c, rp.C, ldc);
@@ -406,7 +405,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
         __syncwarp();
       }
     }
-    if (HT && !rp.tri_first) tri_solve();
+    if (HT) tri_solve();
     if (rp.write_y) {
       if (P.use_bulk) {  // two rows per lane
         const int h = (re - rw) >> 1, hsh = 31 - __clz(max(h, 1));

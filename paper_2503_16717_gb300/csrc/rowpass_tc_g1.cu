@@ -3,7 +3,7 @@
 
 namespace rbo {
 TcKernel tc_kernel_g1(bool hc, int tri) {
-  if (hc) return tri ? rowpass_tc_kernel<true, 1, 1, false> : rowpass_tc_kernel<true, 0, 1, false>;
+  if (hc) return tri ? rowpass_tc_kernel<true, 1, 1, false> : nullptr;
   if (tri) return tri == 2 ? rowpass_tc_kernel<false, 2, 1, false> : rowpass_tc_kernel<false, 1, 1, false>;
   return rowpass_tc_kernel<false, 0, 1, false>;
 }
