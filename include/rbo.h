@@ -62,11 +62,18 @@ extern "C" {
                               for a projection) share a power-of-two scale and enter as
                               55-bit integers, off by at most a quarter of an ulp of the
                               largest of them; a group with a non-finite value or outside
-                              2^+-463 takes float64 FMAs.  The sketch sums 54-bit integers
-                              on the scale of the column's largest value so far.
+                              2^+-463 takes float64 FMAs, and so do passes of few columns.
+                              These errors go by the largest values of a group (backward
+                              stable by columns); where the Gram is the result (rbo_gram
+                              and its kin) chunks of rows whose large values do not meet
+                              are summed by FMAs as well, so that every entry is as good
+                              as a float64 sum.  The sketch sums 54-bit integers on a
+                              scale that follows the column's values over the rows.
                               Triangular solves are float64 substitutions, or for the last
                               factors of big panels (near the identity) the same products
-                              with the float64 inverse; the small factors are IEEE float64 */
+                              with the float64 inverse; the small factors are float64, with
+                              the square roots and reciprocals of those of at most 16
+                              columns to within about an ulp                            */
 #define RBO_PREC_MIXED  1  /* sketch apply and first-pass projection coefficients in
                               float32 with float32 accumulation; Gram matrices feeding
                               the final Cholesky, the small factors, every update of V
@@ -78,7 +85,8 @@ extern "C" {
                               float64 every ~64 terms); first-pass projections, TRSMs,
                               the sketch and the small factors in float64.  Only steps
                               that cannot reach the backward error ||V - QR|| are
-                              moved off the float64 pipe                              */
+                              moved off the float64 pipe.  Slower than RBO_PREC_FP64
+                              since that runs on the tensor cores                     */
 #define RBO_PREC_OZAKI  3  /* float64 data and results; the wide Gram matrices of the BCGS
                               and CholQR reductions (passes of 36 to 64 columns of [X Y'],
                               at most 8 of Y', no projection, no triangular solve) are

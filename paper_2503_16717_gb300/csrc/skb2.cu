@@ -13,7 +13,8 @@
 // exchange: the dot products of the column below row j with all later columns, and row j,
 // determine the reflector and its application.  Q comes from the compact WY form
 // I - V T V^T (Schreiber and Van Loan 1989).  Measured 13 us (d = 244, k = 5, the Householder
-// factor) to 19 us (with a sketched basis); a chain of cluster barriers and float64 latencies.
+// factor) to 19 us (with a sketched basis) between launches of one call, 25 and 39 us a launch
+// serialised with cold caches; a chain of cluster barriers and float64 latencies.
 #include <cooperative_groups.h>
 
 #include <algorithm>

@@ -47,16 +47,15 @@ __device__ __forceinline__ void tc_gram_flush(float (&acc)[7][4], bool small, in
   }
 }
 
-// Chunks whose error the digits do not bound well enough.  With the unit of a product of two top
-// digits, a chunk of k rows is off by at most k 2^-38.6 (the pairs left out, the truncated bits),
-// whatever its terms; the sum of |d_x d_y| over the top digits is the sum of the terms' sizes to
-// within the smallest of them (whole warp).  At 16 k and more (the largest value of a column has a top digit of
-// 64 .. 128: a quarter of that, met in both columns, in every row, or fewer and larger) the chunk is
-// off by at most 2^-41 of the sum of the terms' sizes, less than 4096 roundings of a float64 sum;
-// chunks of Gaussian columns lie ten times above.  Below, the chunk is summed by FMAs.  It costs 5 %
-// (Gram of 60 x 5 columns at 4 million rows 757 -> 790 us, with an outlier in every chunk 1500), so it
-// is for Grams that are results themselves: in the orthogonalization, whose errors are measured
-// against the norms of the columns, the plain ones serve.
+// Whether an item has an entry whose digits are not good enough.  In units of a product of two
+// top digits, a chunk of k rows is off by at most 2^-38.6 k (the pairs left out, the truncated
+// bits), whatever its terms; the sum S of |d_x d_y| over the top digits is the sum of the terms'
+// sizes to within the lower digits.  Where S >= 16 k the chunk is off by at most 2^-41 of that sum,
+// less than 4096 roundings of a float64 sum.  (The largest value of a column has a top digit of 64
+// to 128; chunks of Gaussian columns lie ten times above the line.)  Below it the chunk is summed by
+// FMAs.  The sums S cost 5 % (60 x 5 columns at 4 million rows 757 -> 790 us), so they are for Grams
+// that are results themselves: in the orthogonalization, whose errors are measured against the
+// norms of the columns, the plain items serve.  Whole warp.
 __device__ __forceinline__ bool tc_gram_small(const float (&sizes)[4], int nks, int E0, int E1, int Eb) {
   const int t = threadIdx.x & 3;
   const int Ea = __shfl_sync(0xffffffffu, Eb, 8 * t), Ec = __shfl_sync(0xffffffffu, Eb, 8 * t + 4);
