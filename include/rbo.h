@@ -67,8 +67,10 @@ extern "C" {
                               stable by columns); where the Gram is the result (rbo_gram
                               and its kin) chunks of rows whose large values do not meet
                               are summed by FMAs as well, so that every entry is as good
-                              as a float64 sum.  The sketch sums 54-bit integers on a
-                              scale that follows the column's values over the rows.
+                              as a float64 sum.  The sketch sums 54-bit integers on the
+                              scale of the column's largest value so far, in
+                              rbo_sketch_apply on one that follows its values over
+                              the rows.
                               Triangular solves are float64 substitutions, or for the last
                               factors of big panels (near the identity) the same products
                               with the float64 inverse; the small factors are float64, with

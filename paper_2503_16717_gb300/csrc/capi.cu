@@ -272,6 +272,7 @@ int rbo_sketch_apply(rbo_sketch sk, int64_t n, int32_t k, const double* W, int64
   r.n = n; r.Y = const_cast<double*>(W); r.ldy = ldw; r.b = k;
   set_sketch(r, c);
   r.mixed = precision == RBO_PREC_MIXED ? 1 : 0;
+  r.elementwise = 1;
   const bool cg = sk->type == RBO_SKETCH_COUNT_GAUSS;
   r.epi.op = cg ? EPI_GROUPS : EPI_SKETCH_OUT; r.epi.out_sk = dout;
   int launches = 0;

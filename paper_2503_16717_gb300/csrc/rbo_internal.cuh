@@ -162,7 +162,8 @@ struct RowPass {
   int ozaki = 0;                 // Gram on the tensor cores (exact digit products, ozaki.cu):
                                  // 1 where the pass shape allows it and it is the faster
                                  // kernel, 2 wherever the shape allows it; float64 otherwise
-  int elementwise = 0;           // the Gram is a result: every entry as good as a float64 sum
+  int elementwise = 0;           // the Gram or the sketch is a result: every entry as good as a
+                                 // float64 sum
   int small_coeffs = 0;          // C is a re-orthogonalization (O(eps kappa)) coefficient block
   int max_ctas = 0;              // cap on the grid (0: none); bounds the reduction scratch
   int tag = 0;                   // role for the per-kernel timing (RBO_PROF_PASS_*)

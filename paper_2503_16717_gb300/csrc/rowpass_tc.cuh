@@ -16,13 +16,15 @@
 //   S  (sketch passes) the y' of the tile as 54-bit integers on one scale per column, and
 //      their signed sums per sketch row from the tile's schedule record: the thread that
 //      owns a slot of the record sums the slot's entries and adds them to the row's 64-bit
-//      integer accumulators.  A column's scale follows its tiles: up when a value is past it,
-//      down when a tile's values are all 2^SK_FAR below it.  The accumulators enter the CTA's
-//      float64 partial when a scale falls or rises by more than SK_RISE, and before a sketch row
-//      can have summed 384 entries (a few thousand rows, by the tiles' largest counts), so that
-//      most tiles cost no float64 operation per sketch row, and so that a value is off by at most
-//      2^(SK_FAR - 1 + SK_RISE - 54) of the largest of its own tile, 2^-53 where the tiles of a
-//      column are alike;
+//      integer accumulators.  A column's scale rises when a value is past it, and the accumulators
+//      with it.  They enter the CTA's float64 partial before a sketch row can have summed 384
+//      entries (a few thousand rows, by the tiles' largest counts), so that most tiles cost no
+//      float64 operation per sketch row.  Where the sketch itself is the result, the scale also
+//      falls when a tile's values are all 2^SK_FAR below it, and the accumulators enter the partial
+//      when it falls or rises by more than SK_RISE: a value is then off by at most
+//      2^(SK_FAR - 1 + SK_RISE - 54) of the largest of its own tile.  (In the orthogonalization,
+//      whose errors are measured against the norms of the columns, that would cost 26 % of the pass
+//      on a basis whose sizes vary over the grid: convection-diffusion 2048^2.)
 //   B  the Gram items, (16 Z columns) x (8 Y' columns) x (a chunk of kc rows), are dealt
 //      to the warps; an item always goes to the same warp, which keeps its float64 sums
 //      in its own shared-memory slots.
@@ -116,7 +118,8 @@ struct SkScales {   // per column:
 // partial.  Whole block, all threads past the conversion of the tile; ends with a barrier.  Not
 // inlined: it runs every few dozen tiles, and a pass with it in its loop takes 5 % longer.
 static __device__ __noinline__ bool sk_rescale(SkScales& S, int ys, int yblk, int tsh, int d, int b, int ska_off,
-                                               int skf_off, double* part, bool first, bool full, int cnt) {
+                                               int skf_off, double* part, bool first, bool full, int cnt,
+                                               bool follow) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   long long *ska = reinterpret_cast<long long*>(smem_raw + ska_off), *skf = reinterpret_cast<long long*>(smem_raw + skf_off);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = 1 << tsh;
@@ -132,24 +135,24 @@ static __device__ __noinline__ bool sk_rescale(SkScales& S, int ys, int yblk, in
         // every scale)
         const int old = S.scale[c];
         if (ex == 0x7FF) S.nan[c] = true;
-        S.now[c] = (short)(ex != 0x7FF && ex > 0 && (ex > old || ex + SK_FAR <= old) ? min(ex + 1, 0x7FE) : old);
+        S.now[c] = (short)(ex != 0x7FF && ex > 0 && (ex > old || (follow && ex + SK_FAR <= old)) ? min(ex + 1, 0x7FE) : old);
       }
     }
     __syncthreads();
     for (int c = lane; c < b; c += 32) {
       const int old = S.scale[c], now = S.now[c];
       change = change || now != old;
-      flush = flush || now < old || (old > 0 && now > S.base[c] + SK_RISE);
+      flush = flush || now < old || (follow && old > 0 && now > S.base[c] + SK_RISE);
     }
     change = __any_sync(0xffffffffu, change);  // (the same in every warp)
     flush = __any_sync(0xffffffffu, flush) && cnt > 0;
   }
   if (flush) {  // sums on the scales they were formed with
     sk_flush(ska, d, b, S.scale, S.nan, part, first, false);
-  } else if (change && cnt > 0) {  // small rises: the sums move along
+  } else if (change && cnt > 0) {  // rises without a flush: the sums move along
     for (int t = tid; t < d * b; t += TC_NT) {
       const int k = S.now[t / d] - S.scale[t / d];
-      if (k > 0 && ska[t] != 0) ska[t] = (ska[t] + (1LL << (k - 1))) >> k;
+      if (k > 0 && ska[t] != 0) ska[t] = k >= 62 ? 0 : (ska[t] + (1LL << (k - 1))) >> k;
     }
   }
   __syncthreads();  // scales read above
@@ -444,7 +447,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
         } else {
           const int sc = in ? s_sk.scale[c] : 0, ex = (__double2hiint(v) >> 20) & 0x7FF;
           past = past || ex > sc;
-          const unsigned near = __ballot_sync(0xffffffffu, ex + SK_FAR > sc);
+          const unsigned near = rp.elementwise ? __ballot_sync(0xffffffffu, ex + SK_FAR > sc) : 0xffffffffu;
           if (near < 0x10000u || (near & 0xFFFFu) == 0u) {
             const unsigned some = __ballot_sync(0xffffffffu, ex > 0);
             low = low || (near < 0x10000u && some >= 0x10000u) || ((near & 0xFFFFu) == 0u && (some & 0xFFFFu) != 0u);
@@ -467,7 +470,7 @@ __global__ void __launch_bounds__(TC_NT, tc_min_ctas(HC, TRI, G)) rowpass_tc_ker
         if (full || s_sk.rescale != 0) {
           const int base = (int)(smem - smem_raw);
           if (sk_rescale(s_sk, (int)(ys - smem_raw), yblk, tsh, d, b, base + P.off_sk, base + P.off_skf, mypart, sk_first,
-                         full, sk_cnt)) {
+                         full, sk_cnt, rp.elementwise != 0)) {
             sk_first = false;
             sk_cnt = 0;
           }
